@@ -1,211 +1,32 @@
-// sr_cal.cu -- the CAL finder and filter on the device (McVicar et al., arXiv
-// 1805.00106, Sec. 3.2 CAL finder, Sec. 3.3 CAL filter; the paper's V2 keeps
-// them on the host, Sec. 4.1-4.2).  Same windows, in the same order, as the host
-// stage sr_candidates.
+// sr_cal.cu -- the large-read path of the CAL finder and filter (McVicar et al.,
+// arXiv 1805.00106, Sec. 3.2 CAL finder, Sec. 3.3 CAL filter): the reads whose
+// distinct CALs do not fit the tables of sr_find.cu (over 6144 of them).  Every
+// pass runs on many blocks per read.  Same windows as the host stage
+// sr_candidates.
 //
-//   count / emit  one warp per read: the read's 2-bit codes packed in shared
-//                 memory (with its reverse complement), each lane takes seeds
-//                 o = lane*stride, (lane+32)*stride, ...; per reference the
-//                 hashed canonical seed picks a bucket, its key is found among
-//                 the bucket's (key, position)-sorted entries (or, with bucket
-//                 heads, in the bucket's 64-byte head), and every matching entry
-//                 gives a '+' and/or '-' CAL by its orientation bits.  The count
-//                 pass keeps each lookup for the emit pass.  CALs are packed keys
-//                 ref << 60 | strand << 59 | (cal + 1024).
-//   filter        per read: a sort of its CAL keys, then the merge of
-//                 consecutive CALs <= merge_dist apart into windows represented
-//                 by their most frequent CAL (smallest on ties), the max_cands
-//                 cut by hit count, and the clamped window [cal - pad, cal + m +
-//                 pad).  One warp per read up to 128 CALs, one block up to 8192
-//                 (shared memory); larger reads are emitted, sorted and merged by
-//                 many blocks each, in tiles of 4096 keys.
+//   count / emit  count: one warp per read, its seeds' lookups kept as records;
+//                 emit: the CALs of each read's records by many blocks (reads
+//                 whose lookups do not fit a record are looked up again by one
+//                 warp).  CALs are packed keys ref << 60 | strand << 59 |
+//                 (cal + 1024).
+//   filter        a bitonic sort of each read's keys in tiles of 4096, then the
+//                 merge of consecutive CALs <= merge_dist apart into windows
+//                 represented by their most frequent CAL (smallest on ties), the
+//                 max_cands cut by hit count, and the clamped window [cal - pad,
+//                 cal + m + pad).
 //   compact       per-read windows to contiguous arrays.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
 
+#include "sr_cal.cuh"
 #include "sr_internal.h"
-#include "sr_seed.h"
 
 namespace sr {
 namespace {
 
-constexpr uint32_t FULL = 0xffffffffu;
 constexpr int kCalWarps = 4;
-constexpr uint64_t kCalBias = 1024;
-constexpr uint64_t kCalMask = (1ull << 59) - 1;
-constexpr uint64_t kNoKey = ~0ull;
-
-__device__ __forceinline__ uint64_t cal_key(uint32_t ref, uint32_t strand, int64_t cal) {
-  return (static_cast<uint64_t>(ref) << 60) | (static_cast<uint64_t>(strand) << 59) |
-         static_cast<uint64_t>(cal + static_cast<int64_t>(kCalBias));
-}
-
-// ASCII -> 2-bit code; 4 for a non-ACGT byte
-__device__ __forceinline__ uint32_t code_of(char ch) {
-  switch (static_cast<unsigned>(static_cast<unsigned char>(ch)) | 0x20u) {
-    case 'a': return 0;
-    case 'c': return 1;
-    case 'g': return 2;
-    case 't': return 3;
-    default: return 4;
-  }
-}
-
-// entries [l, e) of the sorted keys K[s0 .. s1) equal to key
-template <typename KT>
-__device__ __forceinline__ void key_range(const KT* K, uint64_t s0, uint64_t s1, uint32_t key, uint64_t* lo,
-                                          uint64_t* hi) {
-  uint64_t l = s0, u = s1;
-  while (l < u) {
-    const uint64_t mid = l + ((u - l) >> 1);
-    if (K[mid] < key) l = mid + 1;
-    else u = mid;
-  }
-  uint64_t e = l;
-  while (e < s1 && K[e] == key) ++e;
-  *lo = l;
-  *hi = e;
-}
-
-// packed index: entries [lo, hi) of reference r with key `key` in bucket b
-// (16-bit keys in key16, 32-bit ones in key)
-__device__ __forceinline__ void lookup_packed(const DevIndex& di, uint64_t b, uint32_t key, int r, uint64_t* lo,
-                                              uint64_t* hi) {
-  const uint64_t s0 = di.jptr[b * di.n_refs + r], s1 = di.jptr[(b + 1) * di.n_refs + r];
-  if (di.key_bits == 16) key_range(di.key16[r], s0, s1, key, lo, hi);
-  else key_range(di.key[r], s0, s1, key, lo, hi);
-}
-
-// 32-bit keys: the head holds up to kHeadKeys32, one per word
-__device__ __forceinline__ bool head_range32(const uint4 v0, const uint4 v1, const uint4 v2, const uint4 v3,
-                                             uint32_t key, uint32_t* lo0, uint32_t* hi0, uint32_t* lo1,
-                                             uint32_t* hi1) {
-  const uint32_t w[13] = {v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w, v3.x, v3.y, v3.z, v3.w};
-  uint32_t eq = 0;
-#pragma unroll
-  for (int j = 0; j < 13; ++j) eq |= (w[j] == key ? 1u : 0u) << j;
-  const uint32_t n0 = v0.z & 0xffffu, n1 = v0.z >> 16;
-  const uint32_t m0 = (1u << n0) - 1u, m1 = ((1u << (n0 + n1)) - 1u) & ~m0;
-  const uint32_t e0 = eq & m0, e1 = eq & m1;
-  *lo0 = v0.x + (e0 ? __ffs(e0) - 1u : 0u);
-  *hi0 = *lo0 + __popc(e0);
-  *lo1 = v0.y + (e1 ? __ffs(e1) - 1u - n0 : 0u);
-  *hi1 = *lo1 + __popc(e1);
-  return true;
-}
-
-// packed index with bucket heads: entries [lo0, hi0) of reference 0 and [lo1,
-// hi1) of reference 1 with key `key` in bucket b, from the bucket's head alone
-// (an empty range may start anywhere); false when the bucket spilled (its
-// entries are then looked up in jptr / key16)
-__device__ __forceinline__ bool lookup_head(const uint4* heads, uint64_t b, uint32_t key, int key_bits,
-                                            uint32_t* lo0, uint32_t* hi0, uint32_t* lo1, uint32_t* hi1) {
-  const uint4* h = heads + b * 4;
-  const uint4 v0 = __ldg(h), v1 = __ldg(h + 1), v2 = __ldg(h + 2), v3 = __ldg(h + 3);
-  if (v0.z == kHeadSpill) return false;
-  if (key_bits != 16) return head_range32(v0, v1, v2, v3, key, lo0, hi0, lo1, hi1);
-  const uint32_t w[13] = {v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w, v3.x, v3.y, v3.z, v3.w};
-  // bit i: the head's key i equals the seed's, two keys per word: a 16-bit half
-  // of w ^ (key, key) is zero exactly when adding 0x7fff to its low 15 bits
-  // leaves its top bit clear and its top bit was clear
-  const uint32_t kk = key | (key << 16);
-  uint32_t eq = 0;
-#pragma unroll
-  for (int j = 0; j < 13; ++j) {
-    const uint32_t x = w[j] ^ kk;
-    const uint32_t z = ~(((x & 0x7fff7fffu) + 0x7fff7fffu) | x) & 0x80008000u;
-    eq |= (((z >> 15) & 1u) | (z >> 30)) << (2 * j);
-  }
-  // equal keys are consecutive within each reference's run of sorted keys
-  const uint32_t n0 = v0.z & 0xffffu, n1 = v0.z >> 16;
-  const uint32_t m0 = (1u << n0) - 1u, m1 = ((1u << (n0 + n1)) - 1u) & ~m0;
-  const uint32_t e0 = eq & m0, e1 = eq & m1;
-  *lo0 = v0.x + (e0 ? __ffs(e0) - 1u : 0u);
-  *hi0 = *lo0 + __popc(e0);
-  *lo1 = v0.y + (e1 ? __ffs(e1) - 1u - n0 : 0u);
-  *hi1 = *lo1 + __popc(e1);
-  return true;
-}
-
-// entries [lo, hi) of reference r whose key equals the seed's
-__device__ __forceinline__ void lookup(const DevIndex& di, int r, uint64_t canon, uint64_t* lo, uint64_t* hi) {
-  const int kb = 2 * (di.k - di.a);
-  const uint64_t h = seed_hash(canon, di.k, di.hash_seed[r]);
-  const uint64_t b = h >> kb;
-  const uint32_t key = static_cast<uint32_t>(h & mask_bits(kb));
-  uint64_t s0 = di.ptr[r][b], s1 = di.ptr[r][b + 1];
-  const uint32_t* K = di.key[r];
-  // lower bound of key in the bucket
-  uint64_t l = s0, u = s1;
-  while (l < u) {
-    const uint64_t mid = l + ((u - l) >> 1);
-    if (K[mid] < key) l = mid + 1;
-    else u = mid;
-  }
-  uint64_t e = l;
-  while (e < s1 && K[e] == key) ++e;
-  *lo = l;
-  *hi = e;
-}
-
-// read r's codes into shared memory; false (and status) on a non-ACGT base
-__device__ __forceinline__ bool load_codes(const char* bases, uint64_t o0, uint32_t m, uint8_t* q, int lane,
-                                           uint32_t* status) {
-  bool bad = false;
-  for (uint32_t t = lane; t < m; t += 32) {
-    const uint32_t c = code_of(bases[o0 + t]);
-    bad |= c > 3;
-    q[t] = static_cast<uint8_t>(c & 3);
-  }
-  bad = __any_sync(FULL, bad);
-  if (bad && lane == 0) atomicOr(status, kStBadBase);
-  __syncwarp();
-  return !bad;
-}
-
-// The read's codes as 2-bit fields, first base highest, in kPackWords 32-bit
-// words (kMaxReadLen bases and two words of padding): Pk for the read, Rk for
-// the reverse complement of the read padded to kMaxReadLen bases, so that a
-// seed's forward and reverse-complement k-mers (Kmer's fwd and rc) are each
-// read with two funnel shifts.  Bases past the read's end are never extracted.
-constexpr int kPackWords = kMaxReadLen / 16 + 2;
-
-// q: the codes (one byte each, 4-byte aligned); lanes 0-15 pack word j
-__device__ __forceinline__ void pack_codes(const uint8_t* q, uint32_t* Pk, uint32_t* Rk, int lane) {
-  const uint32_t* q32 = reinterpret_cast<const uint32_t*>(q);
-  uint32_t w = 0;
-  if (lane < kMaxReadLen / 16) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      // four codes, first in byte 0, to one byte with the first code highest
-      const uint32_t x = __byte_perm(q32[4 * lane + i] & 0x03030303u, 0, 0x0123);
-      const uint32_t t = (x | (x >> 6)) & 0x000F000Fu;
-      w = (w << 8) | ((t | (t >> 12)) & 0xFFu);
-    }
-  }
-  // the reverse complement: words in reverse order, 2-bit fields reversed, complemented
-  const uint32_t src = __shfl_sync(FULL, w, (kMaxReadLen / 16 - 1 - lane) & 31);
-  uint32_t r = __brev(~src);
-  r = ((r >> 1) & 0x55555555u) | ((r << 1) & 0xAAAAAAAAu);
-  if (lane < kMaxReadLen / 16) {
-    Pk[lane] = w;
-    Rk[lane] = r;
-  } else if (lane < kPackWords) {
-    Pk[lane] = 0;
-    Rk[lane] = 0;
-  }
-  __syncwarp();
-}
-
-// the k bases at o of a packed string, first base highest (k <= 32)
-__device__ __forceinline__ uint64_t kmer_at(const uint32_t* W, uint32_t o, int k) {
-  const uint32_t b = 2 * o, j = b >> 5, s = b & 31;
-  const uint32_t w0 = W[j], w1 = W[j + 1], w2 = W[j + 2];
-  const uint64_t win = (static_cast<uint64_t>(__funnelshift_l(w1, w0, s)) << 32) | __funnelshift_l(w2, w1, s);
-  return win >> (64 - 2 * k);
-}
 
 struct SeedArgs {
   DevIndex di;
@@ -218,8 +39,8 @@ struct SeedArgs {
   uint64_t* cals;         // emit pass
   uint32_t* actual;       // emit pass: the CALs written for each read (indexed r - r0)
   uint32_t* status;
-  // Seed lookups kept from the count pass for the emit pass (nullptr: the emit
-  // pass looks its seeds up again): per read (indexed r - rbase) its records
+  // Seed lookups kept from the count pass for the emit pass: per read (indexed r -
+  // rbase) its records
   // start at seed_off, one per (seed, reference) in that order; recount (per
   // read) marks the reads whose records could not hold a lookup
   uint64_t* ranges;
@@ -227,14 +48,6 @@ struct SeedArgs {
   uint8_t* recount;
   uint32_t rbase;
 };
-
-// a kept lookup: first matching entry (38 bits), their number (24 bits) and the
-// seed's orientation bits (2)
-constexpr uint32_t kRangeCntMax = (1u << 24) - 1u;
-constexpr uint64_t kRangeLoMax = (1ull << 38) - 1ull;
-__device__ __forceinline__ uint64_t range_pack(uint64_t lo, uint32_t cnt, uint32_t rori) {
-  return (lo << 26) | (static_cast<uint64_t>(cnt) << 2) | rori;
-}
 
 // seeds x references of each read (the lookup records the count pass keeps);
 // reads with decreasing offsets or over kMaxReadLen bases set kStBadRead
@@ -276,16 +89,13 @@ __global__ void __launch_bounds__(32 * kCalWarps, 12) k_cal_seeds(SeedArgs a) {
     // offsets and lengths: checked on the host for host reads, here for device reads
     const bool len_ok = o1 >= o0 && o1 - o0 <= static_cast<uint64_t>(kMaxReadLen);
     if (!len_ok && lane == 0) atomicOr(a.status, kStBadRead);
-    // the emit pass takes the count pass's lookups when they were kept for this read
-    const bool kept = EMIT && a.ranges && !a.recount[r - a.rbase];
-    // emit pass: a read of more CALs than kCalSmemKeys whose lookups were kept
-    // is left to k_cal_emit_big (its bound, in count, is then its exact count)
-    const bool split = kept && a.count && a.count[rr] > kCalSmemKeys;
+    // emit pass: the reads whose lookups were kept are k_cal_emit_big's (their
+    // bound, in count, is their exact count)
+    const bool split = EMIT && !a.recount[r - a.rbase];
     uint64_t* rec = a.ranges ? a.ranges + (len_ok ? a.seed_off[r - a.rbase] : 0u) : nullptr;
     bool fits = true;
-    if (!split && len_ok && (kept || load_codes(a.bases, o0, m, q, lane, a.status)) &&
-        m >= static_cast<uint32_t>(k)) {
-      if (!kept) pack_codes(q, pk_s[warp], rk_s[warp], lane);
+    if (!split && len_ok && load_codes(a.bases, o0, m, q, lane, a.status) && m >= static_cast<uint32_t>(k)) {
+      pack_codes(q, pk_s[warp], rk_s[warp], lane);
       const uint64_t base = EMIT ? a.off[rr] : 0;
       // 32 seeds per round, one per lane; the matching entries of all of them
       // are then shared out over the warp (a repeat seed may have thousands)
@@ -293,42 +103,30 @@ __global__ void __launch_bounds__(32 * kCalWarps, 12) k_cal_seeds(SeedArgs a) {
         const uint32_t o = o_base + lane * a.stride;
         const uint32_t si = si_base + lane;  // the seed's index in the read
         const bool live = o + k <= m;
-        uint64_t canon = 0;
-        uint32_t rori = 0;
-        if (!kept) {
-          // Kmer's fwd and rc of the seed (the reverse complement's k-mer at
-          // kMaxReadLen - o - k of the padded reverse complement)
-          const uint64_t fwd = live ? kmer_at(pk_s[warp], o, k) : 0;
-          const uint64_t rc = live ? kmer_at(rk_s[warp], kMaxReadLen - o - k, k) : 0;
-          canon = fwd < rc ? fwd : rc;
-          rori = (fwd == canon ? 1u : 0u) | (rc == canon ? 2u : 0u);
-        }
+        // Kmer's fwd and rc of the seed (the reverse complement's k-mer at
+        // kMaxReadLen - o - k of the padded reverse complement)
+        const uint64_t fwd = live ? kmer_at(pk_s[warp], o, k) : 0;
+        const uint64_t rc = live ? kmer_at(rk_s[warp], kMaxReadLen - o - k, k) : 0;
+        const uint64_t canon = fwd < rc ? fwd : rc;
+        const uint32_t rori = (fwd == canon ? 1u : 0u) | (rc == canon ? 2u : 0u);
         // packed index: one hash (the references share its seed) gives the bucket
         // and key in every reference
         uint64_t pb = 0;
         uint32_t pkey = 0;
-        if (a.di.packed && !kept && live) {
+        if (a.di.packed && live) {
           const int kb = 2 * (k - a.di.a);
           const uint64_t h = seed_hash(canon, k, a.di.hash_seed[0]);
           pb = h >> kb;
           pkey = static_cast<uint32_t>(h & mask_bits(kb));
         }
-        // with bucket heads, one access answers both references (at most two);
-        // the count pass only (the emit pass reads the lookups it kept)
+        // with bucket heads, one access answers both references (at most two)
         uint32_t hl0 = 0, hh0 = 0, hl1 = 0, hh1 = 0;
         bool head = false;
-        if (!EMIT && a.di.heads && live)
+        if (a.di.heads && live)
           head = lookup_head(a.di.heads, pb, pkey, a.di.key_bits, &hl0, &hh0, &hl1, &hh1);
         for (int r2 = 0; r2 < a.di.n_refs; ++r2) {
           uint64_t lo = 0, hi = 0;
-          if (kept) {
-            if (live) {
-              const uint64_t x = rec[static_cast<uint64_t>(si) * a.di.n_refs + r2];
-              lo = x >> 26;
-              hi = lo + ((x >> 2) & kRangeCntMax);
-              rori = static_cast<uint32_t>(x & 3u);
-            }
-          } else if (live) {
+          if (live) {
             if (head) {
               lo = r2 ? hl1 : hl0;
               hi = r2 ? hh1 : hh0;
@@ -381,14 +179,9 @@ __global__ void __launch_bounds__(32 * kCalWarps, 12) k_cal_seeds(SeedArgs a) {
             const uint32_t fo = a.di.packed ? po >> 30 : a.di.orient[r2][e];
             const bool plus = ((fo & 1u) && (sro & 1u)) || ((fo & 2u) && (sro & 2u));
             const bool minus = ((fo & 1u) && (sro & 2u)) || ((fo & 2u) && (sro & 1u));
-            if (EMIT) {
-              const int64_t p = a.di.packed ? (po & 0x3fffffffu) : a.di.pos[r2][e];
-              if (plus) a.cals[base + atomicAdd(&ctr[warp], 1u)] = cal_key(r2, 0, p - so);
-              if (minus) a.cals[base + atomicAdd(&ctr[warp], 1u)] =
-                  cal_key(r2, 1, p - static_cast<int64_t>(m - so - k));
-            } else {
-              n += (plus ? 1u : 0u) + (minus ? 1u : 0u);
-            }
+            const int64_t p = a.di.packed ? (po & 0x3fffffffu) : a.di.pos[r2][e];
+            if (plus) a.cals[base + atomicAdd(&ctr[warp], 1u)] = cal_key(r2, 0, p - so);
+            if (minus) a.cals[base + atomicAdd(&ctr[warp], 1u)] = cal_key(r2, 1, p - static_cast<int64_t>(m - so - k));
           }
           __syncwarp();
         }
@@ -406,31 +199,6 @@ __global__ void __launch_bounds__(32 * kCalWarps, 12) k_cal_seeds(SeedArgs a) {
     }
     __syncwarp();
   }
-}
-
-// block-wide bitonic sort of P (a power of two) keys, ascending
-__device__ void bitonic(uint64_t* s, uint32_t P) {
-  for (uint32_t size = 2; size <= P; size <<= 1) {
-    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      for (uint32_t i = threadIdx.x; i < P / 2; i += blockDim.x) {
-        const uint32_t lo = 2 * i - (i & (stride - 1));
-        const uint32_t hi = lo + stride;
-        const bool up = (lo & size) == 0;
-        const uint64_t x = s[lo], y = s[hi];
-        if ((x > y) == up) {
-          s[lo] = y;
-          s[hi] = x;
-        }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__device__ __forceinline__ uint32_t pow2_at_least(uint32_t n) {
-  uint32_t p = 1;
-  while (p < n) p <<= 1;
-  return p;
 }
 
 // the large read (index into big) and the part of it (tile or chunk) this block
@@ -465,130 +233,13 @@ struct FilterArgs {
   const uint32_t* actual; // CALs of each read
   const uint64_t* off;    // first slot of each read in cals / the window arrays
   uint64_t* cals;
-  uint32_t smem_cap;      // reads with more CALs are left to the large-read kernel
   uint32_t* nwin;         // windows per read
   uint64_t* wkey;         // window CAL key (then reused for the start)
   uint32_t* whits;
   uint32_t* wlen;
 };
 
-// Block-wide exclusive prefix sum of one 64-bit value per thread; *total gets
-// the block's sum.  (Two 32-bit counts packed as high:low add without carries
-// while each total stays below 2^32.)
-__device__ uint64_t block_exscan(uint64_t v, uint64_t* total) {
-  __shared__ uint64_t warp_sum[32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  uint64_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t y = __shfl_up_sync(FULL, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_sum[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    uint64_t t = lane < nw ? warp_sum[lane] : 0ull;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(FULL, t, o);
-      if (lane >= o) t += y;
-    }
-    if (lane < nw) warp_sum[lane] = t;
-  }
-  __syncthreads();
-  const uint64_t before = (w ? warp_sum[w - 1] : 0ull) + x - v;
-  *total = warp_sum[nw - 1];
-  __syncthreads();
-  return before;
-}
-
-// The filter of one read (whole block).  keys has room for P CALs (P the power
-// of two at or above n) followed by the merge's work space: cal_filter_words(P)
-// words in all.
-//
-// The merge (Sec. 3.3) in parallel: in the sorted CALs, a window starts where
-// the (ref, strand) changes or the gap to the previous CAL exceeds merge_dist,
-// and a run of equal values starts where the value changes.  One prefix sum
-// numbers both; every run offers (length, position in its window) to its
-// window by an atomic max, so each window keeps its most frequent value and,
-// among equally frequent ones, the first (smallest) -- the rule a serial scan
-// of the sorted CALs applies.
-__device__ void filter_finish(const FilterArgs& a, uint32_t rr, uint64_t* keys, uint32_t nw);
 __device__ __forceinline__ void window_clamp(const FilterArgs& a, uint64_t base, uint32_t m, uint32_t i);
-
-// keys: the read's work space (keys, then the window and run arrays)
-__device__ void filter_read(const FilterArgs& a, uint32_t rr, uint64_t* keys, uint32_t n) {
-  __shared__ uint32_t s_nw;
-  const uint64_t base = a.off[rr];
-  const uint32_t P = pow2_at_least(n);
-  unsigned long long* wbest = reinterpret_cast<unsigned long long*>(keys + P);  // P per window
-  uint32_t* pos_run = reinterpret_cast<uint32_t*>(keys + 2 * P);                // P + 1 run starts
-  uint32_t* pos_win = pos_run + P + 1;                                          // P + 1 window starts
-  for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) keys[i] = i < n ? a.cals[base + i] : kNoKey;
-  __syncthreads();
-  bitonic(keys, P);
-  const uint32_t T = blockDim.x;
-  const uint32_t per = (n + T - 1) / T;  // each thread a contiguous slice of the sorted CALs
-  const uint32_t i0 = min(n, threadIdx.x * per), i1 = min(n, i0 + per);
-  const uint64_t md = a.merge_dist;
-  auto starts = [&](uint32_t i, bool* rs, bool* ws) {
-    const uint64_t k = keys[i];
-    if (i == 0) {
-      *rs = *ws = true;
-      return;
-    }
-    const uint64_t p = keys[i - 1];
-    *rs = k != p;
-    *ws = (k >> 59) != (p >> 59) || k - p > md;
-  };
-  uint64_t cnt = 0;
-  for (uint32_t i = i0; i < i1; ++i) {
-    bool rs, ws;
-    starts(i, &rs, &ws);
-    cnt += (static_cast<uint64_t>(ws) << 32) | static_cast<uint64_t>(rs);
-  }
-  uint64_t tot = 0;
-  const uint64_t pre = block_exscan(cnt, &tot);
-  const uint32_t nruns = static_cast<uint32_t>(tot), nwin = static_cast<uint32_t>(tot >> 32);
-  {
-    uint32_t rk = static_cast<uint32_t>(pre), wk = static_cast<uint32_t>(pre >> 32);
-    for (uint32_t i = i0; i < i1; ++i) {
-      bool rs, ws;
-      starts(i, &rs, &ws);
-      if (rs) pos_run[rk++] = i;
-      if (ws) pos_win[wk++] = i;
-    }
-  }
-  if (threadIdx.x == 0) {
-    pos_run[nruns] = n;
-    pos_win[nwin] = n;
-  }
-  for (uint32_t j = threadIdx.x; j < nwin; j += T) wbest[j] = 0ull;
-  __syncthreads();
-  {
-    uint32_t rk = static_cast<uint32_t>(pre), wk = static_cast<uint32_t>(pre >> 32);
-    for (uint32_t i = i0; i < i1; ++i) {
-      bool rs, ws;
-      starts(i, &rs, &ws);
-      wk += ws ? 1u : 0u;
-      if (rs) {
-        const uint32_t w = wk - 1;  // the window holding this run
-        const uint32_t len = pos_run[rk + 1] - i, at = i - pos_win[w];
-        atomicMax(&wbest[w], (static_cast<unsigned long long>(len) << 32) | (0xffffffffu - at));
-        ++rk;
-      }
-    }
-  }
-  __syncthreads();
-  for (uint32_t j = threadIdx.x; j < nwin; j += T) {
-    const uint32_t at = 0xffffffffu - static_cast<uint32_t>(wbest[j] & 0xffffffffull);
-    a.wkey[base + j] = keys[pos_win[j] + at];
-    a.whits[base + j] = pos_win[j + 1] - pos_win[j];
-  }
-  if (threadIdx.x == 0) s_nw = nwin;
-  __syncthreads();
-  filter_finish(a, rr, keys, s_nw);
-}
 
 // the end of a read's filter once its nw windows have their key and hits: the
 // max_cands cut (keys: work space of at least the power of two of nw), the
@@ -637,179 +288,8 @@ __device__ __forceinline__ void window_clamp(const FilterArgs& a, uint64_t base,
   a.wkey[base + i] = (key & ~kCalMask) | static_cast<uint64_t>(lo);
 }
 
-// The same filter for a read of at most 32 E CALs on one warp, without block
-// barriers: element e = 32 h + lane of the warp's E registers per lane.  A
-// bitonic network sorts the keys (partners in other lanes by shuffle, in the
-// same lane by register); run and window starts become ballot masks; each run
-// offers (its length, its position in its window) to its window by an atomic
-// max in shared memory; the max_cands cut keeps the windows of rank below it
-// (most hits first, then the smaller key), in key order.
-constexpr int kFilterWarps = 8;
-template <int E>
-__global__ void __launch_bounds__(32 * kFilterWarps) k_cal_filter_warp(FilterArgs a, uint32_t lo, uint32_t hi) {
-  constexpr int P = 32 * E;
-  __shared__ uint64_t sk_s[kFilterWarps][P];                 // sorted keys
-  __shared__ unsigned long long sb_s[kFilterWarps][P];       // per window: (run length << 32) | ~position
-  __shared__ uint32_t sp_s[kFilterWarps][P + 1];             // window starts, then n
-  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  uint64_t* sk = sk_s[wi];
-  unsigned long long* sb = sb_s[wi];
-  uint32_t* sp = sp_s[wi];
-  const uint32_t le = (2u << lane) - 1u;  // lanes at or below this one (lane 31: all)
-  for (uint32_t rr = blockIdx.x * kFilterWarps + wi; rr < a.nr; rr += gridDim.x * kFilterWarps) {
-    const uint32_t c = a.count[rr];
-    if (c < lo || c > hi) continue;
-    const uint32_t n = a.actual[rr];
-    const uint32_t r = a.r0 + rr;
-    const uint64_t base = a.off[rr];
-    const uint32_t m = static_cast<uint32_t>(a.read_off[r + 1] - a.read_off[r]);
-    uint64_t k[E];
-#pragma unroll
-    for (int h = 0; h < E; ++h) {
-      const uint32_t e = 32 * h + lane;
-      k[h] = e < n ? a.cals[base + e] : kNoKey;
-    }
-    // bitonic sort, ascending: the lower index of a pair keeps the minimum in
-    // ascending runs ((e & size) == 0), the maximum in descending ones
-#pragma unroll
-    for (int size = 2; size <= P; size <<= 1) {
-#pragma unroll
-      for (int stride = size / 2; stride > 0; stride >>= 1) {
-        if (stride >= 32) {
-          const int hs = stride / 32;
-#pragma unroll
-          for (int h = 0; h < E; ++h) {
-            if (h & hs) continue;
-            const uint32_t e = 32 * h + lane;
-            const bool up = (e & size) == 0;
-            const uint64_t x = k[h], y = k[h | hs];
-            if ((x > y) == up) {
-              k[h] = y;
-              k[h | hs] = x;
-            }
-          }
-        } else {
-#pragma unroll
-          for (int h = 0; h < E; ++h) {
-            const uint32_t e = 32 * h + lane;
-            const uint64_t y = __shfl_xor_sync(FULL, k[h], stride);
-            const bool up = (e & size) == 0, low = (lane & stride) == 0;
-            k[h] = (low == up) ? (k[h] < y ? k[h] : y) : (k[h] > y ? k[h] : y);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < E; ++h) sk[32 * h + lane] = k[h];
-    __syncwarp();
-    // run starts (value changes) and window starts ((ref, strand) changes or a
-    // gap over merge_dist), as masks of the E groups of 32 elements
-    uint32_t rm[E], wm[E];
-    uint32_t nwin = 0;
-#pragma unroll
-    for (int h = 0; h < E; ++h) {
-      const uint32_t e = 32 * h + lane;
-      bool rs = false, ws = false;
-      if (e < n) {
-        if (e == 0) {
-          rs = ws = true;
-        } else {
-          const uint64_t p = sk[e - 1];
-          rs = k[h] != p;
-          ws = (k[h] >> 59) != (p >> 59) || k[h] - p > a.merge_dist;
-        }
-      }
-      rm[h] = __ballot_sync(FULL, rs);
-      wm[h] = __ballot_sync(FULL, ws);
-      nwin += __popc(wm[h]);
-    }
-    for (uint32_t j = lane; j < nwin; j += 32) sb[j] = 0ull;
-    __syncwarp();
-    uint32_t wbefore = 0;  // window starts in the groups before h
-#pragma unroll
-    for (int h = 0; h < E; ++h) {
-      const uint32_t e = 32 * h + lane;
-      if ((wm[h] >> lane) & 1u) sp[wbefore + __popc(wm[h] & (le >> 1))] = e;
-      if ((rm[h] >> lane) & 1u) {
-        // the window holding this run, the next run start, this run's window start
-        const uint32_t w = wbefore + __popc(wm[h] & le) - 1u;
-        uint32_t next = n;
-        const uint32_t above = rm[h] & ~le;
-        if (above) {
-          next = 32 * h + __ffs(above) - 1;
-        } else {
-#pragma unroll
-          for (int h2 = E - 1; h2 > h; --h2)
-            if (rm[h2]) next = 32 * h2 + __ffs(rm[h2]) - 1;
-        }
-        uint32_t wst = 0;
-        const uint32_t below = wm[h] & le;
-        if (below) {
-          wst = 32 * h + 31 - __clz(below);
-        } else {
-#pragma unroll
-          for (int h2 = 0; h2 < h; ++h2)
-            if (wm[h2]) wst = 32 * h2 + 31 - __clz(wm[h2]);
-        }
-        atomicMax(&sb[w], (static_cast<unsigned long long>(next - e) << 32) | (0xffffffffu - (e - wst)));
-      }
-      wbefore += __popc(wm[h]);
-    }
-    if (lane == 0) sp[nwin] = n;
-    __syncwarp();
-    // windows kept (all, or the max_cands of rank below it) in key order, each
-    // clamped to [cal - pad, cal + m + pad) within its reference
-    const bool cut = a.max_cands && nwin > a.max_cands;
-    uint32_t kept_before = 0;
-    for (uint32_t j0 = 0; j0 < nwin; j0 += 32) {
-      const uint32_t j = j0 + lane;
-      const bool in = j < nwin;
-      const uint32_t hits = in ? sp[j + 1] - sp[j] : 0u;
-      bool keep = in;
-      if (cut && in) {
-        uint32_t rank = 0;
-        for (uint32_t q = 0; q < nwin; ++q) {
-          const uint32_t hq = sp[q + 1] - sp[q];
-          rank += (hq > hits || (hq == hits && q < j)) ? 1u : 0u;
-        }
-        keep = rank < a.max_cands;
-      }
-      const uint32_t km = __ballot_sync(FULL, keep);
-      if (keep) {
-        const uint32_t dst = kept_before + __popc(km & (le >> 1));
-        const uint32_t at = 0xffffffffu - static_cast<uint32_t>(sb[j] & 0xffffffffull);
-        const uint64_t key = sk[sp[j] + at];
-        const uint32_t ref = static_cast<uint32_t>(key >> 60);
-        const int64_t cal = static_cast<int64_t>(key & kCalMask) - static_cast<int64_t>(kCalBias);
-        const int64_t N = static_cast<int64_t>(a.di.ref_len[ref]);
-        int64_t wlo = cal - static_cast<int64_t>(a.pad), whi = cal + m + static_cast<int64_t>(a.pad);
-        if (wlo < 0) wlo = 0;
-        if (whi > N) whi = N;
-        a.wkey[base + dst] = (key & ~kCalMask) | static_cast<uint64_t>(wlo);
-        a.whits[base + dst] = hits;
-        a.wlen[base + dst] = static_cast<uint32_t>(whi - wlo);
-      }
-      kept_before += __popc(km);
-    }
-    if (lane == 0) a.nwin[rr] = kept_before;
-    __syncwarp();
-  }
-}
-
-// reads with lo <= count <= hi, keys in shared memory
-__global__ void __launch_bounds__(256) k_cal_filter(FilterArgs a, uint32_t lo, uint32_t hi) {
-  extern __shared__ uint64_t skeys[];
-  for (uint32_t rr = blockIdx.x; rr < a.nr; rr += gridDim.x) {
-    const uint32_t n = a.count[rr];
-    if (n < lo || n > hi) continue;
-    filter_read(a, rr, skeys, a.actual[rr]);
-  }
-}
-
-// one block per large read (big[b]), keys in a global scratch from slot soff[b]
-// reads of more than kCalSmemKeys CALs, one block each, once the large-read
-// merge below has given them their windows: the max_cands cut where it applies
-// (the merge has clamped the windows of the others)
+// one block per read, once the merge below has given the reads their windows:
+// the max_cands cut where it applies (the merge has clamped the other windows)
 __global__ void __launch_bounds__(1024) k_cal_filter_big(FilterArgs a, const uint32_t* big, const uint64_t* soff,
                                                          uint64_t* scratch) {
   const uint32_t rr = big[blockIdx.x];
@@ -1088,7 +568,7 @@ int launch_cal_emit_big(const DevIndex& di, const uint64_t* read_off, uint32_t r
                         const uint32_t* bound, const uint64_t* off, uint64_t* cals, const CalRanges& kept,
                         const uint32_t* big, uint32_t n_big, uint64_t* scratch, uint64_t scratch_words,
                         cudaStream_t st) {
-  if (nr == 0 || n_big == 0 || !kept.ranges) return 0;
+  if (nr == 0 || n_big == 0) return 0;
   SeedArgs a{di, nullptr, read_off, r0, nr, stride, const_cast<uint32_t*>(bound), off, cals, nullptr, nullptr,
              kept.ranges, kept.seed_off, kept.recount, kept.rbase};
   uint32_t* chunks = reinterpret_cast<uint32_t*>(scratch + scratch_words);
@@ -1122,8 +602,9 @@ int launch_cal_seeds(const DevIndex& di, const char* bases, const uint64_t* read
 // value changes) and window starts ((reference, strand) changes, or a gap over
 // merge_dist) are counted per tile, numbered by scans over the tiles, and each
 // run offers (its length, its position in its window) to its window by an
-// atomic max: the rule of filter_read, by many blocks.  The layout of a read's
-// work space is filter_read's (keys, window bests, run starts, window starts).
+// atomic max, so each window keeps its most frequent value and, among equally
+// frequent ones, the first (smallest).  A read's work space: its keys, window
+// bests, run starts, window starts (cal_scratch_words).
 struct MergeTabs {
   uint32_t *trs, *tws;  // run and window starts per tile
   uint64_t *prs, *pws;  // their exclusive prefixes over all tiles (tiles + 1 entries)
@@ -1241,52 +722,11 @@ __global__ void __launch_bounds__(1024) k_bmerge_out(FilterArgs a, const uint32_
 
 int launch_cal_filter(const DevIndex& di, const uint64_t* read_off, uint32_t r0, uint32_t nr, uint32_t merge_dist,
                       uint32_t pad, uint32_t max_cands, const uint32_t* count, const uint32_t* actual,
-                      const uint64_t* off, uint64_t* cals, uint32_t max_small, uint32_t max_mid, const uint32_t* big,
-                      const uint64_t* big_soff, uint32_t n_big, uint64_t* scratch, uint64_t scratch_words,
+                      const uint64_t* off, uint64_t* cals, const uint32_t* big, const uint64_t* big_soff, uint32_t n_big, uint64_t* scratch, uint64_t scratch_words,
                       uint32_t* nwin, uint64_t* wkey, uint32_t* whits, uint32_t* wlen, cudaStream_t st) {
   if (nr == 0) return 0;
-  FilterArgs a{di, read_off, r0, nr, merge_dist, pad, max_cands, count, actual, off, cals, kCalSmemKeys,
-               nwin, wkey, whits, wlen};
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_cal_filter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(cal_filter_words(kCalSmemKeys) * sizeof(uint64_t))) != cudaSuccess)
-      return -1;
-    attr = true;
-  }
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  auto p2 = [](uint32_t n) {
-    uint32_t p = 1;
-    while (p < n) p <<= 1;
-    return p;
-  };
+  FilterArgs a{di, read_off, r0, nr, merge_dist, pad, max_cands, count, actual, off, cals, nwin, wkey, whits, wlen};
   int launched = 0;
-  // reads of at most 64 and of 65-128 CALs: one warp each
-  {
-    const uint32_t warps = static_cast<uint32_t>(nsm) * 8 * kFilterWarps;
-    const uint32_t grid = (std::min(nr, warps) + kFilterWarps - 1) / kFilterWarps;
-    k_cal_filter_warp<2><<<grid, 32 * kFilterWarps, 0, st>>>(a, 0u, 64u);
-    ++launched;
-    if (max_small > 64) {
-      k_cal_filter_warp<4><<<grid, 32 * kFilterWarps, 0, st>>>(a, 65u, 128u);
-      ++launched;
-    }
-  }
-  // the other small reads: 24 KB or less of shared memory per block, many blocks per SM
-  if (max_small > 128) {
-    const size_t smem = static_cast<size_t>(cal_filter_words(p2(max_small))) * sizeof(uint64_t);
-    const uint32_t grid = nr < static_cast<uint32_t>(nsm) * 32 ? nr : static_cast<uint32_t>(nsm) * 32;
-    k_cal_filter<<<grid, 128, smem, st>>>(a, 129u, kCalSmallKeys);
-    ++launched;
-  }
-  if (max_mid) {
-    const size_t smem = static_cast<size_t>(cal_filter_words(p2(max_mid))) * sizeof(uint64_t);
-    const uint32_t grid = static_cast<uint32_t>(nsm) * 2;
-    k_cal_filter<<<grid, 256, smem, st>>>(a, kCalSmallKeys + 1, kCalSmemKeys);
-    ++launched;
-  }
   if (n_big) {
     // the large reads' keys sorted by the whole GPU, then each read's windows by
     // one block; the reads' classes of sort length come back to the host, which
@@ -1400,38 +840,38 @@ __global__ void __launch_bounds__(kScanBlock64) k_scan64_b(uint64_t* sums, uint3
   if (threadIdx.x == 0) *end = carry;
 }
 
+// the whole scan by one block (small n: one launch instead of three)
+constexpr uint32_t kScanOne = 8 * kScanBlock64;
+__global__ void __launch_bounds__(kScanBlock64) k_scan64_one(const uint32_t* in, uint32_t n, uint64_t* out) {
+  uint64_t carry = 0;
+  for (uint32_t b0 = 0; b0 < n; b0 += kScanBlock64) {
+    const uint32_t i = b0 + threadIdx.x;
+    const uint64_t v = i < n ? in[i] : 0u;
+    uint64_t tot = 0;
+    const uint64_t x = block_exscan(v, &tot);
+    if (i < n) out[i] = carry + x;
+    carry += tot;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
 __global__ void k_scan64_c(uint64_t* out, uint32_t n, const uint64_t* sums) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] += sums[i / kScanBlock64];
 }
 
-// the filter's routing of reads by their CAL bounds (big: nullptr to take the
-// maxima only)
+// the reads with CALs listed with their scratch offsets, and the largest bound
+// (big: nullptr to take the maximum only)
 __global__ void k_cal_route(const uint32_t* count, uint32_t nr, uint32_t* big, uint64_t* big_soff, CalPlan* plan) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t c = i < nr ? count[i] : 0u;
-  uint32_t small = 0, mid = 0;
-  if (i < nr) {
-    if (c > kCalSmemKeys) {
-      if (big) {
-        const uint32_t b = atomicAdd(&plan->n_big, 1u);
-        big[b] = i;
-        big_soff[b] = atomicAdd(&plan->scratch, static_cast<unsigned long long>(cal_filter_words(pow2_at_least(c))));
-      }
-    } else if (c > kCalSmallKeys) {
-      mid = c;
-    } else {
-      small = c;
-    }
+  if (c && big) {
+    const uint32_t b = atomicAdd(&plan->n_big, 1u);
+    big[b] = i;
+    big_soff[b] = atomicAdd(&plan->scratch, static_cast<unsigned long long>(cal_scratch_words(pow2_at_least(c))));
   }
   const uint32_t all = __reduce_max_sync(FULL, c);
-  small = __reduce_max_sync(FULL, small);
-  mid = __reduce_max_sync(FULL, mid);
-  if ((threadIdx.x & 31) == 0) {
-    if (small) atomicMax(&plan->max_small, small);
-    if (mid) atomicMax(&plan->max_mid, mid);
-    if (all) atomicMax(&plan->max_all, all);
-  }
+  if ((threadIdx.x & 31) == 0 && all) atomicMax(&plan->max_all, all);
 }
 
 // bounds[p / span] = the first read whose prefix p = pre[r] falls in that span
@@ -1453,6 +893,10 @@ __global__ void k_cal_rebase(const uint64_t* pre, uint32_t a, uint32_t cnt, uint
 }  // namespace
 
 int launch_scan_u64(const uint32_t* in, uint32_t n, uint64_t* out, uint64_t* sums, cudaStream_t st) {
+  if (n <= kScanOne) {
+    k_scan64_one<<<1, kScanBlock64, 0, st>>>(in, n, out);
+    return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+  }
   const uint32_t nb = (n + kScanBlock64 - 1) / kScanBlock64;
   if (nb) k_scan64_a<<<nb, kScanBlock64, 0, st>>>(in, n, out, sums);
   k_scan64_b<<<1, kScanBlock64, 0, st>>>(sums, nb, out + n);
@@ -1499,7 +943,6 @@ int preload_cal() {
   SR_TOUCH(k_cal_heads);
   SR_TOUCH(k_cal_seeds<false>);
   SR_TOUCH(k_cal_seeds<true>);
-  SR_TOUCH(k_cal_filter);
   SR_TOUCH(k_cal_filter_big);
   SR_TOUCH(k_emit_count);
   SR_TOUCH(k_cal_emit_big);
@@ -1512,10 +955,9 @@ int preload_cal() {
   SR_TOUCH(k_bsort_local);
   SR_TOUCH(k_bsort_global);
   SR_TOUCH(k_bsort_tail);
-  SR_TOUCH(k_cal_filter_warp<2>);
-  SR_TOUCH(k_cal_filter_warp<4>);
   SR_TOUCH(k_cal_compact);
   SR_TOUCH(k_cal_offsets);
+  SR_TOUCH(k_scan64_one);
   SR_TOUCH(k_scan64_a);
   SR_TOUCH(k_scan64_b);
   SR_TOUCH(k_scan64_c);

@@ -27,6 +27,8 @@ struct IndexTables {
   uint64_t n_entries;
 };
 IndexTables index_tables(const sr_index* idx);
+// frees a device list of sr_candidates_device; false when l is not one
+bool device_list_free(sr_cand_list* l);
 // a zeroed sr_results whose arrays the caller allocates with malloc (released by sr_results_free)
 sr_results* results_alloc();
 // threads of the host pool (workers + the caller), at most 16

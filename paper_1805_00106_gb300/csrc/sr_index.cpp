@@ -386,7 +386,8 @@ extern "C" sr_status sr_cand_list_alloc(uint32_t n_reads, uint64_t n_cands, sr_c
 extern "C" void sr_cand_list_free(sr_cand_list* l) {
   if (!l) return;
   if (l->flags & SR_FLAG_DEVICE) {
-    // a list sr_candidates_device left on the device
+    if (device_list_free(l)) return;
+    // device arrays that the caller put into a list of its own
     void* arrays[6] = {l->offsets, l->ref_id, l->strand, l->win_start, l->win_len, l->hits};
     for (void* p : arrays)
       if (p) cudaFree(p);

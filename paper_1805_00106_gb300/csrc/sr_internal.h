@@ -39,6 +39,7 @@ enum : uint32_t {
   kStTimeout = 1u << 3,    // a bounded wait (TMA mbarrier) ran out
   kStOverflow = 1u << 4,   // int16 guard tripped (never expected: routing is exact)
   kStInternal = 1u << 5,
+  kStBadStart = 1u << 6,   // the first read offset is not 0
 };
 
 struct DevRefs {
@@ -292,11 +293,13 @@ struct DevIndex {
   uint64_t hash_seed[kMaxRefs];
   int n_refs, k, a;
 };
-constexpr uint32_t kCalSmallKeys = 1024;  // reads up to this many CALs: small-block filter (24 KB)
-constexpr uint32_t kCalSmemKeys = 8192;   // up to this many: filtered in shared memory (192 KB)
-// shared or scratch words (u64) the filter of a read of up to P CALs uses (P a
-// power of two): its keys, each window's best run, run and window start positions
-__host__ __device__ constexpr uint64_t cal_filter_words(uint64_t P) { return 3 * P + 1; }
+// keys per tile of the large-read sort and merge
+constexpr uint32_t kCalSortTile = 4096;
+// scratch words (u64) of a large read of up to P CALs (P a power of two): its
+// keys (at least a tile), each window's best run, run and window starts
+__host__ __device__ constexpr uint64_t cal_scratch_words(uint64_t P) {
+  return 3 * (P > kCalSortTile ? P : kCalSortTile) + 1;
+}
 // count pass (cals == nullptr: an upper bound of the CALs of each read into
 // count, exact unless a seed is its own reverse complement; reads with bad
 // offsets or over kMaxReadLen bases set kStBadRead) or emit pass (CAL keys of
@@ -316,10 +319,9 @@ constexpr int kHeadKeys32 = 13;
 constexpr uint32_t kHeadSpill = 0xffffffffu;
 // the bucket heads of a packed index (nbuckets buckets, n_refs <= 2) into heads
 int launch_cal_heads(const DevIndex& di, uint64_t nbuckets, uint4* heads, cudaStream_t st);
-// Emit pass of the large reads (device list big, n_big of them: over
-// kCalSmemKeys CAL bounds) whose lookups were kept, by many blocks per read,
-// after launch_cal_seeds' emit pass (given the bounds as count, it leaves those
-// reads out); its part tables take cal_sort_words(n_big) words after the
+// Emit pass of the reads whose lookups were kept (device list big, n_big of
+// them), by many blocks per read, after launch_cal_seeds' emit pass (which takes
+// the others); its part tables take cal_sort_words(n_big) words after the
 // filter's scratch_words
 int launch_cal_emit_big(const DevIndex& di, const uint64_t* read_off, uint32_t r0, uint32_t nr, uint32_t stride,
                         const uint32_t* bound, const uint64_t* off, uint64_t* cals, const CalRanges& kept,
@@ -332,19 +334,15 @@ int launch_cal_seeds(const DevIndex& di, const char* bases, const uint64_t* read
 // over kMaxReadLen bases set kStBadRead
 int launch_cal_slots(const uint64_t* read_off, uint32_t n, int k, uint32_t stride, int n_refs, uint32_t* slots,
                      uint32_t* status, cudaStream_t st);
-// windows of each read at off[i] (nwin[i] of them).  Reads with up to
-// kCalSmallKeys CALs (largest: max_small) and up to kCalSmemKeys (largest:
-// max_mid, 0 = none) sort in shared memory; the n_big others (device list big
-// of indices into the chunk) sort in scratch from slot big_soff[b] (pow2 of
-// their count each, scratch_words in all), followed by
-// cal_sort_words(n_big, scratch_words) words of the large-read tables
+// windows of each listed read at off[i] (nwin[i] of them): n_big reads (device
+// list big of indices into the chunk) sorted and merged in scratch from slot
+// big_soff[b] (cal_scratch_words of their count each, scratch_words in all),
+// followed by cal_sort_words(n_big, scratch_words) words of tables
 int launch_cal_filter(const DevIndex& di, const uint64_t* read_off, uint32_t r0, uint32_t nr, uint32_t merge_dist,
                       uint32_t pad, uint32_t max_cands, const uint32_t* count, const uint32_t* actual,
-                      const uint64_t* off, uint64_t* cals, uint32_t max_small, uint32_t max_mid, const uint32_t* big,
-                      const uint64_t* big_soff, uint32_t n_big, uint64_t* scratch, uint64_t scratch_words,
-                      uint32_t* nwin, uint64_t* wkey, uint32_t* whits, uint32_t* wlen, cudaStream_t st);
-// keys per tile of the large-read sort and merge
-constexpr uint32_t kCalSortTile = 4096;
+                      const uint64_t* off, uint64_t* cals, const uint32_t* big, const uint64_t* big_soff,
+                      uint32_t n_big, uint64_t* scratch, uint64_t scratch_words, uint32_t* nwin, uint64_t* wkey,
+                      uint32_t* whits, uint32_t* wlen, cudaStream_t st);
 // words after a filter's scratch (scratch_words) for the tables of the
 // large-read emit (the reads' chunk counts, their prefix and its block sums)
 // and, later, of the large-read sort and merge (class counts and fills, the
@@ -361,13 +359,12 @@ int launch_cal_offsets(const uint32_t* woff, uint32_t nr, uint64_t base, uint64_
 // exclusive 64-bit scan of n counts into out[0..n] (out[n] = the total) with a
 // scratch of n / 1024 + 1 words (sr_cal.cu)
 int launch_scan_u64(const uint32_t* in, uint32_t n, uint64_t* out, uint64_t* sums, cudaStream_t st);
-// The CAL filter's routing of nr reads by their CAL bounds: reads over
-// kCalSmemKeys CALs listed in big (indices into the reads, in any order) with
-// their scratch offsets in big_soff, and the largest small, mid-size and
-// overall bound; big = nullptr takes the maxima only.  plan must be zeroed.
+// The reads with CALs (of nr, by their CAL bounds) listed in big (indices into
+// the reads, in any order) with their scratch offsets in big_soff, and the
+// largest bound; big = nullptr takes the maximum only.  plan must be zeroed.
 struct CalPlan {
-  unsigned long long scratch;  // scratch words of the listed large reads
-  unsigned int n_big, max_small, max_mid, max_all;
+  unsigned long long scratch;  // scratch words of the listed reads
+  unsigned int n_big, max_all;
 };
 int launch_cal_route(const uint32_t* count, uint32_t nr, uint32_t* big, uint64_t* big_soff, CalPlan* plan,
                      cudaStream_t st);
@@ -382,6 +379,51 @@ int launch_cal_rebase(const uint64_t* pre, uint32_t a, uint32_t cnt, uint64_t* o
 int launch_cal_compact(uint32_t nr, const uint64_t* off, const uint32_t* nwin, const uint32_t* woff,
                        const uint64_t* wkey, const uint32_t* whits, const uint32_t* wlen, uint8_t* o_ref,
                        uint8_t* o_strand, uint64_t* o_start, uint32_t* o_len, uint32_t* o_hits, cudaStream_t st);
+
+// The CAL finder in one pass per read (sr_find.cu).  Windows are staged in `win`
+// in any order (a read's nwin[i] from slot wslot[i]); plan->cursor counts the
+// slots taken, also past win_cap, where nothing is written: the caller then runs
+// the call again with more.  Reads with more distinct CALs than the tables take
+// end in list_rest (plan->n_rest of them), with nwin 0.
+struct FindPlan {
+  unsigned long long cursor;
+  unsigned int n_mid, n_wide, n_rest;  // reads listed for the block kernels and the large-read path
+  unsigned int q_mid, q_wide;          // their queues
+};
+struct FindArgs {
+  DevIndex di;
+  const char* bases;
+  const uint64_t* read_off;
+  uint32_t r0, nr;  // reads r0 .. r0 + nr; per-read arrays are indexed r - r0
+  uint32_t stride, merge_dist, pad, max_cands;
+  uint32_t merge_keys;  // most distinct CALs a table takes (at most its own size)
+  uint32_t* status;
+  uint4* win;
+  uint64_t win_cap;
+  uint32_t *nwin, *wslot;
+  uint32_t *list_mid, *list_wide, *list_rest;  // nr entries each
+  FindPlan* plan;                              // zeroed by the caller
+};
+// the arrays of a window list in device memory
+struct FindList {
+  uint64_t* off;
+  uint8_t *ref, *strand;
+  uint64_t* start;
+  uint32_t *len, *hits;
+};
+// offsets of device reads: kStBadRead, kStBadStart (launch_find then does nothing)
+int launch_find_check(const uint64_t* read_off, uint32_t n, uint32_t* status, cudaStream_t st);
+int launch_find(const FindArgs& a, cudaStream_t st);
+// the nw windows of nr reads (woff: the exclusive prefix of nwin) from the
+// staging slots to l from window `base` on, and the offsets l.off[0 .. nr]
+int launch_find_out(const uint64_t* woff, uint32_t nr, uint64_t nw, const uint32_t* wslot, const uint4* win, uint64_t base,
+                    const FindList& l, cudaStream_t st);
+// reads list[0 .. n) of r0 .. as a batch of their own: lengths, offsets (sums: a
+// scan's scratch), bases; and its windows back to the staging slots from base on
+int launch_rest_gather(const char* bases, const uint64_t* read_off, uint32_t r0, const uint32_t* list, uint32_t n,
+                       uint32_t* len, uint64_t* off, uint64_t* sums, char* out, cudaStream_t st);
+int launch_rest_stage(const FindList& l, const uint32_t* list, uint32_t n, uint64_t base, uint4* win, uint32_t* nwin,
+                      uint32_t* wslot, cudaStream_t st);
 
 // report options (sr_report.cu): count pass + scan into a scratch of
 // report_scratch_words(n_reads) words, then the write pass
@@ -411,6 +453,7 @@ int preload_extend();
 int preload_kernels();
 int preload_traceback();
 int preload_cal();
+int preload_find();
 int preload_report();
 int preload_noalloc();
 #define SR_TOUCH(k)                                                             \

@@ -13,6 +13,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <unordered_set>
 #include <vector>
 
 #include "sr_host.h"
@@ -133,6 +134,8 @@ enum CalBuf : int {
   kCbBases, kCbRoff, kCbCount, kCbActual, kCbStatus, kCbSlots, kCbPre, kCbSums, kCbBounds, kCbPlan,
   kCbRanges, kCbSeedOff, kCbRecount, kCbCpre, kCbOff, kCbNwin, kCbWoff, kCbWsums, kCbBig, kCbBigOff,
   kCbCals, kCbWkey, kCbWhits, kCbWlen, kCbScratch, kCbLoff, kCbLref, kCbLstr, kCbLstart, kCbLlen, kCbLhits,
+  kCbFnwin, kCbFslot, kCbFmid, kCbFwide, kCbFrest, kCbFwoff, kCbFsums, kCbFplan, kCbWin, kCbRlen, kCbRoff2, kCbRbases,
+  kCbList0, kCbList1,
   kCalBufs
 };
 }  // namespace
@@ -170,6 +173,9 @@ struct sr_session {
   std::mutex cal_mu;
   void* cal_buf[kCalBufs] = {};
   uint64_t cal_bytes[kCalBufs] = {};
+  void* cal_back = nullptr;  // pinned: what comes back of a call's plan
+  // blocks of freed device lists (guarded by pool_mu, not counted in hbm_used)
+  std::vector<std::pair<void*, uint64_t>> list_pool;
 };
 
 struct sr_batch {
@@ -214,6 +220,7 @@ static void preload_all(int dev) {
   preload_kernels();
   preload_traceback();
   preload_cal();
+  preload_find();
   preload_report();
   preload_noalloc();
   cudaGetLastError();
@@ -342,6 +349,8 @@ static void session_release(sr_session* s) {
   for (auto& a : s->spares) cudaFree(a.first);
   for (void* p : s->cal_buf)
     if (p) cudaFree(p);
+  if (s->cal_back) cudaFreeHost(s->cal_back);
+  for (auto& b : s->list_pool) cudaFree(b.first);
   if (s->stream) cudaStreamDestroy(s->stream);
   for (auto x : s->part_stream)
     if (x) cudaStreamDestroy(x);
@@ -1455,6 +1464,358 @@ extern "C" sr_status sr_session_attach_index(sr_session* s, const sr_index* cons
   return SR_OK;
 }
 
+namespace {
+// One sr_candidates_device call: its stream, its CUDA error and the session's
+// cached scratch (grown with a quarter of headroom when a call needs more, so
+// steady-state calls allocate nothing).
+struct CalCall {
+  sr_session* s;
+  cudaStream_t st;
+  sr_cand_params cp;
+  cudaError_t e = cudaSuccess;
+
+  void* buf(int role, uint64_t bytes) { return grow(role, bytes, 0); }
+  // the buffer grown to `bytes`, its first `keep` bytes kept
+  void* grow(int role, uint64_t bytes, uint64_t keep) {
+    if (e != cudaSuccess) return nullptr;
+    bytes = std::max<uint64_t>(bytes, 16);
+    if (s->cal_bytes[role] >= bytes) return s->cal_buf[role];
+    void* was = s->cal_buf[role];
+    if (was && !keep) {
+      // earlier launches of this call may still use the smaller buffer
+      e = cudaStreamSynchronize(st);
+      cudaFree(was);
+      s->cal_buf[role] = was = nullptr;
+      s->cal_bytes[role] = 0;
+      if (e != cudaSuccess) return nullptr;
+    }
+    void* p = nullptr;
+    const uint64_t want = bytes + bytes / 4;
+    e = cudaMalloc(&p, want);
+    if (e == cudaSuccess && was) {
+      e = cudaMemcpyAsync(p, was, keep, cudaMemcpyDeviceToDevice, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) cudaFree(p);
+    }
+    if (e != cudaSuccess) return nullptr;
+    if (was) cudaFree(was);
+    s->cal_buf[role] = p;
+    s->cal_bytes[role] = want;
+    return p;
+  }
+  sr_status fail(const char* msg) {
+    if (e == cudaSuccess) e = cudaGetLastError();
+    return cuda_error(msg, e == cudaSuccess ? cudaErrorUnknown : e);
+  }
+  sr_status no_memory() { return set_error(SR_ENOMEM, "sr_candidates_device: device allocation failed"); }
+};
+
+// ---- device lists.  A list's arrays share one block; the session keeps up to
+// kKeptLists blocks of freed lists for the next ones.  A freed list waits for the
+// device first, as cudaFree did: work on other streams may still read it.
+constexpr size_t kKeptLists = 2;
+struct DevListBox {
+  sr_cand_list pub;  // first: what the caller holds
+  sr_session* s;
+  void* block;
+  uint64_t bytes;
+};
+std::mutex g_lists_mu;
+std::unordered_set<const void*> g_lists;  // the boxes alive
+
+uint64_t list_layout(uint64_t n, uint64_t cap, uint64_t at[7]) {
+  const uint64_t bytes[6] = {(n + 1) * 8, cap, cap, cap * 8, cap * 4, cap * 4};
+  at[0] = 0;
+  for (int k = 0; k < 6; ++k) at[k + 1] = (at[k] + bytes[k] + 255) & ~255ull;
+  return at[6];
+}
+
+FindList list_arrays(void* block, const uint64_t at[7]) {
+  char* p = static_cast<char*>(block);
+  return FindList{reinterpret_cast<uint64_t*>(p + at[0]), reinterpret_cast<uint8_t*>(p + at[1]),
+                  reinterpret_cast<uint8_t*>(p + at[2]),  reinterpret_cast<uint64_t*>(p + at[3]),
+                  reinterpret_cast<uint32_t*>(p + at[4]), reinterpret_cast<uint32_t*>(p + at[5])};
+}
+
+void* list_block_take(sr_session* s, uint64_t bytes, uint64_t* got) {
+  {
+    std::lock_guard<std::mutex> lk(s->pool_mu);
+    int pick = -1;
+    for (size_t i = 0; i < s->list_pool.size(); ++i)
+      if (s->list_pool[i].second >= bytes && s->list_pool[i].second <= 2 * bytes + (64ull << 20) &&
+          (pick < 0 || s->list_pool[i].second < s->list_pool[pick].second))
+        pick = static_cast<int>(i);
+    if (pick >= 0) {
+      void* p = s->list_pool[pick].first;
+      *got = s->list_pool[pick].second;
+      s->list_pool.erase(s->list_pool.begin() + pick);
+      return p;
+    }
+  }
+  void* p = nullptr;
+  *got = bytes + bytes / 8;  // so that lists a little larger later take this block
+  if (cudaMalloc(&p, *got) == cudaSuccess) return p;
+  cudaGetLastError();
+  *got = bytes;
+  std::vector<std::pair<void*, uint64_t>> kept;  // they may be what is in the way
+  {
+    std::lock_guard<std::mutex> lk(s->pool_mu);
+    kept.swap(s->list_pool);
+  }
+  for (auto& b : kept) cudaFree(b.first);
+  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
+void list_block_give(sr_session* s, void* p, uint64_t bytes) {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  if (dev != s->device) cudaSetDevice(s->device);
+  const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+  void* drop = idle ? nullptr : p;
+  if (idle) {
+    std::lock_guard<std::mutex> lk(s->pool_mu);
+    s->list_pool.emplace_back(p, bytes);
+    if (s->list_pool.size() > kKeptLists) {
+      drop = s->list_pool.front().first;
+      s->list_pool.erase(s->list_pool.begin());
+    }
+  }
+  if (drop) cudaFree(drop);
+  if (dev >= 0 && dev != s->device) cudaSetDevice(dev);
+}
+
+// The large-read path (sr_cal.cu) over n reads: their window list in the
+// session's cached arrays (out), *total windows.
+sr_status cal_large(CalCall& c, const char* d_bases, const uint64_t* d_roff, uint32_t n, FindList* out,
+                    uint64_t* total) {
+  sr_session* s = c.s;
+  const cudaStream_t st = c.st;
+  const sr_cand_params& cp = c.cp;
+  cudaError_t& e = c.e;
+  FindList L{};
+  uint64_t cap_out = 0, total_w = 0;
+  L.off = static_cast<uint64_t*>(c.buf(kCbLoff, (n + 1ull) * 8));
+  // grows the list's arrays to hold `need` windows, keeping the first `keep`
+  auto grow_out = [&](uint64_t need, uint64_t keep) -> bool {
+    if (need <= cap_out) return true;
+    const uint64_t cap = std::max<uint64_t>(need, cap_out + cap_out / 2);
+    L.ref = static_cast<uint8_t*>(c.grow(kCbLref, cap, keep));
+    L.strand = static_cast<uint8_t*>(c.grow(kCbLstr, cap, keep));
+    L.start = static_cast<uint64_t*>(c.grow(kCbLstart, cap * 8, keep * 8));
+    L.len = static_cast<uint32_t*>(c.grow(kCbLlen, cap * 4, keep * 4));
+    L.hits = static_cast<uint32_t*>(c.grow(kCbLhits, cap * 4, keep * 4));
+    if (e != cudaSuccess) return false;
+    cap_out = cap;
+    return true;
+  };
+  uint32_t* d_count = static_cast<uint32_t*>(c.buf(kCbCount, n * 4ull));
+  uint32_t* d_actual = static_cast<uint32_t*>(c.buf(kCbActual, n * 4ull));
+  uint32_t* d_status = static_cast<uint32_t*>(c.buf(kCbStatus, 4));
+  // per read: its lookup records (seeds x references), then their prefix sums
+  uint32_t* d_slots = static_cast<uint32_t*>(c.buf(kCbSlots, n * 4ull));
+  uint64_t* d_pre = static_cast<uint64_t*>(c.buf(kCbPre, (n + 1ull) * 8));
+  uint64_t* d_sums = static_cast<uint64_t*>(c.buf(kCbSums, (n / 1024 + 2ull) * 8));
+  uint32_t* d_bounds = static_cast<uint32_t*>(c.buf(kCbBounds, (n + 1ull) * 4));
+  CalPlan* d_plan = static_cast<CalPlan*>(c.buf(kCbPlan, sizeof(CalPlan)));
+  if (e != cudaSuccess) return c.no_memory();
+  // The count pass keeps each seed's lookup (one record per seed and
+  // reference) for the emit pass.  Reads run in chunks of at most
+  // kRangeRecords records: a chunk is cut where the records' prefix sum crosses
+  // a multiple of kRangeRecords less one read's most records, so that no chunk
+  // exceeds it; all cuts are made on the device.
+  const uint64_t rec_read = (static_cast<uint64_t>(kMaxReadLen) / cp.seed_stride + 1) * s->didx.n_refs;
+  // 1 GiB of kept lookups at most; SR_CAL_CHUNK_RECORDS lowers it (tests of the cuts)
+  const uint64_t kRangeRecords = std::max<uint64_t>(env_u64("SR_CAL_CHUNK_RECORDS", 128ull << 20), 2 * rec_read);
+  const uint64_t rec_span = kRangeRecords - rec_read;
+  uint64_t ends[2] = {};  // prefix of the last read, total records
+  uint32_t status = 0;
+  if (launch_cal_slots(d_roff, n, s->didx.k, cp.seed_stride, s->didx.n_refs, d_slots, d_status, st) < 0 ||
+      launch_scan_u64(d_slots, n, d_pre, d_sums, st) < 0 || launch_cal_bounds(d_pre, n, rec_span, d_bounds, st) < 0) {
+    e = cudaGetLastError();
+    return c.fail("sr_candidates_device slots");
+  }
+  e = cudaMemcpyAsync(ends, d_pre + n - 1, 16, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, d_status, 4, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return c.fail("sr_candidates_device slots copy");
+  if (status & kStBadRead) return set_error(SR_EINVAL, "sr_candidates_device: decreasing read offsets or a read longer than 256 bases");
+  const uint32_t n_chunks = static_cast<uint32_t>(ends[0] / rec_span) + 1;
+  std::vector<uint32_t> rchunk(n_chunks + 1ull);
+  e = cudaMemcpyAsync(rchunk.data(), d_bounds, n_chunks * 4ull, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return c.fail("sr_candidates_device chunks");
+  rchunk[n_chunks] = n;
+  uint32_t max_reads = 0;
+  uint64_t max_rec = 0;
+  for (uint32_t ci = 0; ci < n_chunks; ++ci) max_reads = std::max(max_reads, rchunk[ci + 1] - rchunk[ci]);
+  max_rec = std::min<uint64_t>(ends[1], kRangeRecords);
+  uint64_t* d_ranges = static_cast<uint64_t*>(c.buf(kCbRanges, std::max<uint64_t>(max_rec, 1) * 8));
+  uint32_t* d_seed_off = static_cast<uint32_t*>(c.buf(kCbSeedOff, (max_reads + 1ull) * 4));
+  uint8_t* d_recount = static_cast<uint8_t*>(c.buf(kCbRecount, max_reads + 1ull));
+  // per chunk: the prefix sums of its reads' CAL bounds, a sub-chunk's offsets
+  // (from 0) and its large-read list
+  uint64_t* d_cpre = static_cast<uint64_t*>(c.buf(kCbCpre, (max_reads + 1ull) * 8));
+  uint64_t* d_off = static_cast<uint64_t*>(c.buf(kCbOff, (max_reads + 1ull) * 8));
+  uint32_t* d_nwin = static_cast<uint32_t*>(c.buf(kCbNwin, max_reads * 4ull + 4));
+  uint32_t* d_woff = static_cast<uint32_t*>(c.buf(kCbWoff, (max_reads + 1ull) * 4));
+  uint32_t* d_wsums = static_cast<uint32_t*>(c.buf(kCbWsums, (max_reads / 1024 + 2ull) * 4));
+  uint32_t* d_big = static_cast<uint32_t*>(c.buf(kCbBig, max_reads * 4ull + 4));
+  uint64_t* d_bigoff = static_cast<uint64_t*>(c.buf(kCbBigOff, max_reads * 8ull + 8));
+  if (e != cudaSuccess) return c.no_memory();
+  // the emit / filter buffers, sized for the largest sub-chunk so far
+  uint64_t cap = 0;
+  uint64_t *d_cals = nullptr, *d_wkey = nullptr;
+  uint32_t *d_whits = nullptr, *d_wlen = nullptr;
+  uint64_t* d_scratch = nullptr;
+  uint64_t scratch_keys = 0;
+  std::vector<uint32_t> sub;
+  // one sub-chunk (reads r0 .. r0 + nr of the chunk at R0, offsets in d_off):
+  // routing, emit, filter, window offsets and the compacted windows
+  auto run_sub = [&](uint32_t r0, uint32_t nr, const CalRanges& kept) -> sr_status {
+    CalPlan plan{};
+    e = cudaMemsetAsync(d_plan, 0, sizeof(CalPlan), st);
+    if (e != cudaSuccess || launch_cal_route(d_count + r0, nr, d_big, d_bigoff, d_plan, st) < 0)
+      return c.fail("sr_candidates_device route");
+    e = cudaMemcpyAsync(&plan, d_plan, sizeof(CalPlan), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return c.fail("sr_candidates_device route copy");
+    const uint64_t scratch_need = plan.scratch + (plan.n_big ? cal_sort_words(plan.n_big, plan.scratch) : 0);
+    if (scratch_need > scratch_keys) {
+      d_scratch = static_cast<uint64_t*>(c.buf(kCbScratch, scratch_need * 8));
+      if (e != cudaSuccess) return c.no_memory();
+      scratch_keys = scratch_need;
+    }
+    if (cudaMemsetAsync(d_nwin, 0, nr * 4ull, st) != cudaSuccess ||
+        launch_cal_seeds(s->didx, d_bases, d_roff, r0, nr, cp.seed_stride, d_count + r0, d_off, d_cals, d_actual,
+                         d_status, kept, st) < 0 ||
+        launch_cal_emit_big(s->didx, d_roff, r0, nr, cp.seed_stride, d_count + r0, d_off, d_cals, kept, d_big,
+                            plan.n_big, d_scratch, plan.scratch, st) < 0 ||
+        launch_cal_filter(s->didx, d_roff, r0, nr, cp.merge_dist, cp.pad, cp.max_cands, d_count + r0, d_actual,
+                          d_off, d_cals, d_big, d_bigoff, plan.n_big, d_scratch, plan.scratch, d_nwin, d_wkey, d_whits, d_wlen, st) < 0 ||
+        launch_scan_u32(d_nwin, nr, d_woff, d_wsums, st) < 0) {
+      e = cudaGetLastError();
+      return c.fail("sr_candidates_device filter");
+    }
+    uint32_t nw32 = 0;
+    e = cudaMemcpyAsync(&nw32, d_woff + nr, 4, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return c.fail("sr_candidates_device window count");
+    const uint64_t nw = nw32;
+    // this sub-chunk's offsets in the whole list, its windows compacted
+    // straight into the list's arrays after the windows so far
+    if (launch_cal_offsets(d_woff, nr, total_w, L.off + r0, st) < 0) {
+      e = cudaGetLastError();
+      return c.fail("sr_candidates_device offsets");
+    }
+    if (!grow_out(total_w + nw, total_w)) return c.no_memory();
+    if (launch_cal_compact(nr, d_off, d_nwin, d_woff, d_wkey, d_whits, d_wlen, L.ref + total_w, L.strand + total_w,
+                           L.start + total_w, L.len + total_w, L.hits + total_w, st) < 0) {
+      e = cudaGetLastError();
+      return c.fail("sr_candidates_device compact");
+    }
+    total_w += nw;
+    return static_cast<sr_status>(SR_OK);
+  };
+  for (uint32_t ci = 0; ci < n_chunks; ++ci) {
+    const uint32_t R0 = rchunk[ci], R1 = rchunk[ci + 1], nrc = R1 - R0;
+    // this chunk's record offsets from 0, then its count pass (which keeps the lookups)
+    if (launch_cal_rebase(d_pre, R0, nrc, nullptr, d_seed_off, st) < 0) {
+      e = cudaGetLastError();
+      return c.fail("sr_candidates_device records");
+    }
+    const CalRanges kept{d_ranges, d_seed_off, d_recount, R0};
+    // the chunk's CAL bounds: their prefix sums and largest
+    CalPlan whole{};
+    uint64_t cends[2] = {};  // prefix of the last read, total
+    e = cudaMemsetAsync(d_plan, 0, sizeof(CalPlan), st);
+    if (e != cudaSuccess ||
+        launch_cal_seeds(s->didx, d_bases, d_roff, R0, nrc, cp.seed_stride, d_count + R0, nullptr, nullptr,
+                         nullptr, d_status, kept, st) < 0 ||
+        launch_scan_u64(d_count + R0, nrc, d_cpre, d_sums, st) < 0 ||
+        launch_cal_route(d_count + R0, nrc, nullptr, nullptr, d_plan, st) < 0) {
+      e = cudaGetLastError();
+      return c.fail("sr_candidates_device count");
+    }
+    e = cudaMemcpyAsync(cends, d_cpre + nrc - 1, 16, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&whole, d_plan, sizeof(CalPlan), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, d_status, 4, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return c.fail("sr_candidates_device count copy");
+    if (status & kStBadRead) return set_error(SR_EINVAL, "sr_candidates_device: decreasing read offsets or a read longer than 256 bases");
+    if (status & kStBadBase) return set_error(SR_EBADBASE, "sr_candidates_device: read has a non-ACGT base");
+    // sub-chunks of at most kCalChunkKeys CAL bounds (more only for a read that
+    // alone has more), cut where the prefix sum crosses multiples of that less
+    // the largest read's bound
+    // SR_CAL_CHUNK_KEYS lowers it (tests of the cuts)
+    const uint64_t kCalChunkKeys = std::max<uint64_t>(env_u64("SR_CAL_CHUNK_KEYS", 64ull << 20), 1);
+    const uint64_t one = whole.max_all;
+    const uint64_t want = std::max<uint64_t>(std::min<uint64_t>(std::max<uint64_t>(cends[1], 1), kCalChunkKeys), 2 * one);
+    if (want > cap) {
+      cap = want;
+      d_cals = static_cast<uint64_t*>(c.buf(kCbCals, cap * 8));
+      d_wkey = static_cast<uint64_t*>(c.buf(kCbWkey, cap * 8));
+      d_whits = static_cast<uint32_t*>(c.buf(kCbWhits, cap * 4));
+      d_wlen = static_cast<uint32_t*>(c.buf(kCbWlen, cap * 4));
+      if (e != cudaSuccess) return c.no_memory();
+    }
+    if (cends[1] <= cap) {
+      // the whole chunk in one sub-chunk: its prefix sums are its offsets
+      e = cudaMemcpyAsync(d_off, d_cpre, (nrc + 1ull) * 8, cudaMemcpyDeviceToDevice, st);
+      if (e != cudaSuccess) return c.fail("sr_candidates_device offsets");
+      const sr_status r = run_sub(R0, nrc, kept);
+      if (r != SR_OK) return r;
+      continue;
+    }
+    const uint64_t span = cap - one;
+    const uint32_t n_sub = static_cast<uint32_t>(cends[0] / span) + 1;
+    sub.assign(n_sub + 1ull, 0);
+    if (launch_cal_bounds(d_cpre, nrc, span, d_bounds, st) < 0) {
+      e = cudaGetLastError();
+      return c.fail("sr_candidates_device sub-chunks");
+    }
+    e = cudaMemcpyAsync(sub.data(), d_bounds, n_sub * 4ull, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return c.fail("sr_candidates_device sub-chunks");
+    sub[n_sub] = nrc;
+    for (uint32_t si = 0; si < n_sub; ++si) {
+      const uint32_t a0 = sub[si], a1 = sub[si + 1];
+      if (launch_cal_rebase(d_cpre, a0, a1 - a0, d_off, nullptr, st) < 0) {
+        e = cudaGetLastError();
+        return c.fail("sr_candidates_device offsets");
+      }
+      const sr_status r = run_sub(R0 + a0, a1 - a0, kept);
+      if (r != SR_OK) return r;
+    }
+  }
+  if (!grow_out(std::max<uint64_t>(total_w, 1), total_w)) return c.no_memory();
+  *out = L;
+  *total = total_w;
+  return SR_OK;
+}
+
+// the finder's buffers for ranges of at most nr reads
+struct FindBufs {
+  uint32_t *nwin, *wslot, *mid, *wide, *rest;
+  uint64_t *woff, *sums;
+  FindPlan* plan;
+};
+}  // namespace
+
+bool sr::device_list_free(sr_cand_list* l) {
+  {
+    std::lock_guard<std::mutex> lk(g_lists_mu);
+    if (!g_lists.erase(l)) return false;
+  }
+  auto* box = reinterpret_cast<DevListBox*>(l);
+  sr_session* s = box->s;
+  list_block_give(s, box->block, box->bytes);
+  free(box);
+  session_release(s);
+  return true;
+}
+
 extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, const sr_cand_params* params,
                                           sr_cand_list** out) {
   Trace trace_("sr_candidates_device");
@@ -1469,20 +1830,8 @@ extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, 
   const bool in_dev = (reads->flags & SR_FLAG_DEVICE) != 0, out_dev = (cp.flags & SR_FLAG_DEVICE) != 0;
   const uint32_t n = reads->n_reads;
   if (!reads->offsets || (n && !reads->bases)) return set_error(SR_EINVAL, "sr_candidates_device: null reads");
-  cudaStream_t st = s->stream;
   uint64_t nb = 0;
-  if (in_dev) {
-    // the read lengths are checked by the count kernel
-    uint64_t ends[2] = {};
-    cudaError_t e = cudaMemcpyAsync(&ends[0], reads->offsets, 8, cudaMemcpyDefault, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&ends[1], reads->offsets + n, 8, cudaMemcpyDefault, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_error("sr_candidates_device offsets", e);
-    if (ends[0] != 0) return set_error(SR_EINVAL, "sr_candidates_device: offsets must start at 0");
-    nb = ends[1];
-    if (nb > static_cast<uint64_t>(n) * SR_MAX_READ_LEN)
-      return set_error(SR_EINVAL, "sr_candidates_device: some read is longer than %u bases", SR_MAX_READ_LEN);
-  } else {
+  if (!in_dev) {  // device reads are checked by a kernel
     if (reads->offsets[0] != 0) return set_error(SR_EINVAL, "sr_candidates_device: offsets must start at 0");
     for (uint32_t r = 0; r < n; ++r) {
       if (reads->offsets[r + 1] < reads->offsets[r])
@@ -1492,351 +1841,209 @@ extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, 
     }
     nb = reads->offsets[n];
   }
-  // the call's scratch comes from the session's cache (grown with a quarter of
-  // headroom when a call needs more), so steady-state calls allocate only
-  // their result list
   std::lock_guard<std::mutex> cal_lock(s->cal_mu);
-  cudaError_t e = cudaSuccess;
-  auto cbuf = [&](int role, uint64_t bytes) -> void* {
-    if (e != cudaSuccess) return nullptr;
-    bytes = std::max<uint64_t>(bytes, 16);
-    if (s->cal_bytes[role] < bytes) {
-      if (s->cal_buf[role]) {
-        // earlier launches of this call may still use the smaller buffer
-        e = cudaStreamSynchronize(st);
-        cudaFree(s->cal_buf[role]);
-        s->cal_buf[role] = nullptr;
-        s->cal_bytes[role] = 0;
-        if (e != cudaSuccess) return nullptr;
-      }
-      const uint64_t want = bytes + bytes / 4;
-      e = cudaMalloc(&s->cal_buf[role], want);
-      if (e != cudaSuccess) {
-        s->cal_buf[role] = nullptr;
-        return nullptr;
-      }
-      s->cal_bytes[role] = want;
-    }
-    return s->cal_buf[role];
+  CalCall c{s, s->stream, cp};
+  const cudaStream_t st = c.st;
+  cudaError_t& e = c.e;
+  // what comes back per range of reads: its plan, window total and status
+  struct Back {
+    FindPlan plan;
+    uint64_t total;
+    uint32_t status;
   };
-  // The list is built on the device in either case: in the caller's list arrays
-  // (device output, grown chunk by chunk), or in the session's cached arrays
-  // (host output: copied out once at the end, through a pinned block).
-  sr_cand_list* l = static_cast<sr_cand_list*>(calloc(1, sizeof(sr_cand_list)));
-  if (!l) return set_error(SR_ENOMEM, "sr_candidates_device: out of memory");
-  l->n_reads = n;
-  l->flags = out_dev ? static_cast<uint32_t>(SR_FLAG_DEVICE) : 0u;
-  struct {
-    uint64_t* off;
-    uint8_t *ref, *str;
-    uint64_t* start;
-    uint32_t *len, *hits;
-  } L{};
-  uint64_t cap_out = 0;  // windows the device result arrays hold
-  auto done = [&](sr_status stt, const char* msg) -> sr_status {
+  if (!s->cal_back) {
+    if (cudaMallocHost(&s->cal_back, sizeof(Back)) != cudaSuccess) {
+      cudaGetLastError();
+      s->cal_back = nullptr;
+      return set_error(SR_ENOMEM, "sr_candidates_device: out of memory");
+    }
+  }
+  Back& back = *static_cast<Back*>(s->cal_back);
+  // the list's block: the caller's (device output) or the session's (host output)
+  void* block = nullptr;
+  uint64_t block_bytes = 0, cap = 0, total_w = 0;
+  uint64_t at[7] = {};
+  FindList L{};
+  auto done = [&](sr_status stt) -> sr_status {
     cudaStreamSynchronize(st);
     cudaGetLastError();
-    if (stt == SR_OK) return static_cast<sr_status>(SR_OK);
-    sr_cand_list_free(l);  // host output: its arrays are still unset
-    if (stt == SR_ECUDA) return cuda_error(msg, e == cudaSuccess ? cudaErrorUnknown : e);
-    return set_error(stt, "%s", msg);
+    if (out_dev && block) list_block_give(s, block, block_bytes);
+    return stt;
   };
-  if (out_dev) {
-    if (cudaMalloc(&l->offsets, (n + 1ull) * 8) != cudaSuccess) {
-      e = cudaGetLastError();
-      return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-    }
-    L.off = l->offsets;
-  } else {
-    L.off = static_cast<uint64_t*>(cbuf(kCbLoff, (n + 1ull) * 8));
-    if (e != cudaSuccess) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-  }
-  if (n == 0 && cudaMemsetAsync(L.off, 0, 8, st) != cudaSuccess) {
-    e = cudaGetLastError();
-    return done(SR_ECUDA, "sr_candidates_device offsets");
-  }
-  // a cached array grown to `need` bytes, its first `keep` bytes kept
-  auto cgrow = [&](int role, uint64_t need, uint64_t keep) -> void* {
-    if (s->cal_bytes[role] >= need) return s->cal_buf[role];
-    void* p = nullptr;
-    const uint64_t want = need + need / 4;
-    if (cudaMalloc(&p, want) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    if (keep && s->cal_buf[role] &&
-        cudaMemcpyAsync(p, s->cal_buf[role], keep, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-      cudaGetLastError();
-      cudaFree(p);
-      return nullptr;
-    }
-    cudaStreamSynchronize(st);
-    if (s->cal_buf[role]) cudaFree(s->cal_buf[role]);
-    s->cal_buf[role] = p;
-    s->cal_bytes[role] = want;
-    return p;
-  };
-  // grows the device result arrays to hold `need` windows, keeping the first `keep`
-  auto grow_out = [&](uint64_t need, uint64_t keep) -> bool {
-    if (need <= cap_out) return true;
-    const uint64_t c = std::max<uint64_t>(need, cap_out + cap_out / 2);
+  // room for `need` windows, the list so far kept
+  auto grow_out = [&](uint64_t need) -> bool {
+    if (block && need <= cap) return true;
+    const uint64_t ncap = std::max<uint64_t>(need, cap + cap / 2);
+    uint64_t nat[7], got = 0;
+    const uint64_t bytes = list_layout(n, ncap, nat);
+    void* nblock = out_dev ? list_block_take(s, bytes, &got) : nullptr;
     if (!out_dev) {
-      L.ref = static_cast<uint8_t*>(cgrow(kCbLref, c, keep));
-      L.str = static_cast<uint8_t*>(cgrow(kCbLstr, c, keep));
-      L.start = static_cast<uint64_t*>(cgrow(kCbLstart, c * 8, keep * 8));
-      L.len = static_cast<uint32_t*>(cgrow(kCbLlen, c * 4, keep * 4));
-      L.hits = static_cast<uint32_t*>(cgrow(kCbLhits, c * 4, keep * 4));
-      if (!L.ref || !L.str || !L.start || !L.len || !L.hits) return false;
-      cap_out = c;
-      return true;
+      // the buffers of the two growth steps alternate, so that the list can be moved
+      const int role = s->cal_buf[kCbList0] == block && block ? kCbList1 : kCbList0;
+      nblock = c.buf(role, bytes);
     }
-    void *r8 = nullptr, *s8 = nullptr, *st64 = nullptr, *ln32 = nullptr, *h32 = nullptr;
-    bool ok = cudaMalloc(&r8, c) == cudaSuccess && cudaMalloc(&s8, c) == cudaSuccess &&
-              cudaMalloc(&st64, c * 8) == cudaSuccess && cudaMalloc(&ln32, c * 4) == cudaSuccess &&
-              cudaMalloc(&h32, c * 4) == cudaSuccess;
-    if (ok && keep) {
-      ok = cudaMemcpyAsync(r8, l->ref_id, keep, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-           cudaMemcpyAsync(s8, l->strand, keep, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-           cudaMemcpyAsync(st64, l->win_start, keep * 8, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-           cudaMemcpyAsync(ln32, l->win_len, keep * 4, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-           cudaMemcpyAsync(h32, l->hits, keep * 4, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-           cudaStreamSynchronize(st) == cudaSuccess;
+    if (!nblock) return false;
+    const FindList N = list_arrays(nblock, nat);
+    if (block && total_w) {
+      const void* src[6] = {L.off, L.ref, L.strand, L.start, L.len, L.hits};
+      void* dst[6] = {N.off, N.ref, N.strand, N.start, N.len, N.hits};
+      const uint64_t len[6] = {(n + 1ull) * 8, total_w, total_w, total_w * 8, total_w * 4, total_w * 4};
+      for (int k = 0; k < 6 && e == cudaSuccess; ++k)
+        e = cudaMemcpyAsync(dst[k], src[k], len[k], cudaMemcpyDeviceToDevice, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    void* old[5] = {l->ref_id, l->strand, l->win_start, l->win_len, l->hits};
-    void* fresh[5] = {r8, s8, st64, ln32, h32};
-    if (!ok) {
-      for (void* p : fresh)
-        if (p) cudaFree(p);
-      cudaGetLastError();
-      return false;
-    }
-    for (void* p : old)
-      if (p) cudaFree(p);
-    l->ref_id = static_cast<uint8_t*>(r8);
-    l->strand = static_cast<uint8_t*>(s8);
-    l->win_start = static_cast<uint64_t*>(st64);
-    l->win_len = static_cast<uint32_t*>(ln32);
-    l->hits = static_cast<uint32_t*>(h32);
-    L.ref = l->ref_id;
-    L.str = l->strand;
-    L.start = l->win_start;
-    L.len = l->win_len;
-    L.hits = l->hits;
-    cap_out = c;
-    return true;
+    if (out_dev && block) list_block_give(s, block, block_bytes);
+    block = nblock;
+    block_bytes = got;
+    cap = ncap;
+    L = N;
+    memcpy(at, nat, sizeof(at));
+    return e == cudaSuccess;
   };
-  uint64_t total_w = 0;
-  if (n) {
-    const char* d_bases = in_dev ? reads->bases : static_cast<const char*>(cbuf(kCbBases, nb));
-    const uint64_t* d_roff = in_dev ? reads->offsets : static_cast<const uint64_t*>(cbuf(kCbRoff, (n + 1ull) * 8));
-    uint32_t* d_count = static_cast<uint32_t*>(cbuf(kCbCount, n * 4ull));
-    uint32_t* d_actual = static_cast<uint32_t*>(cbuf(kCbActual, n * 4ull));
-    uint32_t* d_status = static_cast<uint32_t*>(cbuf(kCbStatus, 4));
-    // per read: its lookup records (seeds x references), then their prefix sums
-    uint32_t* d_slots = static_cast<uint32_t*>(cbuf(kCbSlots, n * 4ull));
-    uint64_t* d_pre = static_cast<uint64_t*>(cbuf(kCbPre, (n + 1ull) * 8));
-    uint64_t* d_sums = static_cast<uint64_t*>(cbuf(kCbSums, (n / 1024 + 2ull) * 8));
-    uint32_t* d_bounds = static_cast<uint32_t*>(cbuf(kCbBounds, (n + 1ull) * 4));
-    CalPlan* d_plan = static_cast<CalPlan*>(cbuf(kCbPlan, sizeof(CalPlan)));
-    if (e != cudaSuccess) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
+  if (n == 0) {
+    uint64_t first = 0;
+    if (in_dev) e = cudaMemcpy(&first, reads->offsets, 8, cudaMemcpyDefault);
+    if (e != cudaSuccess) return done(c.fail("sr_candidates_device offsets"));
+    if (first) return done(set_error(SR_EINVAL, "sr_candidates_device: offsets must start at 0"));
+    if (!grow_out(1)) return done(c.no_memory());
+    e = cudaMemsetAsync(L.off, 0, 8, st);
+    if (e != cudaSuccess) return done(c.fail("sr_candidates_device offsets"));
+  } else {
+    const char* d_bases = in_dev ? reads->bases : static_cast<const char*>(c.buf(kCbBases, nb));
+    const uint64_t* d_roff = in_dev ? reads->offsets : static_cast<const uint64_t*>(c.buf(kCbRoff, (n + 1ull) * 8));
+    uint32_t* d_status = static_cast<uint32_t*>(c.buf(kCbStatus, 4));
+    FindBufs f{};
+    f.nwin = static_cast<uint32_t*>(c.buf(kCbFnwin, n * 4ull));
+    f.wslot = static_cast<uint32_t*>(c.buf(kCbFslot, n * 4ull));
+    f.mid = static_cast<uint32_t*>(c.buf(kCbFmid, n * 4ull));
+    f.wide = static_cast<uint32_t*>(c.buf(kCbFwide, n * 4ull));
+    f.rest = static_cast<uint32_t*>(c.buf(kCbFrest, n * 4ull));
+    f.woff = static_cast<uint64_t*>(c.buf(kCbFwoff, (n + 1ull) * 8));
+    f.sums = static_cast<uint64_t*>(c.buf(kCbFsums, (n / 1024 + 2ull) * 8));
+    f.plan = static_cast<FindPlan*>(c.buf(kCbFplan, sizeof(FindPlan)));
+    // staging slots: two windows a read and the warps' chunks to begin with; a
+    // range that needs more is run again with as many as it took, up to kStage
+    // (SR_CAL_CHUNK_KEYS lowers it for tests of the cuts), past which the range
+    // is halved
+    const uint64_t kStage = std::max<uint64_t>(std::min<uint64_t>(env_u64("SR_CAL_CHUNK_KEYS", 64ull << 20), 1ull << 31), 1);
+    c.buf(kCbWin, std::min<uint64_t>(2ull * n + 16ull * std::min<uint64_t>(n, 1u << 15), kStage) * sizeof(uint4));
+    if (e != cudaSuccess) return done(c.no_memory());
     if (!in_dev) {
       if (nb) e = cudaMemcpyAsync(const_cast<char*>(d_bases), reads->bases, nb, cudaMemcpyHostToDevice, st);
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(const_cast<uint64_t*>(d_roff), reads->offsets, (n + 1ull) * 8, cudaMemcpyHostToDevice, st);
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(d_status, 0, 4, st);
-    if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device copy");
-    // The count pass keeps each seed's lookup (one record per seed and
-    // reference) for the emit pass.  Reads run in chunks of at most
-    // kRangeRecords records: a chunk is cut where the records' prefix sum crosses
-    // a multiple of kRangeRecords less one read's most records, so that no chunk
-    // exceeds it; all cuts are made on the device.
-    const uint64_t rec_read = (static_cast<uint64_t>(kMaxReadLen) / cp.seed_stride + 1) * s->didx.n_refs;
-    // 1 GiB of kept lookups at most; SR_CAL_CHUNK_RECORDS lowers it (tests of the cuts)
-    const uint64_t kRangeRecords = std::max<uint64_t>(env_u64("SR_CAL_CHUNK_RECORDS", 128ull << 20), 2 * rec_read);
-    const uint64_t rec_span = kRangeRecords - rec_read;
-    uint64_t ends[2] = {};  // prefix of the last read, total records
-    uint32_t status = 0;
-    if (launch_cal_slots(d_roff, n, s->didx.k, cp.seed_stride, s->didx.n_refs, d_slots, d_status, st) < 0 ||
-        launch_scan_u64(d_slots, n, d_pre, d_sums, st) < 0 || launch_cal_bounds(d_pre, n, rec_span, d_bounds, st) < 0) {
-      e = cudaGetLastError();
-      return done(SR_ECUDA, "sr_candidates_device slots");
-    }
-    e = cudaMemcpyAsync(ends, d_pre + n - 1, 16, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, d_status, 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device slots copy");
-    if (status & kStBadRead) return done(SR_EINVAL, "sr_candidates_device: decreasing read offsets or a read longer than 256 bases");
-    const uint32_t n_chunks = static_cast<uint32_t>(ends[0] / rec_span) + 1;
-    std::vector<uint32_t> rchunk(n_chunks + 1ull);
-    e = cudaMemcpyAsync(rchunk.data(), d_bounds, n_chunks * 4ull, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device chunks");
-    rchunk[n_chunks] = n;
-    uint32_t max_reads = 0;
-    uint64_t max_rec = 0;
-    for (uint32_t c = 0; c < n_chunks; ++c) max_reads = std::max(max_reads, rchunk[c + 1] - rchunk[c]);
-    max_rec = std::min<uint64_t>(ends[1], kRangeRecords);
-    uint64_t* d_ranges = static_cast<uint64_t*>(cbuf(kCbRanges, std::max<uint64_t>(max_rec, 1) * 8));
-    uint32_t* d_seed_off = static_cast<uint32_t*>(cbuf(kCbSeedOff, (max_reads + 1ull) * 4));
-    uint8_t* d_recount = static_cast<uint8_t*>(cbuf(kCbRecount, max_reads + 1ull));
-    // per chunk: the prefix sums of its reads' CAL bounds, a sub-chunk's offsets
-    // (from 0) and its large-read list
-    uint64_t* d_cpre = static_cast<uint64_t*>(cbuf(kCbCpre, (max_reads + 1ull) * 8));
-    uint64_t* d_off = static_cast<uint64_t*>(cbuf(kCbOff, (max_reads + 1ull) * 8));
-    uint32_t* d_nwin = static_cast<uint32_t*>(cbuf(kCbNwin, max_reads * 4ull + 4));
-    uint32_t* d_woff = static_cast<uint32_t*>(cbuf(kCbWoff, (max_reads + 1ull) * 4));
-    uint32_t* d_wsums = static_cast<uint32_t*>(cbuf(kCbWsums, (max_reads / 1024 + 2ull) * 4));
-    uint32_t* d_big = static_cast<uint32_t*>(cbuf(kCbBig, max_reads * 4ull + 4));
-    uint64_t* d_bigoff = static_cast<uint64_t*>(cbuf(kCbBigOff, max_reads * 8ull + 8));
-    if (e != cudaSuccess) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-    // the emit / filter buffers, sized for the largest sub-chunk so far
-    uint64_t cap = 0;
-    uint64_t *d_cals = nullptr, *d_wkey = nullptr;
-    uint32_t *d_whits = nullptr, *d_wlen = nullptr;
-    uint64_t* d_scratch = nullptr;
-    uint64_t scratch_keys = 0;
-    std::vector<uint32_t> sub;
-    // one sub-chunk (reads r0 .. r0 + nr of the chunk at R0, offsets in d_off):
-    // routing, emit, filter, window offsets and the compacted windows
-    auto run_sub = [&](uint32_t r0, uint32_t nr, const CalRanges& kept) -> sr_status {
-      CalPlan plan{};
-      e = cudaMemsetAsync(d_plan, 0, sizeof(CalPlan), st);
-      if (e != cudaSuccess || launch_cal_route(d_count + r0, nr, d_big, d_bigoff, d_plan, st) < 0)
-        return done(SR_ECUDA, "sr_candidates_device route");
-      e = cudaMemcpyAsync(&plan, d_plan, sizeof(CalPlan), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && in_dev && launch_find_check(d_roff, n, d_status, st) < 0) e = cudaGetLastError();
+    if (e != cudaSuccess) return done(c.fail("sr_candidates_device copy"));
+    FindArgs a{s->didx, d_bases, d_roff, 0, 0, cp.seed_stride, cp.merge_dist, cp.pad, cp.max_cands,
+               static_cast<uint32_t>(std::min<uint64_t>(env_u64("SR_CAL_TABLE", 1u << 30), 1u << 30)), d_status, nullptr, 0,
+               f.nwin, f.wslot, f.mid, f.wide, f.rest, f.plan};
+    uint32_t span = n;
+    uint64_t slots = 0;  // slots a single read needs, past kStage
+    for (uint32_t r0 = 0; r0 < n;) {
+      const uint32_t nr = std::min(span, n - r0);
+      a.r0 = r0;
+      a.nr = nr;
+      a.win = static_cast<uint4*>(s->cal_buf[kCbWin]);
+      a.win_cap = std::min<uint64_t>(s->cal_bytes[kCbWin] / sizeof(uint4), std::max(kStage, slots));
+      e = cudaMemsetAsync(f.plan, 0, sizeof(FindPlan), st);
+      if (e == cudaSuccess && (launch_find(a, st) < 0 || launch_scan_u64(f.nwin, nr, f.woff, f.sums, st) < 0))
+        e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&back.plan, f.plan, sizeof(FindPlan), cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&back.total, f.woff + nr, 8, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&back.status, d_status, 4, cudaMemcpyDeviceToHost, st);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device route copy");
-      const uint64_t scratch_need = plan.scratch + (plan.n_big ? cal_sort_words(plan.n_big, plan.scratch) : 0);
-      if (scratch_need > scratch_keys) {
-        d_scratch = static_cast<uint64_t*>(cbuf(kCbScratch, scratch_need * 8));
-        if (e != cudaSuccess) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-        scratch_keys = scratch_need;
-      }
-      if (launch_cal_seeds(s->didx, d_bases, d_roff, r0, nr, cp.seed_stride, d_count + r0, d_off, d_cals, d_actual,
-                           d_status, kept, st) < 0 ||
-          launch_cal_emit_big(s->didx, d_roff, r0, nr, cp.seed_stride, d_count + r0, d_off, d_cals, kept, d_big,
-                              plan.n_big, d_scratch, plan.scratch, st) < 0 ||
-          launch_cal_filter(s->didx, d_roff, r0, nr, cp.merge_dist, cp.pad, cp.max_cands, d_count + r0, d_actual,
-                            d_off, d_cals, std::max(plan.max_small, 1u), plan.max_mid, d_big, d_bigoff, plan.n_big,
-                            d_scratch, plan.scratch, d_nwin, d_wkey, d_whits, d_wlen, st) < 0 ||
-          launch_scan_u32(d_nwin, nr, d_woff, d_wsums, st) < 0) {
-        e = cudaGetLastError();
-        return done(SR_ECUDA, "sr_candidates_device filter");
-      }
-      uint32_t nw32 = 0;
-      e = cudaMemcpyAsync(&nw32, d_woff + nr, 4, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device window count");
-      const uint64_t nw = nw32;
-      // this sub-chunk's offsets in the whole list, its windows compacted
-      // straight into the list's arrays after the windows so far
-      if (launch_cal_offsets(d_woff, nr, total_w, L.off + r0, st) < 0) {
-        e = cudaGetLastError();
-        return done(SR_ECUDA, "sr_candidates_device offsets");
-      }
-      if (!grow_out(total_w + nw, total_w)) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-      if (launch_cal_compact(nr, d_off, d_nwin, d_woff, d_wkey, d_whits, d_wlen, L.ref + total_w, L.str + total_w,
-                             L.start + total_w, L.len + total_w, L.hits + total_w, st) < 0) {
-        e = cudaGetLastError();
-        return done(SR_ECUDA, "sr_candidates_device compact");
-      }
-      total_w += nw;
-      return static_cast<sr_status>(SR_OK);
-    };
-    for (uint32_t ci = 0; ci < n_chunks; ++ci) {
-      const uint32_t R0 = rchunk[ci], R1 = rchunk[ci + 1], nrc = R1 - R0;
-      // this chunk's record offsets from 0, then its count pass (which keeps the lookups)
-      if (launch_cal_rebase(d_pre, R0, nrc, nullptr, d_seed_off, st) < 0) {
-        e = cudaGetLastError();
-        return done(SR_ECUDA, "sr_candidates_device records");
-      }
-      const CalRanges kept{d_ranges, d_seed_off, d_recount, R0};
-      // the chunk's CAL bounds: their prefix sums and largest
-      CalPlan whole{};
-      uint64_t cends[2] = {};  // prefix of the last read, total
-      e = cudaMemsetAsync(d_plan, 0, sizeof(CalPlan), st);
-      if (e != cudaSuccess ||
-          launch_cal_seeds(s->didx, d_bases, d_roff, R0, nrc, cp.seed_stride, d_count + R0, nullptr, nullptr,
-                           nullptr, d_status, kept, st) < 0 ||
-          launch_scan_u64(d_count + R0, nrc, d_cpre, d_sums, st) < 0 ||
-          launch_cal_route(d_count + R0, nrc, nullptr, nullptr, d_plan, st) < 0) {
-        e = cudaGetLastError();
-        return done(SR_ECUDA, "sr_candidates_device count");
-      }
-      e = cudaMemcpyAsync(cends, d_cpre + nrc - 1, 16, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(&whole, d_plan, sizeof(CalPlan), cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(&status, d_status, 4, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device count copy");
-      if (status & kStBadRead) return done(SR_EINVAL, "sr_candidates_device: decreasing read offsets or a read longer than 256 bases");
-      if (status & kStBadBase) return done(SR_EBADBASE, "sr_candidates_device: read has a non-ACGT base");
-      // sub-chunks of at most kCalChunkKeys CAL bounds (more only for a read that
-      // alone has more), cut where the prefix sum crosses multiples of that less
-      // the largest read's bound
-      // SR_CAL_CHUNK_KEYS lowers it (tests of the cuts)
-      const uint64_t kCalChunkKeys = std::max<uint64_t>(env_u64("SR_CAL_CHUNK_KEYS", 64ull << 20), 1);
-      const uint64_t one = whole.max_all;
-      const uint64_t want = std::max<uint64_t>(std::min<uint64_t>(std::max<uint64_t>(cends[1], 1), kCalChunkKeys), 2 * one);
-      if (want > cap) {
-        cap = want;
-        d_cals = static_cast<uint64_t*>(cbuf(kCbCals, cap * 8));
-        d_wkey = static_cast<uint64_t*>(cbuf(kCbWkey, cap * 8));
-        d_whits = static_cast<uint32_t*>(cbuf(kCbWhits, cap * 4));
-        d_wlen = static_cast<uint32_t*>(cbuf(kCbWlen, cap * 4));
-        if (e != cudaSuccess) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-      }
-      if (cends[1] <= cap) {
-        // the whole chunk in one sub-chunk: its prefix sums are its offsets
-        e = cudaMemcpyAsync(d_off, d_cpre, (nrc + 1ull) * 8, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device offsets");
-        const sr_status r = run_sub(R0, nrc, kept);
-        if (r != SR_OK) return r;
+      if (e != cudaSuccess) return done(c.fail("sr_candidates_device find"));
+      if (back.status & kStBadStart) return done(set_error(SR_EINVAL, "sr_candidates_device: offsets must start at 0"));
+      if (back.status & kStBadRead)
+        return done(set_error(SR_EINVAL, "sr_candidates_device: decreasing read offsets or a read longer than %u bases",
+                              SR_MAX_READ_LEN));
+      if (back.status & kStBadBase)
+        return done(set_error(SR_EBADBASE, "sr_candidates_device: read has a non-ACGT base"));
+      const FindPlan plan = back.plan;
+      if (plan.cursor > a.win_cap) {
+        if (plan.cursor > kStage && nr > 1) {
+          span = (nr + 1) / 2;
+        } else {
+          slots = plan.cursor;
+          c.buf(kCbWin, plan.cursor * sizeof(uint4));
+          if (e != cudaSuccess) return done(c.no_memory());
+        }
         continue;
       }
-      const uint64_t span = cap - one;
-      const uint32_t n_sub = static_cast<uint32_t>(cends[0] / span) + 1;
-      sub.assign(n_sub + 1ull, 0);
-      if (launch_cal_bounds(d_cpre, nrc, span, d_bounds, st) < 0) {
-        e = cudaGetLastError();
-        return done(SR_ECUDA, "sr_candidates_device sub-chunks");
-      }
-      e = cudaMemcpyAsync(sub.data(), d_bounds, n_sub * 4ull, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device sub-chunks");
-      sub[n_sub] = nrc;
-      for (uint32_t si = 0; si < n_sub; ++si) {
-        const uint32_t a0 = sub[si], a1 = sub[si + 1];
-        if (launch_cal_rebase(d_cpre, a0, a1 - a0, d_off, nullptr, st) < 0) {
-          e = cudaGetLastError();
-          return done(SR_ECUDA, "sr_candidates_device offsets");
+      uint64_t nw = back.total;
+      if (plan.n_rest) {
+        // the reads of more distinct CALs than the tables take, as a batch of
+        // their own through the large-read path, their windows then staged too
+        const uint32_t nl = plan.n_rest;
+        uint32_t* len = static_cast<uint32_t*>(c.buf(kCbRlen, nl * 4ull));
+        uint64_t* off = static_cast<uint64_t*>(c.buf(kCbRoff2, (nl + 1ull) * 8));
+        char* bases = static_cast<char*>(c.buf(kCbRbases, static_cast<uint64_t>(nl) * kMaxReadLen));
+        if (e != cudaSuccess) return done(c.no_memory());
+        if (launch_rest_gather(d_bases, d_roff, r0, f.rest, nl, len, off, f.sums, bases, st) < 0)
+          return done(c.fail("sr_candidates_device gather"));
+        FindList R{};
+        uint64_t wr = 0;
+        const sr_status ls = cal_large(c, bases, off, nl, &R, &wr);
+        if (ls != SR_OK) return done(ls);
+        if (plan.cursor + wr >= (1ull << 32)) {
+          if (nr == 1) return done(c.no_memory());
+          span = (nr + 1) / 2;
+          continue;
         }
-        const sr_status r = run_sub(R0 + a0, a1 - a0, kept);
-        if (r != SR_OK) return r;
+        uint4* win = static_cast<uint4*>(c.grow(kCbWin, (plan.cursor + wr) * sizeof(uint4), plan.cursor * sizeof(uint4)));
+        if (e != cudaSuccess) return done(c.no_memory());
+        a.win = win;
+        if (launch_rest_stage(R, f.rest, nl, plan.cursor, win, f.nwin, f.wslot, st) < 0 ||
+            launch_scan_u64(f.nwin, nr, f.woff, f.sums, st) < 0)
+          return done(c.fail("sr_candidates_device large reads"));
+        nw += wr;
       }
+      if (!grow_out(std::max<uint64_t>(total_w + nw, 1))) return done(c.no_memory());
+      FindList dst = L;
+      dst.off += r0;
+      if (launch_find_out(f.woff, nr, nw, f.wslot, a.win, total_w, dst, st) < 0)
+        return done(c.fail("sr_candidates_device list"));
+      total_w += nw;
+      r0 += nr;
     }
-    // the device result arrays must be complete before the call returns
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return done(SR_ECUDA, "sr_candidates_device");
   }
-  l->n_cands = total_w;
   if (out_dev) {
-    if (!grow_out(std::max<uint64_t>(total_w, 1), total_w)) return done(SR_ENOMEM, "sr_candidates_device: device allocation failed");
-    sr_status stt = done(SR_OK, "");
-    if (stt != SR_OK) return stt;
-    *out = l;
+    // the list must be complete before the call returns
+    e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return done(c.fail("sr_candidates_device"));
+    auto* box = static_cast<DevListBox*>(calloc(1, sizeof(DevListBox)));
+    if (!box) return done(set_error(SR_ENOMEM, "sr_candidates_device: out of memory"));
+    box->s = s;
+    box->block = block;
+    box->bytes = block_bytes;
+    sr_cand_list& l = box->pub;
+    l.n_reads = n;
+    l.flags = static_cast<uint32_t>(SR_FLAG_DEVICE);
+    l.n_cands = total_w;
+    l.offsets = L.off;
+    l.ref_id = L.ref;
+    l.strand = L.strand;
+    l.win_start = L.start;
+    l.win_len = L.len;
+    l.hits = L.hits;
+    s->live.fetch_add(1);  // a list keeps its session alive
+    {
+      std::lock_guard<std::mutex> lk(g_lists_mu);
+      g_lists.insert(box);
+    }
+    *out = &box->pub;
     return SR_OK;
   }
   // host output: the device list copied out through one pinned block, then
   // spread over the host threads into the list's own arrays
   sr_cand_list* h = nullptr;
   const sr_status sa = sr_cand_list_alloc(n, total_w, &h);
-  if (sa != SR_OK) return done(sa, "sr_candidates_device: out of memory");
+  if (sa != SR_OK) return done(set_error(sa, "sr_candidates_device: out of memory"));
   const uint64_t part_bytes[6] = {(n + 1ull) * 8, total_w, total_w, total_w * 8, total_w * 4, total_w * 4};
-  const void* src[6] = {L.off, L.ref, L.str, L.start, L.len, L.hits};
+  const void* src[6] = {L.off, L.ref, L.strand, L.start, L.len, L.hits};
   void* dst[6] = {h->offsets, h->ref_id, h->strand, h->win_start, h->win_len, h->hits};
-  uint64_t at[7] = {0};
-  for (int k = 0; k < 6; ++k) at[k + 1] = (at[k] + part_bytes[k] + 255) & ~255ull;
   uint64_t got = 0;
   char* blk = static_cast<char*>(pool_take(s, at[6], &got));
   if (!blk) {
@@ -1846,41 +2053,37 @@ extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, 
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
       sr_cand_list_free(h);
-      return done(SR_ECUDA, "sr_candidates_device list copy");
-    }
-    const sr_status stt = done(SR_OK, "");
-    sr_cand_list_free(l);
-    if (stt != SR_OK) {
-      sr_cand_list_free(h);
-      return stt;
+      return done(c.fail("sr_candidates_device list copy"));
     }
     *out = h;
     return SR_OK;
   }
-  for (int k = 0; k < 6 && e == cudaSuccess; ++k)
-    if (part_bytes[k]) e = cudaMemcpyAsync(blk + at[k], src[k], part_bytes[k], cudaMemcpyDeviceToHost, st);
+  if (total_w == cap || at[6] <= (1ull << 20)) {
+    e = cudaMemcpyAsync(blk, block, at[6], cudaMemcpyDeviceToHost, st);  // the arrays as they lie, in one copy
+  } else {
+    for (int k = 0; k < 6 && e == cudaSuccess; ++k)
+      if (part_bytes[k]) e = cudaMemcpyAsync(blk + at[k], src[k], part_bytes[k], cudaMemcpyDeviceToHost, st);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     pool_give(s, blk, got);
     sr_cand_list_free(h);
-    return done(SR_ECUDA, "sr_candidates_device list copy");
+    return done(c.fail("sr_candidates_device list copy"));
   }
-  constexpr uint64_t kSlice = 4ull << 20;  // bytes per host copy task
-  std::vector<std::pair<int, uint64_t>> tasks;
-  for (int k = 0; k < 6; ++k)
-    for (uint64_t o = 0; o < part_bytes[k]; o += kSlice) tasks.emplace_back(k, o);
-  parallel_for(static_cast<uint32_t>(tasks.size()), [&](uint32_t t) {
-    const int k = tasks[t].first;
-    const uint64_t o = tasks[t].second, len = std::min(kSlice, part_bytes[k] - o);
-    std::memcpy(static_cast<char*>(dst[k]) + o, blk + at[k] + o, len);
-  });
+  if (at[6] <= (1ull << 20)) {
+    for (int k = 0; k < 6; ++k) std::memcpy(dst[k], blk + at[k], part_bytes[k]);
+  } else {
+    constexpr uint64_t kSlice = 4ull << 20;  // bytes per host copy task
+    std::vector<std::pair<int, uint64_t>> tasks;
+    for (int k = 0; k < 6; ++k)
+      for (uint64_t o = 0; o < part_bytes[k]; o += kSlice) tasks.emplace_back(k, o);
+    parallel_for(static_cast<uint32_t>(tasks.size()), [&](uint32_t t) {
+      const int k = tasks[t].first;
+      const uint64_t o = tasks[t].second, len = std::min(kSlice, part_bytes[k] - o);
+      std::memcpy(static_cast<char*>(dst[k]) + o, blk + at[k] + o, len);
+    });
+  }
   pool_give(s, blk, got);
-  const sr_status stt = done(SR_OK, "");
-  sr_cand_list_free(l);
-  if (stt != SR_OK) {
-    sr_cand_list_free(h);
-    return stt;
-  }
   *out = h;
   return SR_OK;
 }
