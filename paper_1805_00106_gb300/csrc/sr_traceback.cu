@@ -4,10 +4,11 @@
 //
 // Most winners are traced by a banded DP that also finds the end row i*: two
 // reads per thread in the 16-bit halves of each value, swept row by row, for
-// bands of at most 16 diagonals (k_tb_pair<16>) and of 17-32 (k_tb_pair<32>);
-// when the scores do not fit those 16-bit values, one thread per read for at
-// most 8 diagonals (k_tb_thread) and a wavefront over the band's diagonals for
-// 9-32 (k_tb_wave); two diagonals per lane for 33-64 (k_tb_wave2).  Winners
+// bands of at most 16 diagonals (k_tb_pair<16>) and of 17-32 (k_tb_pair<32>),
+// or, where a class has too few reads to fill the chip that way, a wavefront
+// over the band's diagonals (k_tb_wave); when the scores do not fit the 16-bit
+// values, one thread per read for at most 8 diagonals (k_tb_thread) and the
+// wavefront for 9-32; two diagonals per lane for 33-64 (k_tb_wave2).  Winners
 // whose band is wider than 64 diagonals, and int32-class winners, use
 // k_traceback: one warp
 // per read recomputes the DP of the winning window in exact int32 over rows
@@ -524,9 +525,20 @@ __device__ __forceinline__ void tb_stage_bytes(const TbArgs& a, const TbRead& x,
     qc[i] = static_cast<uint8_t>(x.strand ? 3u - base_at(row, x.m - 1u - i) : base_at(row, i));
 }
 
+// Which kernel traces a band class: k_tb_pair does the least work per read, but
+// its thread sweeps a read's cells one after another (17-32 diagonals: 0.30 ms
+// however few reads, 1-16: 0.17-0.20 ms), so it pays once reads fill the chip;
+// the wavefront's 2 rows + band steps take 0.03 ms.  Traceback phase by counts of
+// reads in the class, pair then wavefront: 17-32 diagonals, 60 reads of a
+// 2049-read batch 349 / 240 us, 5000 of 150k 651 / 651, 17,000 of 480k 1418 /
+// 1903; 1-16 diagonals, 9 reads 200 / 87 us, 2049-read batch 240 / 123, 20,000-read
+// batch 279 / 211, 40,000 931 / 903, 150k 651 / 956.
+constexpr uint32_t kTbWave32Reads = 4096;
+constexpr uint32_t kTbWave16Reads = 16384;
+
 template <int SEG>
-__global__ void __launch_bounds__(32 * kTbWarps) k_tb_wave(TbArgs a, const uint32_t* list,
-                                                           const uint32_t* range) {
+__global__ void __launch_bounds__(32 * kTbWarps) k_tb_wave(TbArgs a, const uint32_t* list, const uint32_t* range_lo,
+                                                           const uint32_t* range_hi, uint32_t most) {
   static_assert(SEG >= 8, "narrow bands run one thread per read (k_tb_thread)");
   constexpr int NSEG = 32 / SEG;
   constexpr int kQB = kMaxReadLen;  // byte codes per read
@@ -545,8 +557,9 @@ __global__ void __launch_bounds__(32 * kTbWarps) k_tb_wave(TbArgs a, const uint3
   uint8_t* dirs = dirs_s[warp][seg] + kTbRowPad * SEG;
   const Codes cd{qbyte_s, rbyte_s};
   const int32_t goe = a.go + a.ge;
-  const uint32_t begin = range[0];
-  const uint32_t count = range[1] - begin;
+  const uint32_t begin = range_lo[0];
+  const uint32_t count = range_hi[1] - begin;
+  if (count > most) return;  // the two-reads-per-thread kernel's
   constexpr uint32_t kPerWarp = 2 * NSEG;
   const uint32_t stride = gridDim.x * kTbWarps * kPerWarp;
   // slot of read X of this segment, and its code offsets
@@ -1263,7 +1276,7 @@ __device__ __forceinline__ void tb_pair_reads(const TbArgs& a, const TbRead (&t)
 template <int MAXW>
 __global__ void __launch_bounds__(32 * kTbPWarps) k_tb_pair(TbArgs a, const uint32_t* list, const uint32_t* range_lo,
                                                           const uint32_t* range_hi, uint32_t* scratch,
-                                                          uint32_t n_warps) {
+                                                          uint32_t n_warps, uint32_t least) {
   constexpr int RW = tbp_rwords<MAXW>();
   constexpr int LANE = tbp_lane<MAXW>();
   __shared__ uint32_t s_s[kTbPWarps][32 * LANE];
@@ -1288,6 +1301,7 @@ __global__ void __launch_bounds__(32 * kTbPWarps) k_tb_pair(TbArgs a, const uint
   c.KN[2] = a.k2 << 11;
   const uint32_t first = range_lo[0];
   const uint32_t count = range_hi[1] - first;
+  if (count < least) return;  // the wavefront's
   for (uint32_t base = gw * 64u; base < count; base += n_warps * 64u) {
     TbRead t[2];
 #pragma unroll
@@ -1483,14 +1497,18 @@ int launch_traceback(const BatchDev& b, const DevRefs& refs, const ScoreConst& s
   int next = 0;
   const int width = fan_width(b.n_reads);
   auto lane_of = [&]() { return fan ? fan->side[next++ % width] : st; };
-  auto wave = [&](auto kern, int bucket, int per_warp) -> bool {
+  auto waves = [&](auto kern, int per_warp, auto... args) -> bool {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTbWarps, 0) != cudaSuccess) return false;
     const uint32_t g0 = static_cast<uint32_t>(nsm) * static_cast<uint32_t>(per_sm > 0 ? per_sm : 1);
     const uint32_t need = (b.n_reads + kTbWarps * per_warp - 1) / (kTbWarps * per_warp);
-    kern<<<need < g0 ? need : g0, 32 * kTbWarps, 0, lane_of()>>>(a, list, ranges + 2 * bucket);
+    kern<<<need < g0 ? need : g0, 32 * kTbWarps, 0, lane_of()>>>(a, list, args...);
     ++launched;
     return cudaPeekAtLastError() == cudaSuccess;
+  };
+  // wavefront over the reads of buckets b0 .. b1, when there are at most `most`
+  auto wave = [&](auto kern, int b0, int b1, int per_warp, uint32_t most) -> bool {
+    return waves(kern, per_warp, ranges + 2 * b0, ranges + 2 * b1, most);
   };
   // bands of at most 8 diagonals (buckets 0-3, adjacent in the sorted list): one
   // thread per read, one launch
@@ -1506,25 +1524,34 @@ int launch_traceback(const BatchDev& b, const DevRefs& refs, const ScoreConst& s
   // bands of at most 16 diagonals (buckets 0-4) and of 17-32 (bucket 5) with
   // packed scores: two reads per thread, one launch each, each with a scratch of
   // its own
-  auto pairs = [&](auto kern, int b0, int b1, uint32_t nw_max, uint32_t* scratch) -> bool {
+  auto pairs = [&](auto kern, int b0, int b1, uint32_t nw_max, uint32_t* scratch, uint32_t least) -> bool {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTbPWarps, 0) != cudaSuccess)
       return false;
     const uint32_t cap = static_cast<uint32_t>(nsm) * static_cast<uint32_t>(per_sm > 0 ? per_sm : 1) * kTbPWarps;
     const uint32_t nw = std::min(nw_max, cap);  // within the carved scratch
     kern<<<(nw + kTbPWarps - 1) / kTbPWarps, 32 * kTbPWarps, 0, lane_of()>>>(a, list, ranges + 2 * b0,
-                                                                          ranges + 2 * b1, scratch, nw);
+                                                                          ranges + 2 * b1, scratch, nw, least);
     ++launched;
     return cudaPeekAtLastError() == cudaSuccess;
   };
   // widest bands (longest kernels) first
   const bool pair = tb_pair_fits(a.sa, a.sb, a.go, a.ge);
-  if (!wave(k_tb_wave2, 6, 2) ||
-      !(pair ? pairs(k_tb_pair<32>, 5, 5, tb_pair32_warps(b.n_reads), b.tb_dirs32)
-             : wave(k_tb_wave<32>, 5, 2)) ||
-      !(pair ? pairs(k_tb_pair<16>, 0, 4, tb_pair_warps(b.n_reads), b.tb_dirs)
-             : (wave(k_tb_wave<16>, 4, 4) && threads())))
+  const uint32_t all = 0xffffffffu;
+  if (!waves(k_tb_wave2, 2, ranges + 2 * 6)) return -1;
+  if (pair) {
+    // few reads: the wavefront; many: two reads per thread.  The counts are on the
+    // device, so both are launched where either may be meant, and one returns
+    if (!wave(k_tb_wave<32>, 5, 5, 2, kTbWave32Reads) || !wave(k_tb_wave<16>, 0, 4, 4, kTbWave16Reads)) return -1;
+    if (b.n_reads > kTbWave32Reads &&
+        !pairs(k_tb_pair<32>, 5, 5, tb_pair32_warps(b.n_reads), b.tb_dirs32, kTbWave32Reads + 1))
+      return -1;
+    if (b.n_reads > kTbWave16Reads &&
+        !pairs(k_tb_pair<16>, 0, 4, tb_pair_warps(b.n_reads), b.tb_dirs, kTbWave16Reads + 1))
+      return -1;
+  } else if (!wave(k_tb_wave<32>, 5, 5, 2, all) || !wave(k_tb_wave<16>, 4, 4, 4, all) || !threads()) {
     return -1;
+  }
   const size_t smem = static_cast<size_t>(kMaxWinLen) * 32 * sizeof(uint32_t);
   static bool attr = false;
   if (!attr) {
