@@ -96,36 +96,64 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
     a.order = nullptr;
     a.cls = 0;
     uint32_t g = lanes ? lanes : 16, r = rows ? rows : 16;
-    uint64_t tasks = (b.n_items + 1) / 2;
+    const uint64_t tasks = (b.n_items + 1) / 2;
     int k = mode == 1 ? dispatch_mode1(false, g, r, a, st, tasks)
                       : dispatch_mode0(false, g, r, a, st, tasks);
     return k < 0 ? -1 : k;
   }
-  if (fan && fanout_begin(*fan, st) < 0) return -1;
-  int next = 0;
-  const int width = fan_width(b.n_reads);
-  // longest reads first: each side stream starts on a large bin
-  for (int c = n_bins - 1; c >= 0; --c) {
-    if (class_items && class_items[c] == 0) continue;
-    a.cls = c;
-    uint32_t g = lanes ? lanes : bins[c].lanes, r = rows ? rows : bins[c].rows;
-    const cudaStream_t s = fan ? fan->side[next++ % width] : st;
-    int k = mode == 1 ? dispatch_mode1(true, g, r, a, s, 0) : dispatch_mode0(true, g, r, a, s, 0);
+  // Few pairs: all classes in one launch (extension phase, us, one kernel per
+  // class / one launch on 16 lanes / on 32).  Reads of 75-250 bases in 23 classes:
+  // 270 pairs 217 / 76 / 48, 3000 218 / 131 / 119, 6000 218 / 205 / 162, 12,000
+  // 281 / 264 / 258, 24,000 410 / 422 / 469, 48,000 702 / 780 / 895; of 100 bases
+  // in one class: 3000 pairs 45 / 43 / 47, 6000 59 / 61 / 78, 24,000 162 / 194 /
+  // 264.  So one launch up to 12k pairs; on 32 lanes up to 8k pairs, or 2k of reads
+  // that 32 lanes x 4 rows (128) pad.
+  // Score sets whose biased scores may be negative (!ext_nonneg) always take it:
+  // their form of the recurrence is built for it alone.
+  uint64_t pairs = 0;
+  uint32_t upper[kNumBins], longest = 0;
+  for (int c = 0; c < n_bins; ++c) {
+    upper[c] = bins[c].upper;
+    pairs += (class_items[c] + 1) / 2;
+    if (class_items[c]) longest = upper[c];
+  }
+  const bool one = !ext_nonneg(a) || (!lanes && pairs <= 12288);
+  cudaStream_t s32 = st;  // the int32 class's stream
+  if (one) {
+    const uint32_t g = pairs <= (longest > 128 ? 8192u : 2048u) ? 32 : 16;
+    const int k = pairs == 0  ? 0
+                  : mode == 1 ? dispatch_all1(g, a, upper, pairs, st)
+                              : dispatch_all0(g, a, upper, pairs, st);
     if (k < 0) return -1;
     launched += k;
+  } else {
+    if (fan && fanout_begin(*fan, st) < 0) return -1;
+    int next = 0;
+    const int width = fan_width(b.n_reads);
+    // longest reads first: each side stream starts on a large bin
+    for (int c = n_bins - 1; c >= 0; --c) {
+      if (class_items[c] == 0) continue;
+      a.cls = c;
+      const uint32_t g = lanes ? lanes : bins[c].lanes, r = rows ? rows : bins[c].rows;
+      const cudaStream_t s = fan ? fan->side[next++ % width] : st;
+      const uint64_t tasks = (class_items[c] + 1) / 2;
+      const int k = mode == 1 ? dispatch_mode1(true, g, r, a, s, tasks) : dispatch_mode0(true, g, r, a, s, tasks);
+      if (k < 0) return -1;
+      launched += k;
+    }
+    if (fan) s32 = fan->side[next % width];
   }
-  a.cls = kI32Class;
-  if (!class_items || class_items[kI32Class] != 0) {
+  if (class_items[kI32Class] != 0) {
+    a.cls = kI32Class;
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const cudaStream_t s = fan ? fan->side[next++ % width] : st;
-    if (mode == 1) k_extend32<1><<<nsm * 4, 128, 0, s>>>(a);
-    else k_extend32<0><<<nsm * 4, 128, 0, s>>>(a);
+    if (mode == 1) k_extend32<1><<<nsm * 4, 128, 0, s32>>>(a);
+    else k_extend32<0><<<nsm * 4, 128, 0, s32>>>(a);
     if (cudaPeekAtLastError() != cudaSuccess) return -1;
     ++launched;
   }
-  if (fan && fanout_end(*fan, st) < 0) return -1;
+  if (!one && fan && fanout_end(*fan, st) < 0) return -1;
   return launched;
 }
 

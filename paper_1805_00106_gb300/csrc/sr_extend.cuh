@@ -14,12 +14,23 @@
 //   H(i,j) = max(0, H(i-1,j-1) + s(q_i, r_j), E(i,j), F(i,j))
 //
 // Values are stored as T = H - (go+ge) plus a bias of kBias, so every half
-// stays positive (the subtraction is a plain 32-bit add without cross-half
-// borrow, which issues at full rate beside the half-rate DPX and PRMT) and the
-// zero floor of H becomes a max with the bias.  The
-// substitution score s + (go+ge) comes from a per-row 8-byte table held in two
-// registers and is picked with one byte permute (prmt.b32) whose selector encodes
-// the two items' window bases at column j (sign-extended int8 -> int16).
+// stays positive: a plain 32-bit add or subtraction then neither carries nor
+// borrows across the halves.  The substitution score s + (go+ge) comes from a
+// per-row 8-byte table held in two registers and is picked with one byte permute
+// (prmt.b32) whose selector encodes the two items' window bases at column j
+// (sign-extended int8 -> int16).
+//
+// The ALU pipe bounds it: the permute and every DPX instruction take two of its
+// cycles per warp, so what can be a plain add is one, on the FMA pipe or beside
+// it.  While s + (go+ge) >= 0 (mismatch <= go + ge, any usual score set) the
+// diagonal term is T + sc, a plain add, so that H = max3(diagonal, E, F) is one
+// DPX instruction; the zero floor goes into E = max3(E - ge, T, 0) (an E below 0
+// is never taken by H, so flooring it changes nothing), and the subtractions of
+// E and T are multiply-adds by 1.  Per row: one permute, three DPX, three adds,
+// where add-max for E and for the diagonal and a maximum with the floor took four
+// DPX and one add.  Extension phase: 900k windows of 139-314 columns 6.02 to 5.61
+// ms, 201k of 314 2.66 to 2.47 ms, 240k of 183 in final-row mode 1.11 to 1.00 ms.
+// Score sets with mismatch > go + ge keep the four-DPX form (NN false).
 //
 // The best cell: per lane, the max over its rows of each column is compared
 // with the running best; a strict improvement records the column, so the
@@ -63,6 +74,9 @@ struct ExtArgs {
   uint32_t k16;
 };
 
+// whether every biased substitution score is >= 0 (the plain diagonal add)
+inline bool ext_nonneg(const ExtArgs& a) { return a.sb <= a.go + a.ge; }
+
 // kernel shapes (lanes per alignment, rows per lane) instantiated for the batched
 // engine; the plain engine uses the 256-row shapes only
 #define SR_SHAPES(X)                                                                         \
@@ -75,10 +89,14 @@ struct ExtArgs {
 
 // launch the int16 kernel of one shape and readout mode; -1 if the shape is not built
 int dispatch_mode0(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st,
-                   uint64_t plain_tasks);
+                   uint64_t tasks);
 int dispatch_mode1(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st,
-                   uint64_t plain_tasks);
+                   uint64_t tasks);
 int dispatch_mode2(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st);
+// every length class (at most upper[c] bases in class c) in one launch on 16 or
+// 32 lanes per pair (16 when !ext_nonneg), `pairs` item pairs in all
+int dispatch_all0(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
+int dispatch_all1(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
 
 namespace {
 
@@ -211,6 +229,58 @@ __device__ __forceinline__ uint32_t read_code(const uint32_t* row, uint32_t m, u
   return strand ? 3u - base_at(row, m - 1u - i) : base_at(row, i);
 }
 
+// The R bases (R <= 32) of a read as aligned from row i0 on, 2 bits each from bit 0
+// (x: rows 0-15, y: 16-31): three words of the packed row shifted into place and,
+// on the '-' strand, reversed and complemented.  Rows outside the read hold
+// anything; words outside its row are not read.
+template <int R>
+__device__ __forceinline__ uint2 lane_codes(const uint32_t* row, uint32_t m, uint32_t strand, int i0) {
+  const int s = strand ? static_cast<int>(m) - i0 - R : i0;  // the first base in read order
+  const int w = s >> 4;
+  uint32_t x[3];
+#pragma unroll
+  for (int k = 0; k < (R > 16 ? 3 : 2); ++k) x[k] = row[min(max(w + k, 0), kReadWords - 1)];
+  const uint32_t sh = 2u * (static_cast<uint32_t>(s) & 15u);
+  uint2 c;
+  c.x = __funnelshift_r(x[0], x[1], sh);
+  c.y = R > 16 ? __funnelshift_r(x[1], x[2], sh) : 0u;
+  if (strand) {
+    auto rev = [](uint32_t v) {
+      v = __brev(~v);
+      return ((v >> 1) & 0x55555555u) | ((v << 1) & 0xAAAAAAAAu);
+    };
+    // reversed, the bases are the top R of 32 (or 16) fields
+    constexpr int kDrop = 2 * ((R > 16 ? 32 : 16) - R);
+    if (R > 16) {
+      const uint32_t hi = rev(c.x), lo = rev(c.y);
+      c.x = __funnelshift_r(lo, hi, kDrop);
+      c.y = kDrop ? hi >> kDrop : hi;
+    } else {
+      c.x = rev(c.x) >> kDrop;
+    }
+  }
+  return c;
+}
+// 8 * code of row k
+__device__ __forceinline__ uint32_t code_shift(uint2 c, int k) {
+  const uint32_t v = k < 16 ? c.x : c.y;
+  const int b = 2 * (k & 15);
+  return (b >= 3 ? v >> (b - 3) : v << (3 - b)) & 24u;
+}
+
+// the codes of window bases p .. p + 3 (of the staged words), one per byte
+__device__ __forceinline__ uint32_t column_codes(const uint32_t* w, uint32_t p) {
+  const uint32_t x = __funnelshift_r(w[p >> 4], w[(p >> 4) + 1], 2u * (p & 15u)) & 0xffu;
+  const uint32_t t = (x | (x << 12)) & 0x000f000fu;
+  return (t | (t << 6)) & 0x03030303u;
+}
+// bytes of v for columns j .. j + 3 below n, of virt from n on
+__device__ __forceinline__ uint32_t keep_columns(uint32_t v, uint32_t virt, uint32_t j, uint32_t n) {
+  const uint32_t left = n > j ? n - j : 0u;
+  const uint32_t keep = left >= 4 ? 0xffffffffu : (1u << (8 * left)) - 1u;
+  return (v & keep) | (virt & ~keep);
+}
+
 // Blocks of 128 threads per SM the register budget is cut for (the sweep is
 // bound by the ALU pipe and the latency of its DPX chains, so resident warps
 // count).  Persistent kernels: up to 12 rows per lane fit 80 registers (6
@@ -226,8 +296,23 @@ constexpr int ext_min_blocks() {
          : (R <= (MODE == 1 ? 30 : 32) ? 3 : 2);
 }
 
-template <int G, int R, int MODE, bool PERSIST>
-__global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_extend16(ExtArgs a) {
+// this group's barrier and the virtual columns before column 0
+template <int G>
+__device__ __forceinline__ void ext_init(GroupSmem* gs, int glane) {
+  if (glane == 0) {
+    mbar_init(&gs->mbar, 1);
+    fence_mbar_init();
+  }
+  for (int c = glane; c < kColLead; c += G) gs->col[c] = static_cast<uint16_t>(kVirtLo | kVirtHi);
+  __syncwarp();
+}
+
+// the tasks (item pairs) of one length class, taken from its queue until it is
+// empty (PERSIST), or one task per group (the plain engine's items in input
+// order); phase: the group's barrier phase; SETUP: the group's barrier is still to
+// be set up.  False when a window copy timed out.
+template <int G, int R, int MODE, bool PERSIST, bool SETUP, bool NN>
+__device__ __forceinline__ bool ext_tasks(const ExtArgs& a, int cls, uint32_t& phase) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int GPW = 32 / G;
   const int lane = threadIdx.x & 31;
@@ -239,24 +324,22 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
   const int32_t goe = a.go + a.ge;
   const uint32_t GOE2 = static_cast<uint32_t>(goe) * 0x10001u;
   const uint32_t NGE2 = (static_cast<uint32_t>(-a.ge) & 0xffffu) * 0x10001u;
+  const uint32_t GE2 = static_cast<uint32_t>(a.ge) * 0x10001u;
   const uint32_t BIAS2 = static_cast<uint32_t>(kBias) * 0x10001u;
   const uint32_t INIT = static_cast<uint32_t>(kBias - goe) * 0x10001u;  // T of H = 0
   const uint32_t mis_b = static_cast<uint32_t>(goe - a.sb) & 0xffu;
   const uint32_t hit_b = static_cast<uint32_t>(a.sa + goe) & 0xffu;
   const uint32_t MIS4 = mis_b * 0x01010101u;
+  // 1, not known at compile time, and the subtracted constants: a multiply-add by
+  // it stays one
+  const uint32_t ONE = a.k16 >> 16, MGE2 = 0u - GE2, MGOE2 = 0u - GOE2;
 
-  if (glane == 0) {
-    mbar_init(&gs->mbar, 1);
-    fence_mbar_init();
-  }
-  for (int c = glane; c < kColLead; c += G) gs->col[c] = static_cast<uint16_t>(kVirtLo | kVirtHi);
-  __syncwarp();
-  uint32_t phase = 0;
+  if (SETUP) ext_init<G>(gs, glane);
 
   uint32_t begin = 0, count;
   if (PERSIST) {
-    begin = a.class_range[2 * a.cls];
-    count = a.class_range[2 * a.cls + 1] - begin;
+    begin = a.class_range[2 * cls];
+    count = a.class_range[2 * cls + 1] - begin;
   } else {
     count = static_cast<uint32_t>(a.n_items);
   }
@@ -267,7 +350,7 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
     uint32_t base;
     if (PERSIST) {
       uint32_t b0 = 0;
-      if (lane == 0) b0 = atomicAdd(a.queue + a.cls, static_cast<uint32_t>(GPW));
+      if (lane == 0) b0 = atomicAdd(a.queue + cls, static_cast<uint32_t>(GPW));
       base = __shfl_sync(FULL, b0, 0);
     } else {
       if (round > 0) break;
@@ -307,27 +390,24 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
       }
     }
 
-    // ---- per-row substitution tables (a4: query profile in registers)
+    // ---- per-row substitution tables (a4: query profile in registers): bytes of
+    // mismatch scores, the row's base's one turned into the match score
     uint32_t TL[R], TH[R];
     const int padlo = G * R - static_cast<int>(lo.m);
     const int padhi = G * R - static_cast<int>(hi.m);
     {
-      const uint32_t* rowlo = a.rpack + static_cast<size_t>(lo.read) * kReadWords;
-      const uint32_t* rowhi = a.rpack + static_cast<size_t>(hi.read) * kReadWords;
+      uint2 clo{}, chi{};
+      if (has_task) {
+        clo = lane_codes<R>(a.rpack + static_cast<size_t>(lo.read) * kReadWords, lo.m, lo.strand, glane * R - padlo);
+        chi = lane_codes<R>(a.rpack + static_cast<size_t>(hi.read) * kReadWords, hi.m, hi.strand, glane * R - padhi);
+      }
+      // rows above the read's first keep the mismatch score for every base
+      const int alo = has_task ? padlo - glane * R : R, ahi = has_task ? padhi - glane * R : R;
+      const uint32_t flip = mis_b ^ hit_b;
 #pragma unroll
       for (int k = 0; k < R; ++k) {
-        const int r = glane * R + k;
-        uint32_t tl = MIS4, th = MIS4;
-        if (has_task && r >= padlo) {
-          uint32_t c = read_code(rowlo, lo.m, lo.strand, static_cast<uint32_t>(r - padlo));
-          tl = (MIS4 & ~(0xffu << (8 * c))) | (hit_b << (8 * c));
-        }
-        if (has_task && r >= padhi) {
-          uint32_t c = read_code(rowhi, hi.m, hi.strand, static_cast<uint32_t>(r - padhi));
-          th = (MIS4 & ~(0xffu << (8 * c))) | (hit_b << (8 * c));
-        }
-        TL[k] = tl;
-        TH[k] = th;
+        TL[k] = MIS4 ^ ((k < alo ? 0u : flip) << code_shift(clo, k));
+        TH[k] = MIS4 ^ ((k < ahi ? 0u : flip) << code_shift(chi, k));
       }
     }
 
@@ -341,20 +421,24 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
       }
       phase ^= 1u;
     }
-    if (__any_sync(FULL, !ok)) break;
+    if (__any_sync(FULL, !ok)) return false;
     const uint32_t nmax = has_task ? max(lo.n, hi.n) : 0u;
     const uint32_t nlo = has_task ? lo.n : 0u, nhi = has_task ? hi.n : 0u;
     const uint32_t wmax = __reduce_max_sync(FULL, nmax);
     const int nsteps = static_cast<int>(wmax) + G - 1;
     {
-      // real columns, then virtual ones up to the last column any lane of the warp reaches
+      // real columns, then virtual ones up to the last column any lane of the warp
+      // reaches, four per lane and pass
       const uint32_t offlo = static_cast<uint32_t>(lo.ws - (w0lo << 4));
       const uint32_t offhi = static_cast<uint32_t>(hi.ws - (w0hi << 4));
       const uint32_t ncol = wmax + G - 1;
-      for (uint32_t j = glane; j < ncol; j += G) {
-        const uint32_t vlo = j < nlo ? kSelLo + base_at(gs->stage[0], offlo + j) * 0x11u : kVirtLo;
-        const uint32_t vhi = j < nhi ? kSelHi + base_at(gs->stage[1], offhi + j) * 0x1100u : kVirtHi;
-        gs->col[kColLead + j] = static_cast<uint16_t>(vlo | vhi);
+      uint2* dst = reinterpret_cast<uint2*>(gs->col + kColLead);
+      for (uint32_t j = 4 * glane; j < ncol; j += 4 * G) {
+        const uint32_t vlo = keep_columns(column_codes(gs->stage[0], offlo + j) * 0x11u + kSelLo * 0x01010101u,
+                                          kVirtLo * 0x01010101u, j, nlo);
+        const uint32_t vhi = keep_columns(column_codes(gs->stage[1], offhi + j) * 0x11u + (kSelHi >> 8) * 0x01010101u,
+                                          (kVirtHi >> 8) * 0x01010101u, j, nhi);
+        dst[j >> 2] = make_uint2(__byte_perm(vlo, vhi, 0x5140), __byte_perm(vlo, vhi, 0x7362));
       }
     }
     __syncwarp();
@@ -386,6 +470,11 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
     }
     const uint32_t lastmask = (MODE == 1 && glane == G - 1) ? FULL : 0u;
     const uint16_t* colp = gs->col + kColLead - glane;  // colp[s] = column s - glane
+    // Four (rows <= 16) or three columns per pass: the loop's own instructions are
+    // shared, and the code of eight classes' kernels still fits the instruction
+    // cache side by side.  33,000 pairs in 23 classes / 450,000: 473 / 5605 us; four
+    // columns for every row count 574 / 5583, two 482 / 5700, one 512 / 6040.
+#pragma unroll (R <= 16 ? 4 : 3)
     for (int s = 0; s < nsteps; ++s) {
       // lane 0's row above is the top border (H = 0, F = -inf): tin = fin = INIT
       const uint32_t tin = imad(__shfl_up_sync(FULL, Tbot, 1, G) - INIT, nz, INIT);
@@ -398,12 +487,21 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
         for (int k = 0; k < R; ++k) {
           const uint32_t sc = prmt(TL[k], TH[k], sel);
           const uint32_t tl = T[k];
-          E[k] = __viaddmax_s16x2(E[k], NGE2, tl);        // E(i,j) = max(E(i,j-1) - ge, T(i,j-1))
-          f = __viaddmax_s16x2(f, NGE2, tup);             // F(i,j) = max(F(i-1,j) - ge, T(i-1,j))
-          const uint32_t x = __viaddmax_s16x2(td, sc, E[k]);  // max(H(i-1,j-1) + s, E)
-          const uint32_t h = __vimax3_s16x2(x, f, BIAS2);     // H = max(x, F, 0)
-          td = tl;
-          tup = h - GOE2;  // plain add: each half stays >= 0
+          uint32_t h;
+          if constexpr (NN) {
+            // E(i,j) = max(E(i,j-1) - ge, T(i,j-1), 0): the floor of H taken here
+            E[k] = __vimax3_s16x2(imad(E[k], ONE, MGE2), tl, BIAS2);
+            f = __viaddmax_s16x2(f, NGE2, tup);       // F(i,j) = max(F(i-1,j) - ge, T(i-1,j))
+            h = __vimax3_s16x2(td + sc, E[k], f);     // H = max(H(i-1,j-1) + s, E, F)
+            td = tl;
+            tup = imad(h, ONE, MGOE2);                // each half stays >= 0
+          } else {
+            E[k] = __viaddmax_s16x2(E[k], NGE2, tl);
+            f = __viaddmax_s16x2(f, NGE2, tup);
+            h = __vimax3_s16x2(__viaddmax_s16x2(td, sc, E[k]), f, BIAS2);
+            td = tl;
+            tup = h - GOE2;
+          }
           T[k] = tup;
         }
         tprev = tin;
@@ -473,6 +571,57 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
       }
     }
     __syncwarp();
+  }
+  return true;
+}
+
+// NN: mismatch <= go + ge (ext_nonneg)
+template <int G, int R, int MODE, bool PERSIST, bool NN = true>
+__global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_extend16(ExtArgs a) {
+  uint32_t phase = 0;
+  ext_tasks<G, R, MODE, PERSIST, true, NN>(a, a.cls, phase);
+}
+
+// Every length class in one launch: a warp takes the longest class's pairs until
+// its queue is empty, then the next class's, each with the fewest rows per lane
+// that hold it (rows[c]: the class's reads have at most G * rows[c] bases).  One
+// kernel per class (k_extend16 on 8 lanes) does less work per cell, but a pair on
+// 8 lanes x 31 rows takes 0.15 ms however few there are, 23 classes queue up on
+// eight streams, and each ends in a tail of its own.  Bound by the ALU pipe once
+// its warps fill the chip, before that by the rows' chains of one pair.
+struct ExtRows {
+  uint8_t r[kNumBins];
+};
+template <int G, int MODE, bool NN>
+__global__ void __launch_bounds__(128, G == 32 ? 6 : MODE == 1 ? 4 : 5) k_extend_all(ExtArgs a, ExtRows rows) {
+  static_assert(G == 16 || G == 32, "16 or 32 lanes per pair");
+  {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31;
+    ext_init<G>(reinterpret_cast<GroupSmem*>(smem_raw) + ((threadIdx.x >> 5) * (32 / G) + lane / G), lane & (G - 1));
+  }
+  uint32_t phase = 0;
+  for (int c = kNumBins - 1; c >= 0; --c) {
+    if (a.class_range[2 * c] == a.class_range[2 * c + 1]) continue;
+    bool ok = true;
+#define SR_ROWS(g, n)                                         \
+  case n:                                                     \
+    ok = ext_tasks<g, n, MODE, true, false, NN>(a, c, phase); \
+    break;
+    if constexpr (G == 32) {
+      switch (rows.r[c]) {
+        SR_ROWS(32, 4) SR_ROWS(32, 5) SR_ROWS(32, 6) SR_ROWS(32, 7)
+        default: ok = ext_tasks<32, 8, MODE, true, false, NN>(a, c, phase);
+      }
+    } else {
+      switch (rows.r[c]) {
+        SR_ROWS(16, 5) SR_ROWS(16, 6) SR_ROWS(16, 7) SR_ROWS(16, 8) SR_ROWS(16, 9) SR_ROWS(16, 10)
+        SR_ROWS(16, 11) SR_ROWS(16, 12) SR_ROWS(16, 13) SR_ROWS(16, 14) SR_ROWS(16, 15)
+        default: ok = ext_tasks<16, 16, MODE, true, false, NN>(a, c, phase);
+      }
+    }
+#undef SR_ROWS
+    if (!ok) return;
   }
 }
 
@@ -577,12 +726,14 @@ __global__ void __launch_bounds__(128) k_extend32(ExtArgs a) {
   }
 }
 
-template <int G, int R, int MODE, bool PERSIST>
-int launch16(const ExtArgs& a, cudaStream_t st, uint64_t plain_tasks) {
+// tasks: the item pairs (0 with PERSIST: not known); a class of few pairs gets
+// only the blocks it needs, which leaves the others to the classes beside it
+template <int G, int R, int MODE, bool PERSIST, bool NN = true>
+int launch16(const ExtArgs& a, cudaStream_t st, uint64_t tasks) {
   constexpr int kThreads = 128;
   constexpr int groups = (kThreads / 32) * (32 / G);
   const size_t smem = sizeof(GroupSmem) * groups;
-  auto kern = k_extend16<G, R, MODE, PERSIST>;
+  auto kern = k_extend16<G, R, MODE, PERSIST, NN>;
   static bool attr_set = false;
   if (!attr_set) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -599,8 +750,10 @@ int launch16(const ExtArgs& a, cudaStream_t st, uint64_t plain_tasks) {
         cudaSuccess)
       return -1;
     grid = nsm * (per_sm > 0 ? per_sm : 1);
+    const uint64_t need = (tasks + groups - 1) / groups;
+    if (need && need < static_cast<uint64_t>(grid)) grid = static_cast<int>(need);
   } else {
-    uint64_t g = (plain_tasks + groups - 1) / groups;
+    uint64_t g = (tasks + groups - 1) / groups;
     if (g == 0) return 0;
     grid = static_cast<int>(g);
   }
@@ -608,6 +761,32 @@ int launch16(const ExtArgs& a, cudaStream_t st, uint64_t plain_tasks) {
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
+
+template <int G, int MODE, bool NN>
+int launch_all(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
+  constexpr int kThreads = 128;
+  constexpr int groups = (kThreads / 32) * (32 / G);
+  const size_t smem = sizeof(GroupSmem) * groups;
+  auto kern = k_extend_all<G, MODE, NN>;
+  static bool attr_set = false;
+  if (!attr_set) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+      return -1;
+    attr_set = true;
+  }
+  int dev = 0, nsm = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess) return -1;
+  const uint64_t most = static_cast<uint64_t>(nsm) * (per_sm > 0 ? per_sm : 1), need = (pairs + groups - 1) / groups;
+  ExtRows rows;
+  for (int c = 0; c < kNumBins; ++c) {
+    const uint32_t n = (upper[c] + G - 1) / G, lo = G == 32 ? 4 : 5, hi = 256 / G;
+    rows.r[c] = static_cast<uint8_t>(n < lo ? lo : n > hi ? hi : n);
+  }
+  kern<<<static_cast<unsigned>(need < most ? need : most), kThreads, smem, st>>>(a, rows);
+  return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+}
 
 }  // namespace
 }  // namespace sr

@@ -5,23 +5,33 @@
 namespace sr {
 
 int dispatch_mode0(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st,
-                   uint64_t plain_tasks) {
+                   uint64_t tasks) {
   if (!persist) {
+    if (!ext_nonneg(a)) return launch16<16, 16, 0, false, false>(a, st, tasks);
 #define SR_CASE(g, r) \
-  if (lanes == g && rows == r) return launch16<g, r, 0, false>(a, st, plain_tasks);
+  if (lanes == g && rows == r) return launch16<g, r, 0, false>(a, st, tasks);
     SR_PLAIN_SHAPES(SR_CASE)
 #undef SR_CASE
     return -1;
   }
 #define SR_CASE(g, r) \
-  if (lanes == g && rows == r) return launch16<g, r, 0, true>(a, st, 0);
+  if (lanes == g && rows == r) return launch16<g, r, 0, true>(a, st, tasks);
   SR_SHAPES(SR_CASE)
 #undef SR_CASE
   return -1;
 }
 
+int dispatch_all0(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
+  if (!ext_nonneg(a)) return launch_all<16, 0, false>(a, upper, pairs, st);
+  return lanes == 32 ? launch_all<32, 0, true>(a, upper, pairs, st) : launch_all<16, 0, true>(a, upper, pairs, st);
+}
+
 int preload_mode0() {
   int n_ = 0;
+  SR_TOUCH((k_extend_all<16, 0, true>));
+  SR_TOUCH((k_extend_all<32, 0, true>));
+  SR_TOUCH((k_extend_all<16, 0, false>));
+  SR_TOUCH((k_extend16<16, 16, 0, false, false>));
 #define SR_CASE(g, r) SR_TOUCH((k_extend16<g, r, 0, true>));
   SR_SHAPES(SR_CASE)
 #undef SR_CASE

@@ -226,11 +226,11 @@ int launch_pack_refs(const char* ascii, uint64_t len, uint32_t* words, uint32_t*
 int launch_prepare(const BatchDev& b, const DevRefs& refs, cudaStream_t st);
 int launch_bins(const BatchDev& b, const ScoreConst& sc, const TuneBin* bins, int n_bins,
                 bool force_i32, bool plain, cudaStream_t st);
-// class_items: items per length class (host; nullptr = launch every class);
+// class_items: items per length class (host; not read by the plain engine);
 // fan: side streams for the per-class kernels (nullptr = all on st)
 int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
                   const TuneBin* bins, int n_bins, int mode, bool plain, uint32_t lanes,
-                  uint32_t rows, cudaStream_t st, const uint64_t* class_items = nullptr,
+                  uint32_t rows, cudaStream_t st, const uint64_t* class_items,
                   const Fanout* fan = nullptr);
 int launch_select(const BatchDev& b, int n_refs, cudaStream_t st);
 int launch_winners(const BatchDev& b, const ScoreConst& sc, int mode, int n_refs, bool plain,
