@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "sr_extend.cuh"
 
 namespace sr {
@@ -37,15 +39,15 @@ ExtArgs make_args(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc) 
 
 }  // namespace
 
-int fanout_begin(const Fanout& f, cudaStream_t st) {
+int fanout_begin(const Fanout& f, cudaStream_t st, int n) {
   if (cudaEventRecord(f.fork, st) != cudaSuccess) return -1;
-  for (int i = 0; i < kSide; ++i)
+  for (int i = 0; i < n; ++i)
     if (cudaStreamWaitEvent(f.side[i], f.fork, 0) != cudaSuccess) return -1;
   return 0;
 }
 
-int fanout_end(const Fanout& f, cudaStream_t st) {
-  for (int i = 0; i < kSide; ++i) {
+int fanout_end(const Fanout& f, cudaStream_t st, int n) {
+  for (int i = 0; i < n; ++i) {
     if (cudaEventRecord(f.join[i], f.side[i]) != cudaSuccess) return -1;
     if (cudaStreamWaitEvent(st, f.join[i], 0) != cudaSuccess) return -1;
   }
@@ -112,8 +114,10 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
   // their form of the recurrence is built for it alone.
   uint64_t pairs = 0;
   uint32_t upper[kNumBins], longest = 0;
+  int present = 0, width = 0;
   for (int c = 0; c < n_bins; ++c) {
     upper[c] = bins[c].upper;
+    present += class_items[c] != 0 ? 1 : 0;
     pairs += (class_items[c] + 1) / 2;
     if (class_items[c]) longest = upper[c];
   }
@@ -127,9 +131,9 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
     if (k < 0) return -1;
     launched += k;
   } else {
-    if (fan && fanout_begin(*fan, st) < 0) return -1;
     int next = 0;
-    const int width = fan_width(b.n_reads);
+    width = std::min(fan_width(b.n_reads), present + (class_items[kI32Class] != 0 ? 1 : 0));
+    if (fan && fanout_begin(*fan, st, width) < 0) return -1;
     // longest reads first: each side stream starts on a large bin
     for (int c = n_bins - 1; c >= 0; --c) {
       if (class_items[c] == 0) continue;
@@ -153,7 +157,7 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
     if (cudaPeekAtLastError() != cudaSuccess) return -1;
     ++launched;
   }
-  if (!one && fan && fanout_end(*fan, st) < 0) return -1;
+  if (!one && fan && fanout_end(*fan, st, width) < 0) return -1;
   return launched;
 }
 

@@ -209,10 +209,10 @@ struct Fanout {
   cudaEvent_t fork;
   cudaEvent_t join[kSide];
 };
-// record the fork on st and make every side stream wait for it
-int fanout_begin(const Fanout& f, cudaStream_t st);
-// make st wait for everything enqueued on the side streams
-int fanout_end(const Fanout& f, cudaStream_t st);
+// record the fork on st and make the first n side streams wait for it
+int fanout_begin(const Fanout& f, cudaStream_t st, int n);
+// make st wait for everything enqueued on the first n side streams
+int fanout_end(const Fanout& f, cudaStream_t st, int n);
 
 struct TuneBin {
   uint32_t upper;  // largest read length in the bin

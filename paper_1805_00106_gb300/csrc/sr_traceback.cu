@@ -528,12 +528,16 @@ __device__ __forceinline__ void tb_stage_bytes(const TbArgs& a, const TbRead& x,
 // Which kernel traces a band class: k_tb_pair does the least work per read, but
 // its thread sweeps a read's cells one after another (17-32 diagonals: 0.30 ms
 // however few reads, 1-16: 0.17-0.20 ms), so it pays once reads fill the chip;
-// the wavefront's 2 rows + band steps take 0.03 ms.  Traceback phase by counts of
-// reads in the class, pair then wavefront: 17-32 diagonals, 60 reads of a
-// 2049-read batch 349 / 240 us, 5000 of 150k 651 / 651, 17,000 of 480k 1418 /
-// 1903; 1-16 diagonals, 9 reads 200 / 87 us, 2049-read batch 240 / 123, 20,000-read
-// batch 279 / 211, 40,000 931 / 903, 150k 651 / 956.
-constexpr uint32_t kTbWave32Reads = 4096;
+// the wavefront's 2 rows + band steps take 0.04 ms.  Traceback phase (us) by batch
+// size, pair then wavefront.  17-32 diagonals: 2049 reads 358 / 131, 40,000 421 /
+// 371, 40,000 of 250 bases with match 1 (wider bands) 877 / 850, 150,000 with match
+// 1 1243 / 1044, 480,000 1418 / 1903 (the class is a few percent of the reads, a
+// fifth with match 1, so the line is crossed between the last two).
+// 1-16 diagonals: 9 reads 202 / 88, a 2049-read batch 245 / 131, 10,000 reads 249 /
+// 144, 20,000 282 / 230, 150,000 651 / 956.  (Direction bytes in device memory
+// instead of shared memory, for more resident warps, made mid-size batches slower:
+// 80,000 reads 470 to 632 us.)
+constexpr uint32_t kTbWave32Reads = 16384;
 constexpr uint32_t kTbWave16Reads = 16384;
 
 template <int SEG>
@@ -1493,9 +1497,11 @@ int launch_traceback(const BatchDev& b, const DevRefs& refs, const ScoreConst& s
   k_tb_scan<<<1, kTbScanThreads, 0, st>>>(b.tb_count);
   k_tb_scatter<<<(b.n_reads + 255) / 256, 256, 0, st>>>(b.n_reads, code, cursor, list);
   int launched = 3;
-  if (fan && fanout_begin(*fan, st) < 0) return -1;
+  const bool pair = tb_pair_fits(a.sa, a.sb, a.go, a.ge);
+  const int kernels = pair ? 4 + (b.n_reads > kTbWave32Reads ? 1 : 0) + (b.n_reads > kTbWave16Reads ? 1 : 0) : 5;
   int next = 0;
-  const int width = fan_width(b.n_reads);
+  const int width = std::min(fan_width(b.n_reads), kernels);
+  if (fan && fanout_begin(*fan, st, width) < 0) return -1;
   auto lane_of = [&]() { return fan ? fan->side[next++ % width] : st; };
   auto waves = [&](auto kern, int per_warp, auto... args) -> bool {
     int per_sm = 0;
@@ -1536,7 +1542,6 @@ int launch_traceback(const BatchDev& b, const DevRefs& refs, const ScoreConst& s
     return cudaPeekAtLastError() == cudaSuccess;
   };
   // widest bands (longest kernels) first
-  const bool pair = tb_pair_fits(a.sa, a.sb, a.go, a.ge);
   const uint32_t all = 0xffffffffu;
   if (!waves(k_tb_wave2, 2, ranges + 2 * 6)) return -1;
   if (pair) {
@@ -1566,7 +1571,7 @@ int launch_traceback(const BatchDev& b, const DevRefs& refs, const ScoreConst& s
   k_traceback<<<grid, 32, smem, lane_of()>>>(a, list, ranges + 2 * (kTbBuckets - 1));
   ++launched;
   if (cudaPeekAtLastError() != cudaSuccess) return -1;
-  if (fan && fanout_end(*fan, st) < 0) return -1;
+  if (fan && fanout_end(*fan, st, width) < 0) return -1;
   return launched;
 }
 
