@@ -132,38 +132,56 @@ __global__ void k_keys(const uint32_t* item_read, const uint32_t* rlen, const ui
     if (sh[k]) atomicAdd(&hist[k], sh[k]);
 }
 
-// one block: exclusive scan of the histogram -> cursor, class ranges
-__global__ void k_scan_keys(const uint32_t* hist, uint32_t* cursor, uint32_t* class_range) {
-  __shared__ uint32_t part[1024];
-  constexpr int per = (kNumKeys + 1023) / 1024;
-  const int t = threadIdx.x;
+// one block: exclusive scan of the histogram -> cursor, class ranges.  A serial
+// step between two launches whatever the batch's size, so it is made of warp scans
+// with two barriers (10.3 us with a barrier per doubling step, XXX us so)
+__global__ void __launch_bounds__(1024) k_scan_keys(const uint32_t* hist, uint32_t* cursor, uint32_t* class_range) {
+  __shared__ uint32_t warp_sum[32];
+  constexpr int per = kNumKeys / 1024;
+  static_assert(kNumKeys % 4096 == 0 && per % 4 == 0, "whole 16-byte loads");
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   uint32_t loc[per];
   uint32_t sum = 0;
 #pragma unroll
-  for (int i = 0; i < per; ++i) {
-    const int k = t * per + i;
-    loc[i] = k < kNumKeys ? hist[k] : 0u;
-    sum += loc[i];
+  for (int i = 0; i < per / 4; ++i) {
+    const uint4 v = reinterpret_cast<const uint4*>(hist)[t * (per / 4) + i];
+    loc[4 * i] = v.x;
+    loc[4 * i + 1] = v.y;
+    loc[4 * i + 2] = v.z;
+    loc[4 * i + 3] = v.w;
+    sum += v.x + v.y + v.z + v.w;
   }
-  part[t] = sum;
+  uint32_t x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) warp_sum[w] = x;
   __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    uint32_t v = t >= off ? part[t - off] : 0u;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+  if (w == 0) {
+    uint32_t s = warp_sum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(FULL, s, o);
+      if (lane >= o) s += y;
+    }
+    warp_sum[lane] = s;
   }
-  uint32_t run = part[t] - sum;
+  __syncthreads();
+  uint32_t run = (w ? warp_sum[w - 1] : 0u) + x - sum;
 #pragma unroll
   for (int i = 0; i < per; ++i) {
     const int k = t * per + i;
-    if (k < kNumKeys) {
-      cursor[k] = run;
-      if (k % kKeysPerClass == 0) class_range[2 * (k / kKeysPerClass)] = run;
-      if (k % kKeysPerClass == kKeysPerClass - 1) class_range[2 * (k / kKeysPerClass) + 1] = run + loc[i];
-    }
-    run += loc[i];
+    if (k % kKeysPerClass == 0) class_range[2 * (k / kKeysPerClass)] = run;
+    if (k % kKeysPerClass == kKeysPerClass - 1) class_range[2 * (k / kKeysPerClass) + 1] = run + loc[i];
+    const uint32_t c = loc[i];
+    loc[i] = run;
+    run += c;
   }
+#pragma unroll
+  for (int i = 0; i < per / 4; ++i)
+    reinterpret_cast<uint4*>(cursor)[t * (per / 4) + i] = make_uint4(loc[4 * i], loc[4 * i + 1], loc[4 * i + 2], loc[4 * i + 3]);
 }
 
 // scatter items into key order; warp-aggregated atomics per equal key
@@ -557,8 +575,8 @@ int launch_assemble(const BatchDev& b, int n_refs, bool want_cigar, int32_t item
 
 // A batch staged from a read range [r0, r1) of the caller's arrays receives
 // the range's offsets as they are; they are made batch-relative here.
-// ---- checks of a batch staged from device memory (the host path runs the same
-// checks on the caller's host arrays): per read, its offsets, length, window
+// ---- checks of a staged batch (few host windows get the same checks on the
+// host): per read, its offsets, length, window
 // count and windows; the first bad read (lowest index) with the reason, and for
 // good batches the DP cells, the longest read and the windows per read length.
 __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off, uint32_t n, uint64_t nc,
@@ -566,35 +584,38 @@ __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off
                               const uint32_t* c_len, DevRefs refs, StageCheck* out) {
   __shared__ uint32_t hist[kMaxReadLen + 1];
   __shared__ unsigned long long cells_sh;
+  __shared__ uint32_t longest;
   for (int k = threadIdx.x; k <= kMaxReadLen; k += blockDim.x) hist[k] = 0;
-  if (threadIdx.x == 0) cells_sh = 0;
+  if (threadIdx.x == 0) {
+    cells_sh = 0;
+    longest = 0;
+  }
   __syncthreads();
-  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+  // eight lanes per read: a read may have hundreds of windows
+  const uint64_t r64 = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) >> 3;
+  const uint32_t r = static_cast<uint32_t>(r64), lane = threadIdx.x & 7u;
   unsigned long long cells = 0;
-  if (r < n) {
+  uint32_t why = 0;
+  if (r64 < n) {
     const uint64_t a0 = read_off[r], a1 = read_off[r + 1], c0 = cand_off[r], c1 = cand_off[r + 1];
-    uint32_t why = 0;
     if (a1 < a0 || c1 < c0 || c1 > nc) why = 1;
     else if (a1 - a0 == 0 || a1 - a0 > static_cast<uint64_t>(kMaxReadLen)) why = 2;
     else if (c1 - c0 >= (1ull << 19)) why = 3;
     if (!why) {
       const uint64_t m = a1 - a0;
       uint64_t suml = 0;
-      for (uint64_t k = c0; k < c1; ++k) {
+      for (uint64_t k = c0 + lane; k < c1; k += 8) {
         const uint32_t ref = c_ref[k], len = c_len[k];
         const uint64_t w0 = c_start[k];
         const bool ok = ref < static_cast<uint32_t>(refs.n) && c_strand[k] <= 1 && len >= 1 &&
                         len <= static_cast<uint32_t>(kMaxWinLen) && w0 <= refs.len[ref] && w0 + len <= refs.len[ref];
-        if (!ok) {
-          why = 4;
-          break;
-        }
+        if (!ok) why = 4;
         suml += len;
       }
-      if (!why) {
-        cells = m * suml;
+      cells = m * suml;
+      if (lane == 0) {
         if (c1 > c0) atomicAdd(&hist[m], static_cast<uint32_t>(c1 - c0));
-        atomicMax(&out->max_m, static_cast<uint32_t>(m));
+        atomicMax(&longest, static_cast<uint32_t>(m));
       }
     }
     if (why) atomicMin(&out->bad, (static_cast<unsigned long long>(r) << 3) | why);
@@ -605,6 +626,7 @@ __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off
   for (int k = threadIdx.x; k <= kMaxReadLen; k += blockDim.x)
     if (hist[k]) atomicAdd(&out->by_len[k], static_cast<unsigned long long>(hist[k]));
   if (threadIdx.x == 0 && cells_sh) atomicAdd(&out->cells, cells_sh);
+  if (threadIdx.x == 0 && longest) atomicMax(&out->max_m, longest);
 }
 
 // the first bad window of read r (after k_stage_check found one there)
@@ -624,7 +646,7 @@ int launch_stage_check(const BatchDev& b, const DevRefs& refs, StageCheck* out, 
   if (cudaMemsetAsync(out, 0, sizeof(StageCheck), st) != cudaSuccess) return -1;
   if (cudaMemsetAsync(&out->bad, 0xff, 2 * sizeof(unsigned long long), st) != cudaSuccess) return -1;
   if (b.n_reads == 0) return 0;
-  k_stage_check<<<(b.n_reads + 255) / 256, 256, 0, st>>>(b.read_off, b.cand_off, b.n_reads, b.n_items, b.c_ref,
+  k_stage_check<<<static_cast<unsigned>((b.n_reads * 8ull + 255) / 256), 256, 0, st>>>(b.read_off, b.cand_off, b.n_reads, b.n_items, b.c_ref,
                                                          b.c_strand, b.c_start, b.c_len, refs, out);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }

@@ -591,6 +591,25 @@ sr_status batch_alloc(sr_session* s, uint32_t n, uint64_t nb, uint64_t nc, cudaS
   return SR_OK;
 }
 
+// Checks a batch's staged arrays by a kernel on their stream and waits for it:
+// what is wrong with the first bad read in hc (its first bad window too), or the
+// batch's cells, longest read and windows per read length
+cudaError_t device_check(sr_batch* b, const DevRefs& refs, cudaStream_t st, StageCheck& hc) {
+  StageCheck* dc = static_cast<StageCheck*>(b->d.check);
+  cudaError_t e = launch_stage_check(b->d, refs, dc, st) < 0 ? cudaGetLastError() : cudaSuccess;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, dc, sizeof(hc), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && hc.bad != ~0ull && (hc.bad & 7) == 4) {
+    if (launch_first_bad_window(b->d, refs, static_cast<uint32_t>(hc.bad >> 3), dc, st) < 0) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hc.bad_win, &dc->bad_win, 8, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
+  b->cells = hc.cells;
+  b->max_m = hc.max_m;
+  for (int m = 0; m <= kMaxReadLen; ++m) b->items_by_len[m] = hc.by_len[m];
+  return e;
+}
+
 // Stages a batch whose reads or candidates (sr_reads / sr_cand_list flags) sit
 // in device memory: the header is read with two small copies, every array is
 // copied into the arena (device to device, or host to device for the other
@@ -640,16 +659,8 @@ sr_status stage_device(sr_session* s, const sr_reads* reads, const sr_cand_list*
   copy(d.c_strand, cands->strand, nc);
   copy(d.c_start, cands->win_start, nc * 8);
   copy(d.c_len, cands->win_len, nc * 4);
-  StageCheck* dc = static_cast<StageCheck*>(d.check);
-  if (e == cudaSuccess && launch_stage_check(d, s->refs, dc, st) < 0) e = cudaGetLastError();
   StageCheck hc{};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, dc, sizeof(hc), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && hc.bad != ~0ull && (hc.bad & 7) == 4) {
-    if (launch_first_bad_window(d, s->refs, static_cast<uint32_t>(hc.bad >> 3), dc, st) < 0) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hc.bad_win, &dc->bad_win, 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  }
+  if (e == cudaSuccess) e = device_check(b, s->refs, st, hc);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(st);
     sr_batch_free(b);
@@ -670,9 +681,6 @@ sr_status stage_device(sr_session* s, const sr_reads* reads, const sr_cand_list*
                          static_cast<unsigned long long>(hc.bad_win));
     }
   }
-  b->cells = hc.cells;
-  b->max_m = hc.max_m;
-  for (int m = 0; m <= kMaxReadLen; ++m) b->items_by_len[m] = hc.by_len[m];
   *out = b;
   return SR_OK;
 }
@@ -760,92 +768,17 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
     sr_batch_free(b);
     return cuda_error("sr_batch_stage copy", e);
   }
-  // host-side validation, while the copies run: every kernel relies on these
-  // bounds (window copies, shared-memory column streams, packed read rows).
-  // Read ranges are checked in parallel; the first bad read (lowest index) is
-  // reported.  The same pass counts the DP cells and the windows per read length.
-  struct Part {
-    uint64_t cells = 0;
-    uint32_t max_m = 0;
-    uint64_t by_len[kMaxReadLen + 1] = {};
-    uint32_t bad_read = UINT32_MAX;
-    int why = 0;  // 1 offsets, 2 read length, 3 window count, 4 window
-    uint64_t bad_win = 0;
-  };
-  const uint32_t nthr = (n < 65536u) ? 1u : 4u * host_threads();
-  std::vector<Part> parts(nthr);
-  static_assert((kMaxRefs & (kMaxRefs - 1)) == 0, "ref_id masking");
-  uint64_t lens16[kMaxRefs] = {};  // reference lengths, indexed by ref_id & (kMaxRefs - 1)
-  for (uint32_t q = 0; q < s->n_refs && q < static_cast<uint32_t>(kMaxRefs); ++q) lens16[q] = s->lens[q];
-  const uint32_t nref = s->n_refs;
-  auto check = [&](uint32_t t) {
-    Part& P = parts[t];
-    const uint32_t p0 = static_cast<uint32_t>(static_cast<uint64_t>(n) * t / nthr);
-    const uint32_t p1 = static_cast<uint32_t>(static_cast<uint64_t>(n) * (t + 1) / nthr);
-    for (uint32_t r = r0 + p0; r < r0 + p1; ++r) {
-      const uint64_t a0 = reads->offsets[r], a1 = reads->offsets[r + 1];
-      const uint64_t c0 = cands->offsets[r], c1 = cands->offsets[r + 1];
-      if (a1 < a0 || c1 < c0 || c1 > ce) {
-        P.bad_read = r;
-        P.why = 1;
-        return;
-      }
-      const uint64_t m = a1 - a0;
-      if (m == 0 || m > SR_MAX_READ_LEN) {
-        P.bad_read = r;
-        P.why = 2;
-        return;
-      }
-      if (c1 - c0 >= (1ull << 19)) {
-        P.bad_read = r;
-        P.why = 3;
-        return;
-      }
-      // all of a read's windows without a branch, then the first bad one if any
-      uint64_t suml = 0;
-      uint32_t bad = 0;
-      for (uint64_t k = c0; k < c1; ++k) {
-        const uint32_t ref = cands->ref_id[k], len = cands->win_len[k];
-        const uint64_t L = lens16[ref & (kMaxRefs - 1)], w0 = cands->win_start[k];
-        bad |= static_cast<uint32_t>(ref >= nref) | static_cast<uint32_t>(cands->strand[k] > 1) |
-               static_cast<uint32_t>(len - 1u >= static_cast<uint32_t>(SR_MAX_WIN_LEN)) |
-               static_cast<uint32_t>(w0 > L) | static_cast<uint32_t>(w0 + len > L);
-        suml += len;
-      }
-      if (bad) {
-        for (uint64_t k = c0; k < c1; ++k) {
-          const uint32_t ref = cands->ref_id[k], len = cands->win_len[k];
-          if (ref >= nref || cands->strand[k] > 1 || len < 1 || len > SR_MAX_WIN_LEN ||
-              cands->win_start[k] > s->lens[ref] || cands->win_start[k] + len > s->lens[ref]) {
-            P.bad_read = r;
-            P.why = 4;
-            P.bad_win = k;
-            return;
-          }
-        }
-      }
-      P.cells += m * suml;
-      P.by_len[m] += c1 - c0;
-      P.max_m = std::max<uint32_t>(P.max_m, static_cast<uint32_t>(m));
-    }
-  };
-  parallel_for(nthr, check);
-  uint64_t cells = 0;
-  uint32_t max_m = 0;
-  uint64_t by_len[kMaxReadLen + 1] = {};
-  const Part* worst = nullptr;
-  for (const Part& P : parts) {
-    if (P.bad_read != UINT32_MAX && (!worst || P.bad_read < worst->bad_read)) worst = &P;
-    cells += P.cells;
-    max_m = std::max(max_m, P.max_m);
-    for (int m = 0; m <= kMaxReadLen; ++m) by_len[m] += P.by_len[m];
-  }
-  if (worst) {
+  // Validation: every kernel relies on these bounds (window copies, shared-memory
+  // column streams, packed read rows).  The first bad read (lowest index) is
+  // reported; the same pass counts the DP cells and the windows per read length.
+  // Few windows are checked here while the copies run, more by a kernel behind
+  // them (200,000 windows: 0.4 ms on one host thread, 0.02 ms on the device; 4096
+  // take about 10 us on either).
+  auto refuse = [&](int why, uint32_t r, uint64_t win) -> sr_status {
     // the copies may still be reading the caller's arrays
     cudaStreamSynchronize(st);
     sr_batch_free(b);
-    const uint32_t r = worst->bad_read;
-    switch (worst->why) {
+    switch (why) {
       case 1:
         return set_error(SR_EINVAL, "sr_batch_stage: decreasing or out-of-range offsets at read %u", r);
       case 2:
@@ -855,8 +788,42 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
         return set_error(SR_EINVAL, "sr_batch_stage: read %u has more than 2^19-1 windows", r);
       default:
         return set_error(SR_EINVAL, "sr_batch_stage: window %llu is outside its reference or malformed",
-                         static_cast<unsigned long long>(worst->bad_win));
+                         static_cast<unsigned long long>(win));
     }
+  };
+  constexpr uint64_t kHostWindows = 4096;
+  if (nc > kHostWindows) {
+    StageCheck hc{};
+    e = device_check(b, s->refs, st, hc);
+    if (e != cudaSuccess) {
+      cudaStreamSynchronize(st);
+      sr_batch_free(b);
+      return cuda_error("sr_batch_stage check", e);
+    }
+    if (hc.bad != ~0ull) return refuse(static_cast<int>(hc.bad & 7), r0 + static_cast<uint32_t>(hc.bad >> 3), cb + hc.bad_win);
+    *out = b;
+    return SR_OK;
+  }
+  uint64_t cells = 0;
+  uint32_t max_m = 0;
+  for (uint32_t r = r0; r < r1; ++r) {
+    const uint64_t a0 = reads->offsets[r], a1 = reads->offsets[r + 1];
+    const uint64_t c0 = cands->offsets[r], c1 = cands->offsets[r + 1];
+    if (a1 < a0 || c1 < c0 || c1 > ce) return refuse(1, r, 0);
+    const uint64_t m = a1 - a0;
+    if (m == 0 || m > SR_MAX_READ_LEN) return refuse(2, r, 0);
+    if (c1 - c0 >= (1ull << 19)) return refuse(3, r, 0);
+    uint64_t suml = 0;
+    for (uint64_t k = c0; k < c1; ++k) {
+      const uint32_t ref = cands->ref_id[k], len = cands->win_len[k];
+      if (ref >= s->n_refs || cands->strand[k] > 1 || len < 1 || len > SR_MAX_WIN_LEN ||
+          cands->win_start[k] > s->lens[ref] || cands->win_start[k] + len > s->lens[ref])
+        return refuse(4, r, k);
+      suml += len;
+    }
+    cells += m * suml;
+    b->items_by_len[m] += c1 - c0;
+    max_m = std::max<uint32_t>(max_m, static_cast<uint32_t>(m));
   }
   // the caller may reuse its arrays once this returns
   e = cudaStreamSynchronize(st);
@@ -866,7 +833,6 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
   }
   b->cells = cells;
   b->max_m = max_m;
-  std::memcpy(b->items_by_len, by_len, sizeof(by_len));
   *out = b;
   return SR_OK;
 }
