@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(32 * kCalWarps, 12) k_cal_seeds(SeedArgs a) {
         uint32_t hl0 = 0, hh0 = 0, hl1 = 0, hh1 = 0;
         bool head = false;
         if (a.di.heads && live)
-          head = lookup_head(a.di.heads, pb, pkey, a.di.key_bits, &hl0, &hh0, &hl1, &hh1);
+          head = lookup_head(a.di, pb, pkey, &hl0, &hh0, &hl1, &hh1);
         for (int r2 = 0; r2 < a.di.n_refs; ++r2) {
           uint64_t lo = 0, hi = 0;
           if (live) {
@@ -465,33 +465,34 @@ int launch_cal_slots(const uint64_t* read_off, uint32_t n, int k, uint32_t strid
 }
 
 // one thread per bucket: its head from jptr and key16 / key (the layout at DevIndex)
-__global__ void k_cal_heads(DevIndex di, uint64_t nb, uint4* heads) {
+__global__ void k_cal_heads(DevIndex di, uint64_t nb, uint32_t* heads) {
   const uint64_t b = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
   if (b >= nb) return;
   const int R = di.n_refs;
   const uint32_t s0 = di.jptr[b * R], e0 = di.jptr[(b + 1) * R];
   const uint32_t s1 = R > 1 ? di.jptr[b * R + 1] : 0u, e1 = R > 1 ? di.jptr[(b + 1) * R + 1] : 0u;
   const uint64_t n0 = e0 - s0, n1 = e1 - s1;
+  const bool k16 = di.key_bits == 16, wide = di.head_words == 16;
+  const int most = k16 ? (wide ? kHeadKeys16 : kHeadNear16) : (wide ? kHeadKeys32 : kHeadNear32);
   uint32_t w[16];
   for (int i = 0; i < 16; ++i) w[i] = 0;
   w[0] = s0;
   w[1] = s1;
-  if (di.key_bits == 16 && n0 + n1 <= static_cast<uint64_t>(kHeadKeys)) {
-    w[2] = static_cast<uint32_t>(n0 | (n1 << 16));
-    for (uint32_t i = 0; i < n0 + n1; ++i) {
-      const uint32_t kk = i < n0 ? di.key16[0][s0 + i] : di.key16[1][s1 + (i - n0)];
-      w[3 + (i >> 1)] |= kk << (16 * (i & 1));
-    }
-  } else if (di.key_bits != 16 && n0 + n1 <= static_cast<uint64_t>(kHeadKeys32)) {
-    w[2] = static_cast<uint32_t>(n0 | (n1 << 16));
-    for (uint32_t i = 0; i < n0 + n1; ++i) w[3 + i] = i < n0 ? di.key[0][s0 + i] : di.key[1][s1 + (i - n0)];
-  } else {
+  if (n0 + n1 > static_cast<uint64_t>(most)) {
     w[2] = kHeadSpill;
+  } else {
+    w[2] = static_cast<uint32_t>(n0 | (n1 << 8));
+    for (uint32_t i = 0; i < n0 + n1; ++i) {
+      const int r = i < n0 ? 0 : 1;
+      const uint32_t e = r ? s1 + (i - static_cast<uint32_t>(n0)) : s0 + i;
+      if (k16) w[2 + ((i + 1) >> 1)] |= static_cast<uint32_t>(di.key16[r][e]) << (16 * ((i + 1) & 1));
+      else w[3 + i] = di.key[r][e];
+    }
   }
-  for (int j = 0; j < 4; ++j) heads[b * 4 + j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+  for (int i = 0; i < di.head_words; ++i) heads[b * di.head_words + i] = w[i];
 }
 
-int launch_cal_heads(const DevIndex& di, uint64_t nbuckets, uint4* heads, cudaStream_t st) {
+int launch_cal_heads(const DevIndex& di, uint64_t nbuckets, uint32_t* heads, cudaStream_t st) {
   if (!di.packed || di.n_refs < 1 || di.n_refs > 2) return -1;
   if (nbuckets == 0) return 0;
   k_cal_heads<<<static_cast<unsigned>((nbuckets + 255) / 256), 256, 0, st>>>(di, nbuckets, heads);

@@ -75,53 +75,68 @@ __device__ __forceinline__ void lookup_packed(const DevIndex& di, uint64_t b, ui
   else key_range(di.key[r], s0, s1, key, lo, hi);
 }
 
-// 32-bit keys: the head holds up to kHeadKeys32, one per word
-__device__ __forceinline__ bool head_range32(const uint4 v0, const uint4 v1, const uint4 v2, const uint4 v3,
-                                             uint32_t key, uint32_t* lo0, uint32_t* hi0, uint32_t* lo1,
-                                             uint32_t* hi1) {
-  const uint32_t w[13] = {v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w, v3.x, v3.y, v3.z, v3.w};
-  uint32_t eq = 0;
-#pragma unroll
-  for (int j = 0; j < 13; ++j) eq |= (w[j] == key ? 1u : 0u) << j;
-  const uint32_t n0 = v0.z & 0xffffu, n1 = v0.z >> 16;
-  const uint32_t m0 = (1u << n0) - 1u, m1 = ((1u << (n0 + n1)) - 1u) & ~m0;
-  const uint32_t e0 = eq & m0, e1 = eq & m1;
-  *lo0 = v0.x + (e0 ? __ffs(e0) - 1u : 0u);
-  *hi0 = *lo0 + __popc(e0);
-  *lo1 = v0.y + (e1 ? __ffs(e1) - 1u - n0 : 0u);
-  *hi1 = *lo1 + __popc(e1);
-  return true;
+// 32 aligned bytes, used once (no L1 line kept), as one request
+__device__ __forceinline__ void ld_once_32(const uint32_t* p, uint32_t (&v)[8]) {
+  asm("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+      : "l"(p));
+}
+
+// bits 0 and 1: the low and the high half of w equal key (kk: it in both halves).
+// A half of w ^ kk is zero exactly when adding 0x7fff to its low 15 bits leaves
+// its top bit clear and its top bit was clear.
+__device__ __forceinline__ uint32_t halves_equal(uint32_t w, uint32_t kk) {
+  const uint32_t x = w ^ kk;
+  const uint32_t z = ~(((x & 0x7fff7fffu) + 0x7fff7fffu) | x) & 0x80008000u;
+  return ((z >> 15) & 1u) | (z >> 30);
 }
 
 // packed index with bucket heads: entries [lo0, hi0) of reference 0 and [lo1,
 // hi1) of reference 1 with key `key` in bucket b, from the bucket's head alone
 // (an empty range may start anywhere); false when the bucket spilled (its
-// entries are then looked up in jptr / key16)
-__device__ __forceinline__ bool lookup_head(const uint4* heads, uint64_t b, uint32_t key, int key_bits,
-                                            uint32_t* lo0, uint32_t* hi0, uint32_t* lo1, uint32_t* hi1) {
-  const uint4* h = heads + b * 4;
-  const uint4 v0 = __ldg(h), v1 = __ldg(h + 1), v2 = __ldg(h + 2), v3 = __ldg(h + 3);
-  if (v0.z == kHeadSpill) return false;
-  if (key_bits != 16) return head_range32(v0, v1, v2, v3, key, lo0, hi0, lo1, hi1);
-  const uint32_t w[13] = {v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w, v3.x, v3.y, v3.z, v3.w};
-  // bit i: the head's key i equals the seed's, two keys per word: a 16-bit half
-  // of w ^ (key, key) is zero exactly when adding 0x7fff to its low 15 bits
-  // leaves its top bit clear and its top bit was clear
-  const uint32_t kk = key | (key << 16);
-  uint32_t eq = 0;
+// entries are then looked up in jptr and the keys).
+//
+// Random reads of a table past the L2 are bound by the number of 32-byte requests,
+// each of which moves about 106 bytes of DRAM: 293 G/s over 32 MB, 76 over 256 MB,
+// 59 over 512 MB and 54 over 1 GB (6.3 TB/s of DRAM), and 64 bytes as two of them
+// at half that.  So the counts and the first keys lie in the first 32 bytes, and
+// the others are read only where a bucket has more: 300k xenograft reads against
+// 2 x 16 Mbp 1.21 ms with one 64-byte head per seed, 0.77 with 32.
+__device__ __forceinline__ bool lookup_head(const DevIndex& di, uint64_t b, uint32_t key, uint32_t* lo0, uint32_t* hi0,
+                                            uint32_t* lo1, uint32_t* hi1) {
+  const uint32_t* h = di.heads + b * static_cast<uint32_t>(di.head_words);
+  uint32_t v[8];
+  ld_once_32(h, v);
+  if (v[2] == kHeadSpill) return false;
+  const uint32_t n0 = v[2] & 0xffu, n1 = (v[2] >> 8) & 0xffu;
+  uint32_t eq = 0;  // bit i: key i of the head
+  if (di.key_bits == 16) {
+    const uint32_t kk = key | (key << 16);
 #pragma unroll
-  for (int j = 0; j < 13; ++j) {
-    const uint32_t x = w[j] ^ kk;
-    const uint32_t z = ~(((x & 0x7fff7fffu) + 0x7fff7fffu) | x) & 0x80008000u;
-    eq |= (((z >> 15) & 1u) | (z >> 30)) << (2 * j);
+    for (int j = 0; j < 6; ++j) eq |= halves_equal(v[2 + j], kk) << (2 * j);
+    eq >>= 1;  // the first half holds the counts
+    if (n0 + n1 > static_cast<uint32_t>(kHeadNear16)) {
+      uint32_t u[8];
+      ld_once_32(h + 8, u);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) eq |= halves_equal(u[j], kk) << (kHeadNear16 + 2 * j);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < kHeadNear32; ++j) eq |= (v[3 + j] == key ? 1u : 0u) << j;
+    if (n0 + n1 > static_cast<uint32_t>(kHeadNear32)) {
+      uint32_t u[8];
+      ld_once_32(h + 8, u);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) eq |= (u[j] == key ? 1u : 0u) << (kHeadNear32 + j);
+    }
   }
   // equal keys are consecutive within each reference's run of sorted keys
-  const uint32_t n0 = v0.z & 0xffffu, n1 = v0.z >> 16;
   const uint32_t m0 = (1u << n0) - 1u, m1 = ((1u << (n0 + n1)) - 1u) & ~m0;
   const uint32_t e0 = eq & m0, e1 = eq & m1;
-  *lo0 = v0.x + (e0 ? __ffs(e0) - 1u : 0u);
+  *lo0 = v[0] + (e0 ? __ffs(e0) - 1u : 0u);
   *hi0 = *lo0 + __popc(e0);
-  *lo1 = v0.y + (e1 ? __ffs(e1) - 1u - n0 : 0u);
+  *lo1 = v[1] + (e1 ? __ffs(e1) - 1u - n0 : 0u);
   *hi1 = *lo1 + __popc(e1);
   return true;
 }

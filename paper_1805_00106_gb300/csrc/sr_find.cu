@@ -196,13 +196,14 @@ __device__ __forceinline__ uint32_t warp_merge(WarpSpace& w, uint32_t nh, uint64
   return nwin;
 }
 
-// What bounds it: dependent random accesses (a seed's 64-byte bucket head, then
-// its entry's position), hidden by resident warps; so nothing but the lookups
-// touches device memory and the registers are held to 40 warps per SM.  1M
-// xenograft reads of 100 bases against 2 x 16 Mbp: 4.0 ms, where the count, emit,
-// filter and compaction passes over kept lookups and CALs took 7.2 ms.  128 runs
-// and 64 ranks: a unique 250-base read has about 8 runs, and a read with more
-// copies than that shares its counting better over a block.
+// What bounds it: random requests to the index, a seed's bucket head and its
+// entry's position (300k reads of 100 bases against 2 x 16 Mbp: 45M of them in 0.77
+// ms, 58 G/s, DRAM 75% busy; the issue slots are 62% busy).  So nothing but the
+// lookups touches device memory, and the registers are held to 40 warps per SM to
+// hide their latency.  1M such reads: 2.6 ms, where the count, emit, filter and
+// compaction passes over kept lookups and CALs took 7.2 ms.  128 runs and 64
+// ranks: a unique 250-base read has about 8 runs, and a read with more copies than
+// that shares its counting better over a block.
 __global__ void __launch_bounds__(32 * kFindWarps, 10) k_find_warp(FindArgs a) {
   __shared__ __align__(16) WarpSpace ws[kFindWarps];
   if (bad_reads(a)) return;
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(32 * kFindWarps, 10) k_find_warp(FindArgs a) {
           const uint64_t h = seed_hash(canon, k, a.di.hash_seed[0]);
           pb = h >> kb;
           pkey = static_cast<uint32_t>(h & mask_bits(kb));
-          if (a.di.heads) head = lookup_head(a.di.heads, pb, pkey, a.di.key_bits, &hl0, &hh0, &hl1, &hh1);
+          if (a.di.heads) head = lookup_head(a.di, pb, pkey, &hl0, &hh0, &hl1, &hh1);
         }
         for (int r2 = 0; r2 < a.di.n_refs && !bail; ++r2) {
           uint64_t lo = 0, hi = 0;
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
           const uint64_t h = seed_hash(canon, k, a.di.hash_seed[0]), pb = h >> kb;
           const uint32_t pkey = static_cast<uint32_t>(h & mask_bits(kb));
           uint32_t hl0 = 0, hh0 = 0, hl1 = 0, hh1 = 0;
-          if (a.di.heads && lookup_head(a.di.heads, pb, pkey, a.di.key_bits, &hl0, &hh0, &hl1, &hh1)) {
+          if (a.di.heads && lookup_head(a.di, pb, pkey, &hl0, &hh0, &hl1, &hh1)) {
             lo = r2 ? hl1 : hl0;
             hi = r2 ? hh1 : hh0;
           } else {

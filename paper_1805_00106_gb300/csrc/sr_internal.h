@@ -281,14 +281,16 @@ struct DevIndex {
   const uint16_t* key16[kMaxRefs];
   const uint32_t* posor[kMaxRefs];
   int packed, key_bits;
-  // bucket heads (packed form, one or two references; nullptr otherwise): 64
-  // bytes per bucket, read with one access: its first entry in references 0 and
-  // 1 (words 0, 1), their entry counts (word 2, 16 bits each) and up to
-  // kHeadKeys 16-bit keys (two per word, low half first) or kHeadKeys32 32-bit
-  // ones, reference 0's then reference 1's in entry order (words 3-15).  Word 2
-  // is kHeadSpill where they do not fit: that bucket is looked up in jptr and
-  // the keys.
-  const uint4* heads;
+  // bucket heads (packed form, one or two references; nullptr otherwise): one of
+  // head_words words (8 or 16) per bucket: its first entry in references 0 and 1
+  // (words 0, 1), their entry counts (the low two bytes of word 2) and its keys,
+  // reference 0's then reference 1's in entry order: 16-bit ones from the high
+  // half of word 2 on, two per word, or 32-bit ones from word 3 on.  The first
+  // kHeadNear16 or kHeadNear32 keys sit in the first 32 bytes; a head of 8 words
+  // holds no more, one of 16 words kHeadKeys16 or kHeadKeys32.  Word 2 is
+  // kHeadSpill where a bucket does not fit: it is looked up in jptr and the keys.
+  const uint32_t* heads;
+  int head_words;
   uint64_t ref_len[kMaxRefs];
   uint64_t hash_seed[kMaxRefs];
   int n_refs, k, a;
@@ -314,11 +316,12 @@ struct CalRanges {
   uint8_t* recount = nullptr;
   uint32_t rbase = 0;
 };
-constexpr int kHeadKeys = 26;
-constexpr int kHeadKeys32 = 13;
+constexpr int kHeadNear16 = 11, kHeadKeys16 = 27;
+constexpr int kHeadNear32 = 5, kHeadKeys32 = 13;
 constexpr uint32_t kHeadSpill = 0xffffffffu;
-// the bucket heads of a packed index (nbuckets buckets, n_refs <= 2) into heads
-int launch_cal_heads(const DevIndex& di, uint64_t nbuckets, uint4* heads, cudaStream_t st);
+// the bucket heads of a packed index (nbuckets buckets, n_refs <= 2, head_words
+// set) into heads
+int launch_cal_heads(const DevIndex& di, uint64_t nbuckets, uint32_t* heads, cudaStream_t st);
 // Emit pass of the reads whose lookups were kept (device list big, n_big of
 // them), by many blocks per read, after launch_cal_seeds' emit pass (which takes
 // the others); its part tables take cal_sort_words(n_big) words after the

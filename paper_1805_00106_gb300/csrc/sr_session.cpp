@@ -121,13 +121,13 @@ bool res_create(BatchRes& r) {
 }
 constexpr size_t kResPool = 16;
 constexpr size_t kKeptArenas = 3;
-// a positive integer from the environment, else dflt
-uint64_t env_u64(const char* name, uint64_t dflt) {
+// a positive integer from the environment (with zero: or 0), else dflt
+uint64_t env_u64(const char* name, uint64_t dflt, bool zero = false) {
   const char* v = getenv(name);
   if (!v || !*v) return dflt;
   char* end = nullptr;
   const unsigned long long x = strtoull(v, &end, 10);
-  return (end && *end == 0 && x > 0) ? static_cast<uint64_t>(x) : dflt;
+  return (end && *end == 0 && (x > 0 || (zero && end != v))) ? static_cast<uint64_t>(x) : dflt;
 }
 // roles of the device CAL finder's cached scratch buffers
 enum CalBuf : int {
@@ -1406,23 +1406,27 @@ extern "C" sr_status sr_session_attach_index(sr_session* s, const sr_index* cons
   s->didx.n_refs = static_cast<int>(n_refs);
   s->didx.k = static_cast<int>(t[0].seed_len);
   s->didx.a = static_cast<int>(t[0].address_bases);
-  // bucket heads, built on the device from the packed tables: where buckets are
-  // small (on average at most half a head's 16-bit keys, or 8 of its 13 32-bit
-  // ones, so that few spill) a seed's lookup in both references is one 64-byte
-  // access instead of three dependent ones (SR_CAL_HEADS=0 leaves them out)
+  // bucket heads, built on the device from the packed tables, where buckets are
+  // small: a seed's lookup in both references is one access instead of three
+  // dependent ones.  With at most 4 entries per bucket on average (2 with 32-bit
+  // keys) heads of 32 bytes: fewer than 1 bucket in 1000 (60) spills, and random
+  // reads of the table run the faster the smaller it is (537 MB at a = 12: 59 G/s;
+  // 1.07 GB: 54).  Else, with at most half of what 64 bytes hold (13 of 27 16-bit
+  // keys, 8 of 13 32-bit ones), those.  SR_CAL_HEADS=0 leaves the heads out.
   const uint64_t nbk = t[0].n_ptr ? t[0].n_ptr - 1 : 0;
   uint64_t entries = 0;
   for (uint32_t r = 0; r < n_refs; ++r) entries += t[r].n_entries;
-  const uint64_t per_bucket = keys16 ? kHeadKeys / 2 : 8;
-  if (packed && n_refs <= 2 && nbk && nbk <= (1ull << 26) && entries <= nbk * per_bucket &&
-      env_u64("SR_CAL_HEADS", 1) != 0) {
+  const uint64_t per_wide = keys16 ? 13 : 8, per_near = keys16 ? 4 : 2;
+  if (packed && n_refs <= 2 && nbk && nbk <= (1ull << 26) && entries <= nbk * per_wide &&
+      env_u64("SR_CAL_HEADS", 1, true) != 0) {
     void* ph = nullptr;
-    if (cudaMalloc(&ph, nbk * 64) == cudaSuccess) {
+    s->didx.head_words = entries <= nbk * per_near ? 8 : 16;
+    if (cudaMalloc(&ph, nbk * s->didx.head_words * 4) == cudaSuccess) {
       s->idx_bufs.push_back(ph);
-      if (launch_cal_heads(s->didx, nbk, static_cast<uint4*>(ph), s->stream) < 0 ||
+      if (launch_cal_heads(s->didx, nbk, static_cast<uint32_t*>(ph), s->stream) < 0 ||
           cudaStreamSynchronize(s->stream) != cudaSuccess)
         return fail();
-      s->didx.heads = static_cast<const uint4*>(ph);
+      s->didx.heads = static_cast<const uint32_t*>(ph);
     } else {
       cudaGetLastError();  // the heads are optional: without them the lookups read jptr / key16
     }

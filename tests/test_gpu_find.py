@@ -60,12 +60,14 @@ def test_distinct_cals_around_each_table(sr, unit, copies):
 
 
 @pytest.mark.parametrize("table", ["1", "3", "40", "1000000"])
-@pytest.mark.parametrize("k,addr,seeds,heads", [(20, 12, (0, 0), "1"), (20, 12, (0, 0), "0"), (25, 12, (0, 0), "1"),
-                                                (20, 10, (5, 9), "1"), (16, 8, (0, 0, 0), "1")])
+@pytest.mark.parametrize("k,addr,seeds,heads", [(20, 12, (0, 0), "1"), (20, 12, (0, 0), "0"),
+                                                (25, 12, (0, 0), "1"), (16, 8, (0, 0), "1"),
+                                                (18, 7, (0, 0), "1"), (20, 10, (5, 9), "1"), (16, 8, (0, 0, 0), "1")])
 def test_every_index_form_and_table_size(sr, monkeypatch, table, k, addr, seeds, heads):
-    """The index forms (heads, packed, per reference, three references) with the
-    tables held to few distinct CALs, so that reads go on to the next path, the
-    large-read one included; its chunks cut small too."""
+    """The index forms (heads of both sizes, few or most of their buckets spilled,
+    no heads, per reference, three references) with the tables held to few
+    distinct CALs, so that reads go on to the next path, the large-read one
+    included; its chunks cut small too."""
     monkeypatch.setenv("SR_CAL_TABLE", table)
     monkeypatch.setenv("SR_CAL_HEADS", heads)
     w = S.workload("c3", scale=0.0005, seed=31, rc_frac=0.5)
