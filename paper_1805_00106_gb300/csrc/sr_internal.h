@@ -83,7 +83,7 @@ struct BatchDev {
   uint32_t* class_range = nullptr;  // 2 * kNumClasses
   uint32_t* queue = nullptr;      // kNumClasses + 8 counters
   unsigned long long* cells = nullptr;  // 1 counter
-  uint32_t* status = nullptr;     // 1 word
+  uint32_t* status = nullptr;     // status word, then the CIGAR words of the batch
   // outputs
   int32_t* item_score = nullptr;
   uint32_t* item_end = nullptr;

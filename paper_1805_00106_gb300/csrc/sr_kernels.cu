@@ -399,7 +399,7 @@ __global__ void k_scan_block(const DevHit* hits, int slots, uint32_t n, uint32_t
   if (threadIdx.x == 1023) block_sums[blockIdx.x] = sh[1023];
 }
 
-__global__ void k_scan_sums(uint32_t* block_sums, uint32_t nb, uint32_t* total_out) {
+__global__ void k_scan_sums(uint32_t* block_sums, uint32_t nb, uint32_t* total_out, uint32_t* total_copy) {
   __shared__ uint32_t carry;
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
@@ -420,7 +420,7 @@ __global__ void k_scan_sums(uint32_t* block_sums, uint32_t nb, uint32_t* total_o
     if (threadIdx.x == 1023) carry += sh[1023];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *total_out = carry;
+  if (threadIdx.x == 0) *total_out = *total_copy = carry;
 }
 
 __global__ void k_cigar_gather(const DevHit* hits, int slots, uint32_t n, const uint32_t* block_sums,
@@ -694,7 +694,7 @@ int launch_cigar_compact(const BatchDev& b, int n_refs, cudaStream_t st) {
   const int slots = 1 + n_refs;
   const uint32_t nb = (b.n_reads + 1023) / 1024;
   k_scan_block<<<nb, 1024, 0, st>>>(b.hits, slots, b.n_reads, b.cigar_off, b.scan_tmp);
-  k_scan_sums<<<1, 1024, 0, st>>>(b.scan_tmp, nb, b.cigar_off + b.n_reads);
+  k_scan_sums<<<1, 1024, 0, st>>>(b.scan_tmp, nb, b.cigar_off + b.n_reads, b.status + 1);
   k_cigar_gather<<<(b.n_reads + 255) / 256, 256, 0, st>>>(b.hits, slots, b.n_reads, b.scan_tmp,
                                                           b.cigar_off, b.cigar_slots, b.cigar);
   return cudaPeekAtLastError() == cudaSuccess ? 3 : -1;

@@ -198,6 +198,7 @@ struct sr_batch {
   uint64_t i32_items = 0;
   bool ran = false;
   bool assembled = false;  // the last run also assembled the result records (serving rounds)
+  std::vector<char> inputs;  // few input bytes, gathered for one copy
   sr_align_opts last_opts{};
   BatchRes res{};  // events, side streams (from the session's pool)
   bool res_ok = false;
@@ -433,14 +434,17 @@ uint64_t carve_batch(BatchDev& d, uint32_t n, uint64_t nb, uint64_t nc, uint32_t
   c.take(d.cursor, kNumKeys);
   c.take(d.class_range, 2 * kNumClasses);
   c.take(d.queue, kNumClasses + 8);
-  c.take(d.status, 4);
-  c.take(d.item_score, nc);
-  c.take(d.item_end, nc);
   c.take(d.hits, static_cast<uint64_t>(n) * (1 + n_refs));
   c.take(d.cigar_slots, static_cast<uint64_t>(n) * kCigarStride);
   c.take(d.cigar_off, n + 1ull);
-  c.take(d.cigar, static_cast<uint64_t>(n) * kCigarStride);
+  // what a fetch copies, in one piece
+  c.take(d.status, 4);
+  c.take(d.item_score, nc);
+  c.take(d.item_end, nc);
+  c.take(d.out_best, n);
+  c.take(d.out_per_ref, static_cast<uint64_t>(n) * n_refs);
   c.take(d.read_class, n);
+  c.take(d.cigar, static_cast<uint64_t>(n) * kCigarStride);
   c.take(d.scan_tmp, n / 1024 + 4ull);
   c.take(d.item_iend, nc);
   c.take(d.wcount, kNumClasses);
@@ -451,8 +455,6 @@ uint64_t carve_batch(BatchDev& d, uint32_t n, uint64_t nb, uint64_t nc, uint32_t
   c.take(d.tb_count, kTbCountWords);
   c.take(d.tb_dirs, tb_dirs_words(n));
   c.take(d.tb_dirs32, tb_dirs32_words(n));
-  c.take(d.out_best, n);
-  c.take(d.out_per_ref, static_cast<uint64_t>(n) * n_refs);
   StageCheck* pc;
   c.take(pc, 1);
   d.check = pc;
@@ -742,23 +744,31 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
   const BatchDev& d = b->d;
   cudaError_t e = cudaSuccess;
   cudaStream_t st = b->stream;
-  if (nb) e = cudaMemcpyAsync(const_cast<char*>(d.bases), reads->bases + rb, nb, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(const_cast<uint64_t*>(d.read_off), reads->offsets + r0, (n + 1ull) * 8,
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(const_cast<uint64_t*>(d.cand_off), cands->offsets + r0, (n + 1ull) * 8,
-                        cudaMemcpyHostToDevice, st);
-  if (nc) {
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(const_cast<uint8_t*>(d.c_ref), cands->ref_id + cb, nc, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(const_cast<uint8_t*>(d.c_strand), cands->strand + cb, nc, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(const_cast<uint64_t*>(d.c_start), cands->win_start + cb, nc * 8, cudaMemcpyHostToDevice,
-                          st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(const_cast<uint32_t*>(d.c_len), cands->win_len + cb, nc * 4, cudaMemcpyHostToDevice, st);
+  // the input arrays lie behind one another on the device: few bytes are gathered
+  // here, kept with the batch until its stream has read them, and copied in one
+  // piece; more are copied array by array
+  const struct {
+    const void *dst, *src;
+    uint64_t bytes;
+  } in[7] = {{d.bases, reads->bases + rb, nb},
+             {d.read_off, reads->offsets + r0, n ? (n + 1ull) * 8 : 0},
+             {d.cand_off, cands->offsets + r0, n ? (n + 1ull) * 8 : 0},
+             {d.c_ref, cands->ref_id + cb, nc},
+             {d.c_strand, cands->strand + cb, nc},
+             {d.c_start, cands->win_start + cb, nc * 8},
+             {d.c_len, cands->win_len + cb, nc * 4}};
+  const char* in0 = d.bases;
+  const uint64_t in_bytes = static_cast<uint64_t>(reinterpret_cast<const char*>(d.c_len) - in0) + nc * 4;
+  const bool gathered = in_bytes <= (48u << 10);
+  if (gathered) {
+    b->inputs.resize(in_bytes);
+    for (const auto& x : in)
+      if (x.bytes) memcpy(b->inputs.data() + (static_cast<const char*>(x.dst) - in0), x.src, x.bytes);
+    if (in_bytes) e = cudaMemcpyAsync(const_cast<char*>(in0), b->inputs.data(), in_bytes, cudaMemcpyHostToDevice, st);
+  } else {
+    for (const auto& x : in)
+      if (e == cudaSuccess && x.bytes)
+        e = cudaMemcpyAsync(const_cast<void*>(x.dst), x.src, x.bytes, cudaMemcpyHostToDevice, st);
   }
   if (e == cudaSuccess && n && (launch_rebase_offsets(const_cast<uint64_t*>(d.read_off), n + 1ull, rb, st) < 0 ||
                                 launch_rebase_offsets(const_cast<uint64_t*>(d.cand_off), n + 1ull, cb, st) < 0))
@@ -826,7 +836,7 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
     max_m = std::max<uint32_t>(max_m, static_cast<uint32_t>(m));
   }
   // the caller may reuse its arrays once this returns
-  e = cudaStreamSynchronize(st);
+  if (!gathered) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     sr_batch_free(b);
     return cuda_error("sr_batch_stage copy", e);
@@ -1087,18 +1097,23 @@ sr_status batch_run_async(sr_session* s, sr_batch* b, const sr_score_params* sp,
   return SR_OK;
 }
 
-sr_status batch_sync(sr_batch* b, cudaStream_t stream) {
-  cudaError_t e = cudaStreamSynchronize(stream);
-  if (e != cudaSuccess) return cuda_error("sr_batch_sync", e);
-  uint32_t st = 0;
-  e = cudaMemcpy(&st, b->d.status, 4, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_error("sr_batch_sync status", e);
+// a run's status word as a status
+static sr_status run_status(uint32_t st) {
   if (st & kStBadBase) return set_error(SR_EBADBASE, "read has a non-ACGT base");
   if (st & kStBadRead) return set_error(SR_EINVAL, "read length must be 1..256");
   if (st & kStBadWindow) return set_error(SR_EINVAL, "window outside its reference, bad ref id/strand or length not in 1..512");
   if (st & kStTimeout) return set_error(SR_ETIMEOUT, "device wait for a window copy ran out");
   if (st & (kStOverflow | kStInternal)) return set_error(SR_ECUDA, "device internal check failed (status %u)", st);
   return SR_OK;
+}
+
+sr_status batch_sync(sr_batch* b, cudaStream_t stream) {
+  cudaError_t e = cudaStreamSynchronize(stream);
+  if (e != cudaSuccess) return cuda_error("sr_batch_sync", e);
+  uint32_t st = 0;
+  e = cudaMemcpy(&st, b->d.status, 4, cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_error("sr_batch_sync status", e);
+  return run_status(st);
 }
 
 }  // namespace sr
@@ -1161,6 +1176,8 @@ struct ResultsBox {
   uint64_t block_bytes = 0;
   void* cig_block = nullptr;  // the CIGAR words, when they sit in a block of their own
   uint64_t cig_block_bytes = 0;
+  void* plain = nullptr;      // small results: every array in one malloc'ed block,
+  void* plain_cig = nullptr;  // the CIGAR words in another when the first had no room
 };
 
 sr_results* results_alloc() {
@@ -1222,6 +1239,12 @@ extern "C" void sr_results_free(sr_results* r) {
     session_release(s);
     return;
   }
+  if (box->plain) {
+    free(box->plain);
+    free(box->plain_cig);
+    free(box);
+    return;
+  }
   free(r->best);
   free(r->best_per_ref);
   free(r->item_score);
@@ -1237,10 +1260,71 @@ extern "C" sr_status sr_batch_fetch(sr_session* s, sr_batch* b, sr_results** out
   if (!b->ran) return set_error(SR_EINVAL, "sr_batch_fetch: batch has not run");
   *out = nullptr;
   cudaStream_t stream = b->last_opts.cuda_stream ? static_cast<cudaStream_t>(b->last_opts.cuda_stream) : b->stream;
-  sr_status st = batch_sync(b, stream);
-  if (st != SR_OK) return st;
   const uint32_t n = b->n_reads, nr = s->n_refs;
   const uint64_t nc = b->n_items;
+  {
+    // small results (serving rounds, requests): the status, every array and room
+    // for the CIGAR words lie behind one another on the device, so one copy into
+    // one block of plain memory and one wait fetch them (pinning costs more than
+    // it saves); CIGARs longer than the room come after
+    const bool cig = b->last_opts.want_cigar != 0;
+    const char* from = reinterpret_cast<const char*>(b->d.status);
+    const uint64_t cig_at = static_cast<uint64_t>(reinterpret_cast<const char*>(b->d.cigar) - from);
+    const uint64_t room = cig ? std::min<uint64_t>(6ull * n + 256, static_cast<uint64_t>(n) * kCigarStride) : 0;
+    const uint64_t bytes = cig_at + 4 * room;
+    if (bytes < (16ull << 20)) {
+      sr_results* r = results_alloc();
+      char* blk = r ? static_cast<char*>(malloc(bytes)) : nullptr;
+      if (!blk) {
+        free(r);
+        return set_error(SR_ENOMEM, "sr_batch_fetch: out of memory");
+      }
+      auto* box = reinterpret_cast<ResultsBox*>(r);
+      box->plain = blk;
+      if (!b->assembled && launch_assemble(b->d, static_cast<int>(nr), cig, 0, 0, stream) < 0) {
+        sr_results_free(r);
+        return cuda_error("sr_batch_fetch assemble", cudaGetLastError());
+      }
+      cudaError_t e = cudaMemcpyAsync(blk, from, bytes, cudaMemcpyDeviceToHost, stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+      const uint32_t* word = reinterpret_cast<const uint32_t*>(blk);  // status, CIGAR words
+      sr_status st = e == cudaSuccess ? run_status(word[0]) : cuda_error("sr_batch_fetch copy", e);
+      auto host = [&](const void* p) { return blk + (reinterpret_cast<const char*>(p) - from); };
+      r->cigar = cig ? reinterpret_cast<uint32_t*>(blk + cig_at) : nullptr;
+      if (st == SR_OK && cig && n) {
+        r->n_cigar = word[1];
+        if (r->n_cigar > room) {
+          box->plain_cig = malloc(r->n_cigar * 4);
+          if (!box->plain_cig) {
+            st = set_error(SR_ENOMEM, "sr_batch_fetch: out of memory");
+          } else {
+            e = cudaMemcpyAsync(box->plain_cig, b->d.cigar, r->n_cigar * 4, cudaMemcpyDeviceToHost, stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+            if (e != cudaSuccess) st = cuda_error("sr_batch_fetch copy", e);
+            r->cigar = static_cast<uint32_t*>(box->plain_cig);
+          }
+        }
+      }
+      if (st != SR_OK) {
+        sr_results_free(r);
+        return st;
+      }
+      r->n_reads = n;
+      r->n_refs = nr;
+      r->n_items = nc;
+      r->cells = b->cells;
+      r->n_i32_items = b->i32_items;
+      r->item_score = reinterpret_cast<int32_t*>(host(b->d.item_score));
+      r->item_end = reinterpret_cast<uint32_t*>(host(b->d.item_end));
+      r->best = reinterpret_cast<sr_hit*>(host(b->d.out_best));
+      r->best_per_ref = reinterpret_cast<sr_hit*>(host(b->d.out_per_ref));
+      if (b->last_opts.classify) r->read_class = reinterpret_cast<uint8_t*>(host(b->d.read_class));
+      *out = r;
+      return SR_OK;
+    }
+  }
+  sr_status st = batch_sync(b, stream);
+  if (st != SR_OK) return st;
   sr_results* r = results_alloc();
   if (!r) return set_error(SR_ENOMEM, "sr_batch_fetch: out of memory");
   r->n_reads = n;
@@ -1280,8 +1364,7 @@ extern "C" sr_status sr_batch_fetch(sr_session* s, sr_batch* b, sr_results** out
   const uint64_t o_cig = cig ? part(static_cast<uint64_t>(total) * 4) : 0;
   const uint64_t o_cls = cls ? part(n) : 0;
   uint64_t got = 0;
-  // small results (serving rounds) use plain memory: pinning costs more than it saves
-  char* blk = off >= (16ull << 20) ? static_cast<char*>(pool_take(s, off, &got)) : nullptr;
+  char* blk = static_cast<char*>(pool_take(s, off, &got));
   if (blk) {
     auto* box = reinterpret_cast<ResultsBox*>(r);
     box->pool_of = s;
@@ -2354,7 +2437,7 @@ extern "C" sr_status sr_align_batch(sr_session* s, const sr_reads* reads, const 
   sr_batch* b = nullptr;
   sr_status st = sr_batch_stage(s, reads, cands, opts ? opts->cuda_stream : nullptr, &b);
   if (st != SR_OK) return st;
-  st = sr_batch_run(s, b, sp, opts);
+  st = batch_run_async(s, b, sp, opts);  // the fetch waits, and checks the run's status
   if (st == SR_OK) st = sr_batch_fetch(s, b, out);
   sr_batch_free(b);
   return st;
