@@ -1,6 +1,6 @@
 // sr_cal.cu -- the large-read path of the CAL finder and filter (McVicar et al.,
 // arXiv 1805.00106, Sec. 3.2 CAL finder, Sec. 3.3 CAL filter): the reads whose
-// distinct CALs do not fit the tables of sr_find.cu (over 6144 of them).  Every
+// distinct CALs do not fit the tables of sr_find.cu (over 12288 of them).  Every
 // pass runs on many blocks per read.  Same windows as the host stage
 // sr_candidates.
 //

@@ -16,7 +16,7 @@
 //                 ballot folds into one (CAL, count) run.  Up to kRuns runs and
 //                 kRanks ranks; other reads are listed for
 //   k_find_block  one block per read, the CALs counted in a hash table in shared
-//                 memory (768, then 6144 distinct ones); reads with more are
+//                 memory (768, then 12288 distinct ones); reads with more are
 //                 listed for the large-read path (sr_cal.cu).
 //   k_find_out    the windows, staged in any order, into the list's arrays.
 #include <cuda_runtime.h>
@@ -341,38 +341,48 @@ __global__ void __launch_bounds__(32 * kFindWarps, 10) k_find_warp(FindArgs a) {
 }
 
 // One block per read.  S table slots (a power of two), up to 3/4 of them used; T
-// threads.  Records of one reference's seeds at a time are taken by groups of
-// eight lanes: most hold a few entries, a repeat's hold thousands, consecutive.
-// Bound by the shared-memory table (a load and an add per CAL).  10k reads of 250
-// bases, 30% repeats, no CAL limit (51M CALs): 0.82 ms in the small table and
-// 0.60 ms in the large one, where sorting the CALs took 6.6 ms.  The small table
-// leaves room for 9 blocks per SM; the large one (160 KB) takes the few reads of
-// short tandem units.
-template <int S, int T>
+// threads; reads of more than ENTRIES entries are left to the larger block.
+// Records of one reference's seeds at a time are taken by groups of eight lanes:
+// most hold a few entries, a repeat's hold thousands, consecutive.  Bound by the
+// shared-memory table (a load and an add per CAL) and, before reads of many
+// entries went to the larger block, by the last small block's read.  10k reads of
+// 250 bases, 30% repeats, no CAL limit (36M CALs, half of them of 294 reads with
+// more than 16384): whole call 2.47 to 1.90 ms by that line (8192: 1.88, 32768:
+// 2.04), 20k reads with limit 1024 1.94 to 1.40 (1.50, 1.78); 1.19 and 1.33 with
+// 16384 instead of 8192 slots in the large table, which keeps reads like the one
+// here of 8721 distinct CALs off the large-read path.  The small table leaves room
+// for 10 blocks per SM.
+constexpr int kElBits = 14;  // bits of an element's number beside its count (at most one per seed)
+constexpr uint32_t kElMask = (1u << kElBits) - 1u;
+static_assert(2 * kMaxReadLen < (1 << (32 - kElBits)), "a CAL's count and an element number in 32 bits");
+constexpr uint32_t kCutWindows = 4096;  // more windows are cut to max_cands by the large-read path
+
+template <int S, int T, uint32_t ENTRIES>
 struct BlockSpace {
   static constexpr uint32_t kDistinct = S / 4 * 3;
-  // the table (keys, counts), then in its place the sorted elements (S), each
-  // window's best (kDistinct), the count prefixes and the window starts
-  static constexpr uint32_t kBytes = S * 8 + kDistinct * 8 + 2 * (kDistinct + 2) * 4;
+  static constexpr uint32_t kEntries = ENTRIES;
+  // the table (keys, counts), then in its place the sorted elements (S) and each
+  // window's best element and hits (kDistinct)
+  static constexpr uint32_t kBytes = S * 8 + kDistinct * 8;
+  static_assert(S <= (1 << kElBits), "element numbers");
 };
 
-template <int S, int T>
+template <int S, int T, uint32_t ENTRIES>
 __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* list, const uint32_t* n_list, uint32_t* queue,
                                                   uint32_t* next, uint32_t* n_next) {
-  using Space = BlockSpace<S, T>;
+  using Space = BlockSpace<S, T, ENTRIES>;
   constexpr int kGroup = 8, kGroups = T / kGroup, kPer = S / T;
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ __align__(16) uint8_t q[kMaxReadLen];
   __shared__ uint32_t pk[kPackWords], rk[kPackWords];
   __shared__ uint64_t rec[kMaxReadLen];
-  __shared__ uint32_t s_item, s_distinct, s_over;
+  __shared__ uint32_t s_item, s_distinct, s_over, s_total;
   __shared__ unsigned long long s_slot;
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(sm);
   uint32_t* cnts = reinterpret_cast<uint32_t*>(sm + S * 8);
   uint64_t* el = reinterpret_cast<uint64_t*>(sm);
-  unsigned long long* best = reinterpret_cast<unsigned long long*>(sm + S * 8);
-  uint32_t* pre = reinterpret_cast<uint32_t*>(sm + S * 8 + Space::kDistinct * 8);
-  uint32_t* wst = pre + Space::kDistinct + 2;
+  uint32_t* best = reinterpret_cast<uint32_t*>(sm + S * 8);
+  uint32_t* hits = best + Space::kDistinct;
   const uint32_t tid = threadIdx.x;
   const uint32_t most = min(Space::kDistinct, a.merge_keys);
   if (bad_reads(a)) return;
@@ -394,7 +404,7 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
       cnts[i] = 0;
     }
     if (tid == 0) {
-      s_distinct = s_over = 0;
+      s_distinct = s_over = s_total = 0;
     }
     const uint32_t nseeds = (m - k) / a.stride + 1;  // listed reads have m >= k
     // one CAL into the table; past `most` distinct ones the read is given up (the
@@ -445,7 +455,11 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
         const bool fits = hi - lo <= most && lo <= kRangeLoMax;
         if (!fits) s_over = 1;
         rec[si] = fits ? range_pack(lo, static_cast<uint32_t>(hi - lo), rori) : 0ull;
+        if (fits && hi > lo) atomicAdd(&s_total, static_cast<uint32_t>(hi - lo));
       }
+      __syncthreads();
+      // too much work for this many threads: left to the larger block
+      if (s_total > Space::kEntries) s_over = 1;
       __syncthreads();
       for (uint32_t si = tid / kGroup; si < nseeds; si += kGroups) {
         const uint64_t x = rec[si];
@@ -495,66 +509,76 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
     for (uint32_t i = n + tid; i < P; i += T) el[i] = kNone;
     __syncthreads();
     bitonic(el, P);
-    // windows: starts numbered by one prefix sum with the counts'
+    // windows, their starts numbered by a prefix sum over the threads' slices; each
+    // slice offers its part of a window its most frequent CAL (the smallest of
+    // equally frequent ones) and adds its hits
     const uint32_t per = (n + T - 1) / T, i0 = min(n, tid * per), i1 = min(n, i0 + per);
     auto starts = [&](uint32_t i) {
       if (i == 0) return true;
       const uint64_t c = el[i] >> kCntBits, p = el[i - 1] >> kCntBits;
       return (c >> kCalBits) != (p >> kCalBits) || c - p > static_cast<uint64_t>(a.merge_dist);
     };
-    uint64_t sum = 0;
-    for (uint32_t i = i0; i < i1; ++i) sum += (el[i] & kCntMask) | (starts(i) ? 1ull << 32 : 0ull);
-    const uint64_t ex = block_exscan(sum, &tot);
-    const uint32_t nwin = static_cast<uint32_t>(tot >> 32);
-    {
-      uint32_t c = static_cast<uint32_t>(ex), wk = static_cast<uint32_t>(ex >> 32);
-      for (uint32_t i = i0; i < i1; ++i) {
-        pre[i] = c;
-        c += static_cast<uint32_t>(el[i]) & kCntMask;
-        if (starts(i)) wst[wk++] = i;
-      }
-    }
-    if (tid == 0) {
-      pre[n] = static_cast<uint32_t>(tot);
-      wst[nwin] = n;
-    }
-    for (uint32_t j = tid; j < nwin; j += T) best[j] = 0ull;
+    uint32_t sum = 0;
+    for (uint32_t i = i0; i < i1; ++i) sum += starts(i) ? 1u : 0u;
+    uint32_t wk = static_cast<uint32_t>(block_exscan(sum, &tot));
+    const uint32_t nwin = static_cast<uint32_t>(tot);
+    for (uint32_t j = tid; j < nwin; j += T) best[j] = hits[j] = 0;
     __syncthreads();
     {
-      uint32_t wk = static_cast<uint32_t>(ex >> 32);
+      uint32_t top = 0, add = 0;
       for (uint32_t i = i0; i < i1; ++i) {
-        if (starts(i)) ++wk;
-        // the most frequent CAL, the smallest of equally frequent ones
-        atomicMax(&best[wk - 1], static_cast<unsigned long long>(((el[i] & kCntMask) << 32) | (0xffffffffu - i)));
+        if (starts(i)) {
+          if (add) {
+            atomicMax(&best[wk - 1], top);
+            atomicAdd(&hits[wk - 1], add);
+          }
+          top = add = 0;
+          ++wk;
+        }
+        const uint32_t c = static_cast<uint32_t>(el[i]) & kCntMask;
+        top = max(top, (c << kElBits) | (kElMask - i));
+        add += c;
+      }
+      if (add) {
+        atomicMax(&best[wk - 1], top);
+        atomicAdd(&hits[wk - 1], add);
       }
     }
     __syncthreads();
-    for (uint32_t j = tid; j < nwin; j += T) best[j] = el[0xffffffffu - static_cast<uint32_t>(best[j])] >> kCntBits;
-    uint32_t kept = nwin;
-    __syncthreads();
-    if (a.max_cands && nwin > a.max_cands) {
-      // keep the max_cands windows with most hits (ties: smaller key), in key order
-      kept = a.max_cands;
-      const uint32_t P2 = pow2_at_least(nwin);
-      for (uint32_t i = tid; i < P2; i += T)
-        el[i] = i < nwin ? (static_cast<uint64_t>(0xffffffffu - (pre[wst[i + 1]] - pre[wst[i]])) << 32) | i : kNone;
+    const bool cut = a.max_cands && nwin > a.max_cands;
+    if (cut && nwin > kCutWindows) {
+      if (tid == 0) {
+        a.list_rest[atomicAdd(&a.plan->n_rest, 1u)] = rr;
+        a.nwin[rr] = 0;
+      }
       __syncthreads();
-      bitonic(el, P2);
-      for (uint32_t i = tid; i < P2; i += T) el[i] = i < kept ? (el[i] & 0xffffffffull) : kNone;
-      __syncthreads();
-      bitonic(el, P2);
+      continue;
     }
+    const uint32_t kept = cut ? a.max_cands : nwin;
     if (tid == 0) {
       s_slot = atomicAdd(&a.plan->cursor, static_cast<unsigned long long>(kept));
       a.wslot[rr] = static_cast<uint32_t>(s_slot);
       a.nwin[rr] = kept;
     }
     __syncthreads();
-    if (s_slot + kept <= a.win_cap) {
-      for (uint32_t i = tid; i < kept; i += T) {
-        const uint32_t j = kept < nwin ? static_cast<uint32_t>(el[i]) : i;
-        a.win[s_slot + i] = find_window(a, best[j], m, pre[wst[j + 1]] - pre[wst[j]]);
+    const bool room = s_slot + kept <= a.win_cap;
+    uint32_t before = 0;
+    for (uint32_t j0 = 0; j0 < nwin; j0 += T) {
+      const uint32_t j = j0 + tid;
+      uint32_t at = j;
+      bool keep = j < nwin;
+      if (cut) {
+        // the max_cands windows of most hits, the smaller key of equal ones, in key order
+        if (keep) {
+          uint32_t rank = 0;
+          const uint32_t h = hits[j];
+          for (uint32_t q2 = 0; q2 < nwin; ++q2) rank += (hits[q2] > h || (hits[q2] == h && q2 < j)) ? 1u : 0u;
+          keep = rank < a.max_cands;
+        }
+        at = before + static_cast<uint32_t>(block_exscan(keep ? 1u : 0u, &tot));
+        before += static_cast<uint32_t>(tot);
       }
+      if (keep && room) a.win[s_slot + at] = find_window(a, el[kElMask - (best[j] & kElMask)] >> kCntBits, m, hits[j]);
     }
     __syncthreads();
   }
@@ -624,9 +648,10 @@ __global__ void k_rest_stage(FindList l, const uint32_t* list, uint32_t n, uint6
   }
 }
 
-constexpr int kMidS = 1024, kMidT = 128, kWideS = 8192, kWideT = 1024;
-using MidSpace = BlockSpace<kMidS, kMidT>;
-using WideSpace = BlockSpace<kWideS, kWideT>;
+constexpr int kMidS = 1024, kMidT = 128, kWideS = 16384, kWideT = 1024;
+constexpr uint32_t kMidEntries = 16384, kWideEntries = 0xffffffffu;
+using MidSpace = BlockSpace<kMidS, kMidT, kMidEntries>;
+using WideSpace = BlockSpace<kWideS, kWideT, kWideEntries>;
 
 }  // namespace
 
@@ -639,7 +664,7 @@ int launch_find(const FindArgs& a, cudaStream_t st) {
   if (a.nr == 0) return 0;
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(k_find_block<kWideS, kWideT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_find_block<kWideS, kWideT, kWideEntries>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(WideSpace::kBytes)) != cudaSuccess)
       return -1;
     attr = true;
@@ -652,9 +677,9 @@ int launch_find(const FindArgs& a, cudaStream_t st) {
     return need < most ? need : most;
   };
   k_find_warp<<<grid(kFindWarps, 40), 32 * kFindWarps, 0, st>>>(a);
-  k_find_block<kMidS, kMidT><<<grid(1, 9), kMidT, MidSpace::kBytes, st>>>(a, a.list_mid, &a.plan->n_mid, &a.plan->q_mid,
+  k_find_block<kMidS, kMidT, kMidEntries><<<grid(1, 10), kMidT, MidSpace::kBytes, st>>>(a, a.list_mid, &a.plan->n_mid, &a.plan->q_mid,
                                                                          a.list_wide, &a.plan->n_wide);
-  k_find_block<kWideS, kWideT><<<grid(1, 1), kWideT, WideSpace::kBytes, st>>>(a, a.list_wide, &a.plan->n_wide,
+  k_find_block<kWideS, kWideT, kWideEntries><<<grid(1, 1), kWideT, WideSpace::kBytes, st>>>(a, a.list_wide, &a.plan->n_wide,
                                                                              &a.plan->q_wide, a.list_rest, &a.plan->n_rest);
   return cudaPeekAtLastError() == cudaSuccess ? 3 : -1;
 }
@@ -686,8 +711,8 @@ int preload_find() {
   int n_ = 0;
   SR_TOUCH(k_find_check);
   SR_TOUCH(k_find_warp);
-  SR_TOUCH((k_find_block<kMidS, kMidT>));
-  SR_TOUCH((k_find_block<kWideS, kWideT>));
+  SR_TOUCH((k_find_block<kMidS, kMidT, kMidEntries>));
+  SR_TOUCH((k_find_block<kWideS, kWideT, kWideEntries>));
   SR_TOUCH(k_find_out);
   SR_TOUCH(k_rest_len);
   SR_TOUCH(k_rest_bases);

@@ -1,6 +1,6 @@
 """The one-pass CAL finder's paths (warp, block tables, large reads) against the
 host stage, at the edges of each: distinct CALs around what a warp (128 runs, 64
-ranks), the two tables (768, 6144) and the large-read path take, every index form,
+ranks), the two tables (768, 12288) and the large-read path take, every index form,
 seeds that are their own reverse complement, and CALs off the reference's ends."""
 import numpy as np
 import pytest
@@ -42,8 +42,8 @@ PRMS = [dict(merge_dist=32, pad=32), dict(merge_dist=0, pad=4), dict(merge_dist=
         dict(seed_stride=7, merge_dist=200, pad=0, max_cands=1)]
 
 
-@pytest.mark.parametrize("unit,copies", [(29, 62), (29, 65), (37, 127), (37, 130), (23, 760), (23, 770), (11, 6130),
-                                         (11, 6150)])
+@pytest.mark.parametrize("unit,copies", [(29, 62), (29, 65), (37, 127), (37, 130), (23, 760), (23, 770), (13, 6150),
+                                         (7, 12150), (7, 12300)])
 def test_distinct_cals_around_each_table(sr, unit, copies):
     """Reads inside, across the ends of and outside a tandem repeat: one inside
     has about one distinct CAL per copy (counted with merge_dist 0)."""
