@@ -3,6 +3,7 @@
 // classification (Sec. 6.1-6.4) and CIGAR compaction.
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <algorithm>
 
 #include "sr_internal.h"
 
@@ -88,16 +89,17 @@ __global__ void k_pack_reads(const char* bases, const uint64_t* off, uint32_t n_
   if (bad) atomicOr(status, kStBadBase);
 }
 
-// eight lanes per read: item -> read map and window validation
+// G lanes per read: item -> read map and window validation
+template <int G>
 __global__ void k_items(const uint64_t* cand_off, uint32_t n_reads, const uint8_t* c_ref,
                         const uint8_t* c_strand, const uint64_t* c_start, const uint32_t* c_len,
                         DevRefs refs, uint32_t* item_read, uint32_t* status) {
-  const uint64_t r = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) >> 3;
-  const int lane = threadIdx.x & 7;
+  const uint64_t r = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) / G;
+  const int lane = threadIdx.x & (G - 1);
   if (r >= n_reads) return;
   const uint64_t c0 = cand_off[r], c1 = cand_off[r + 1];
   bool bad = c1 < c0;
-  for (uint64_t c = c0 + lane; c < c1 && !bad; c += 8) {
+  for (uint64_t c = c0 + lane; c < c1 && !bad; c += G) {
     item_read[c] = static_cast<uint32_t>(r);
     const uint32_t k = c_ref[c];
     const uint32_t n = c_len[c];
@@ -134,7 +136,7 @@ __global__ void k_keys(const uint32_t* item_read, const uint32_t* rlen, const ui
 
 // one block: exclusive scan of the histogram -> cursor, class ranges.  A serial
 // step between two launches whatever the batch's size, so it is made of warp scans
-// with two barriers (10.3 us with a barrier per doubling step, XXX us so)
+// with two barriers (10.3 us with a barrier per doubling step, 4.5 us so)
 __global__ void __launch_bounds__(1024) k_scan_keys(const uint32_t* hist, uint32_t* cursor, uint32_t* class_range) {
   __shared__ uint32_t warp_sum[32];
   constexpr int per = kNumKeys / 1024;
@@ -446,13 +448,20 @@ int launch_pack_refs(const char* ascii, uint64_t len, uint32_t* words, uint32_t*
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
+// Lanes per read of the kernels that walk a read's windows once: one where reads
+// hold one or two windows on average, eight where they hold more (a read may have
+// hundreds).
+bool few_windows(const BatchDev& b) { return b.n_items <= 2ull * b.n_reads; }
+
 int launch_prepare(const BatchDev& b, const DevRefs& refs, cudaStream_t st) {
   if (b.n_reads == 0) return 0;
   const uint64_t t = static_cast<uint64_t>(b.n_reads) * 16;
   k_pack_reads<<<static_cast<unsigned>((t + 255) / 256), 256, 0, st>>>(
       b.bases, b.read_off, b.n_reads, b.rpack, b.rlen, b.status);
-  const uint64_t tw = static_cast<uint64_t>(b.n_reads) * 8;
-  k_items<<<static_cast<unsigned>((tw + 255) / 256), 256, 0, st>>>(
+  const bool few = few_windows(b);
+  const uint64_t tw = static_cast<uint64_t>(b.n_reads) * (few ? 1 : 8);
+  auto* items = few ? k_items<1> : k_items<8>;
+  items<<<static_cast<unsigned>((tw + 255) / 256), 256, 0, st>>>(
       b.cand_off, b.n_reads, b.c_ref, b.c_strand, b.c_start, b.c_len, refs, b.item_read, b.status);
   return cudaPeekAtLastError() == cudaSuccess ? 2 : -1;
 }
@@ -579,6 +588,7 @@ int launch_assemble(const BatchDev& b, int n_refs, bool want_cigar, int32_t item
 // host): per read, its offsets, length, window
 // count and windows; the first bad read (lowest index) with the reason, and for
 // good batches the DP cells, the longest read and the windows per read length.
+template <int G>
 __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off, uint32_t n, uint64_t nc,
                               const uint8_t* c_ref, const uint8_t* c_strand, const uint64_t* c_start,
                               const uint32_t* c_len, DevRefs refs, StageCheck* out) {
@@ -591,12 +601,14 @@ __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off
     longest = 0;
   }
   __syncthreads();
-  // eight lanes per read: a read may have hundreds of windows
-  const uint64_t r64 = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) >> 3;
-  const uint32_t r = static_cast<uint32_t>(r64), lane = threadIdx.x & 7u;
+  // G lanes per read; the blocks stride over the reads, so that the histogram is
+  // cleared and handed on once per block and not once per 256 / G reads
+  const uint32_t lane = threadIdx.x & (G - 1);
+  const uint64_t step = static_cast<uint64_t>(gridDim.x) * blockDim.x / G;
   unsigned long long cells = 0;
-  uint32_t why = 0;
-  if (r64 < n) {
+  uint32_t top = 0;
+  for (uint64_t r = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) / G; r < n; r += step) {
+    uint32_t why = 0;
     const uint64_t a0 = read_off[r], a1 = read_off[r + 1], c0 = cand_off[r], c1 = cand_off[r + 1];
     if (a1 < a0 || c1 < c0 || c1 > nc) why = 1;
     else if (a1 - a0 == 0 || a1 - a0 > static_cast<uint64_t>(kMaxReadLen)) why = 2;
@@ -604,7 +616,7 @@ __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off
     if (!why) {
       const uint64_t m = a1 - a0;
       uint64_t suml = 0;
-      for (uint64_t k = c0 + lane; k < c1; k += 8) {
+      for (uint64_t k = c0 + lane; k < c1; k += G) {
         const uint32_t ref = c_ref[k], len = c_len[k];
         const uint64_t w0 = c_start[k];
         const bool ok = ref < static_cast<uint32_t>(refs.n) && c_strand[k] <= 1 && len >= 1 &&
@@ -612,14 +624,16 @@ __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off
         if (!ok) why = 4;
         suml += len;
       }
-      cells = m * suml;
+      cells += m * suml;
       if (lane == 0) {
         if (c1 > c0) atomicAdd(&hist[m], static_cast<uint32_t>(c1 - c0));
-        atomicMax(&longest, static_cast<uint32_t>(m));
+        top = max(top, static_cast<uint32_t>(m));
       }
     }
     if (why) atomicMin(&out->bad, (static_cast<unsigned long long>(r) << 3) | why);
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0 && top) atomicMax(&longest, top);
   for (int o = 16; o; o >>= 1) cells += __shfl_xor_sync(0xffffffffu, cells, o);
   if ((threadIdx.x & 31) == 0 && cells) atomicAdd(&cells_sh, cells);
   __syncthreads();
@@ -646,8 +660,12 @@ int launch_stage_check(const BatchDev& b, const DevRefs& refs, StageCheck* out, 
   if (cudaMemsetAsync(out, 0, sizeof(StageCheck), st) != cudaSuccess) return -1;
   if (cudaMemsetAsync(&out->bad, 0xff, 2 * sizeof(unsigned long long), st) != cudaSuccess) return -1;
   if (b.n_reads == 0) return 0;
-  k_stage_check<<<static_cast<unsigned>((b.n_reads * 8ull + 255) / 256), 256, 0, st>>>(b.read_off, b.cand_off, b.n_reads, b.n_items, b.c_ref,
-                                                         b.c_strand, b.c_start, b.c_len, refs, out);
+  // at most one block per resident slot (eight of 256 threads on each SM)
+  const bool few = few_windows(b);
+  const uint64_t blocks = std::min<uint64_t>((b.n_reads * (few ? 1ull : 8ull) + 255) / 256, 152ull * 8);
+  auto* kern = few ? k_stage_check<1> : k_stage_check<8>;
+  kern<<<static_cast<unsigned>(blocks), 256, 0, st>>>(b.read_off, b.cand_off, b.n_reads, b.n_items, b.c_ref, b.c_strand,
+                                                      b.c_start, b.c_len, refs, out);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -704,7 +722,8 @@ int preload_kernels() {
   int n_ = 0;
   SR_TOUCH(k_pack_ref);
   SR_TOUCH(k_pack_reads);
-  SR_TOUCH(k_items);
+  SR_TOUCH(k_items<1>);
+  SR_TOUCH(k_items<8>);
   SR_TOUCH(k_keys);
   SR_TOUCH(k_scan_keys);
   SR_TOUCH(k_scatter);
@@ -719,7 +738,8 @@ int preload_kernels() {
   SR_TOUCH(k_scan_sums);
   SR_TOUCH(k_cigar_gather);
   SR_TOUCH(k_assemble);
-  SR_TOUCH(k_stage_check);
+  SR_TOUCH(k_stage_check<1>);
+  SR_TOUCH(k_stage_check<8>);
   SR_TOUCH(k_first_bad_window);
   SR_TOUCH(k_rebase_offsets);
   return n_;

@@ -53,3 +53,37 @@ def test_few_and_many_windows_are_refused_alike(kind):
     g = gpu_run(s, w)
     assert np.array_equal(g["item_score"], oracle_run(w)["item_score"])
     assert g["cells"] == int(np.sum(np.repeat(np.diff(w["read_off"]), np.diff(w["cand_off"])) * w["c_len"].astype(np.int64)))
+
+
+@pytest.mark.parametrize("reads,windows", [(9000, 1), (320_001, 1), (160_001, 2), (40_001, 3)])
+def test_more_reads_than_resident_groups(reads, windows):
+    """One lane per read up to two windows on average, eight above; the blocks stride
+    over the reads past 311,296 (38,912) of them.  Every read counts, the last too."""
+    from paper_1805_00106_gb300 import sr
+    ref = S.ref_iid(20_000, 3)
+    s = sr.Session.open([bytes(ref)])
+    rd = S.reads([ref], reads, 5, 20, 24)
+    w = dict(refs=[ref], **rd, **S.cands(rd, [len(ref)], 6, S.COUNT_FIXED, windows, 4))
+    args = [w[k] for k in ("bases", "read_off", "cand_off", "c_ref", "c_strand", "c_start", "c_len")]
+    cells = int(np.sum(np.repeat(np.diff(w["read_off"]), windows) * w["c_len"].astype(np.int64)))
+    g = gpu_run(s, w)
+    assert g["cells"] == cells
+    k = np.r_[0:200, reads - 200:reads]
+    want = oracle_run(_reads(w, k))["item_score"]
+    got = np.concatenate([g["item_score"][w["cand_off"][i]:w["cand_off"][i + 1]] for i in k])
+    assert np.array_equal(got, want)
+    args[6] = args[6].copy()
+    args[6][-1] = 0
+    with pytest.raises(sr.SrError) as e:
+        s.align(*args)
+    assert e.value.status == sr.SR_EINVAL and str(len(args[6]) - 1) in str(e.value)
+
+
+def _reads(w, k):
+    """the reads k of a workload, with their windows"""
+    ro, co = w["read_off"], w["cand_off"]
+    items = np.concatenate([np.arange(co[i], co[i + 1]) for i in k])
+    return dict(refs=w["refs"], bases=np.concatenate([w["bases"][ro[i]:ro[i + 1]] for i in k]),
+                read_off=np.r_[0, np.cumsum([ro[i + 1] - ro[i] for i in k])].astype(np.uint64),
+                cand_off=np.r_[0, np.cumsum([co[i + 1] - co[i] for i in k])].astype(np.uint64),
+                **{x: np.ascontiguousarray(w[x][items]) for x in ("c_ref", "c_strand", "c_start", "c_len")})
