@@ -103,13 +103,16 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
                       : dispatch_mode0(false, g, r, a, st, tasks);
     return k < 0 ? -1 : k;
   }
-  // Few pairs: all classes in one launch (extension phase, us, one kernel per
-  // class / one launch on 16 lanes / on 32).  Reads of 75-250 bases in 23 classes:
-  // 270 pairs 217 / 76 / 48, 3000 218 / 131 / 119, 6000 218 / 205 / 162, 12,000
-  // 281 / 264 / 258, 24,000 410 / 422 / 469, 48,000 702 / 780 / 895; of 100 bases
-  // in one class: 3000 pairs 45 / 43 / 47, 6000 59 / 61 / 78, 24,000 162 / 194 /
-  // 264.  So one launch up to 12k pairs; on 32 lanes up to 8k pairs, or 2k of reads
-  // that 32 lanes x 4 rows (128) pad.
+  // Few pairs: all classes in one launch on 32 lanes per pair, which spares the
+  // latency of a class's kernel and the queue of many of them; once the pairs fill
+  // the chip the kernels per class do less work per cell.  Extension phase (us),
+  // kernel per class / one launch: reads of 75-250 bases (23 classes) 900 pairs 201 /
+  // 55, 3000 203 / 117, 6000 203 / 156, 9000 232 / 206, 12,000 252 / 254, 24,000 382
+  // / 467; of 200-250 (7 classes) 3000 132 / 111, 6000 173 / 190; of 250 bases 900 96
+  // / 53, 3000 135 / 110, 6000 192 / 204; of 100 bases 900 30 / 26, 3000 40 / 45,
+  // 6000 53 / 81; of 64 3000 30 / 43.  So up to 4096 pairs and 256 for each class,
+  // or 2048 of reads that 32 lanes x 4 rows (128) pad.  (16 lanes per pair were
+  // never the fastest by more than 4 us near these lines.)
   // Score sets whose biased scores may be negative (!ext_nonneg) always take it:
   // their form of the recurrence is built for it alone.
   uint64_t pairs = 0;
@@ -121,13 +124,12 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
     pairs += (class_items[c] + 1) / 2;
     if (class_items[c]) longest = upper[c];
   }
-  const bool one = !ext_nonneg(a) || (!lanes && pairs <= 12288);
+  const bool one = !ext_nonneg(a) || (!lanes && pairs <= (longest > 128 ? 4096u + 256u * present : 2048u));
   cudaStream_t s32 = st;  // the int32 class's stream
   if (one) {
-    const uint32_t g = pairs <= (longest > 128 ? 8192u : 2048u) ? 32 : 16;
     const int k = pairs == 0  ? 0
-                  : mode == 1 ? dispatch_all1(g, a, upper, pairs, st)
-                              : dispatch_all0(g, a, upper, pairs, st);
+                  : mode == 1 ? dispatch_all1(a, upper, pairs, st)
+                              : dispatch_all0(a, upper, pairs, st);
     if (k < 0) return -1;
     launched += k;
   } else {

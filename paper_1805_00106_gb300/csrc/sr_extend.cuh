@@ -95,8 +95,8 @@ int dispatch_mode1(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a
 int dispatch_mode2(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st);
 // every length class (at most upper[c] bases in class c) in one launch on 16 or
 // 32 lanes per pair (16 when !ext_nonneg), `pairs` item pairs in all
-int dispatch_all0(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
-int dispatch_all1(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
+int dispatch_all0(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
+int dispatch_all1(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
 
 namespace {
 
@@ -586,8 +586,10 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
 // its queue is empty, then the next class's, each with the fewest rows per lane
 // that hold it (rows[c]: the class's reads have at most G * rows[c] bases).  One
 // kernel per class (k_extend16 on 8 lanes) does less work per cell, but a pair on
-// 8 lanes x 31 rows takes 0.15 ms however few there are, 23 classes queue up on
-// eight streams, and each ends in a tail of its own.  Bound by the ALU pipe once
+// 8 lanes x 32 rows takes 0.09 ms however few there are (0.04 on 32 lanes x 8), 23
+// classes queue up on eight streams, and each ends in a tail of its own.  32 lanes
+// per pair; 16 for the score sets whose biased scores may be negative, which take
+// it for batches of any size.  Bound by the ALU pipe once
 // its warps fill the chip, before that by the rows' chains of one pair.
 struct ExtRows {
   uint8_t r[kNumBins];
@@ -768,12 +770,9 @@ int launch_all(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStre
   constexpr int groups = (kThreads / 32) * (32 / G);
   const size_t smem = sizeof(GroupSmem) * groups;
   auto kern = k_extend_all<G, MODE, NN>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
-      return -1;
-    attr_set = true;
-  }
+  // per device, so set for each launch
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    return -1;
   int dev = 0, nsm = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

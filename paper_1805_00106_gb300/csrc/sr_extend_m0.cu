@@ -21,14 +21,12 @@ int dispatch_mode0(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a
   return -1;
 }
 
-int dispatch_all0(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
-  if (!ext_nonneg(a)) return launch_all<16, 0, false>(a, upper, pairs, st);
-  return lanes == 32 ? launch_all<32, 0, true>(a, upper, pairs, st) : launch_all<16, 0, true>(a, upper, pairs, st);
+int dispatch_all0(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
+  return ext_nonneg(a) ? launch_all<32, 0, true>(a, upper, pairs, st) : launch_all<16, 0, false>(a, upper, pairs, st);
 }
 
 int preload_mode0() {
   int n_ = 0;
-  SR_TOUCH((k_extend_all<16, 0, true>));
   SR_TOUCH((k_extend_all<32, 0, true>));
   SR_TOUCH((k_extend_all<16, 0, false>));
   SR_TOUCH((k_extend16<16, 16, 0, false, false>));

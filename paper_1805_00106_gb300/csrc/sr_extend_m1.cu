@@ -21,14 +21,12 @@ int dispatch_mode1(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a
   return -1;
 }
 
-int dispatch_all1(uint32_t lanes, const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
-  if (!ext_nonneg(a)) return launch_all<16, 1, false>(a, upper, pairs, st);
-  return lanes == 32 ? launch_all<32, 1, true>(a, upper, pairs, st) : launch_all<16, 1, true>(a, upper, pairs, st);
+int dispatch_all1(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
+  return ext_nonneg(a) ? launch_all<32, 1, true>(a, upper, pairs, st) : launch_all<16, 1, false>(a, upper, pairs, st);
 }
 
 int preload_mode1() {
   int n_ = 0;
-  SR_TOUCH((k_extend_all<16, 1, true>));
   SR_TOUCH((k_extend_all<32, 1, true>));
   SR_TOUCH((k_extend_all<16, 1, false>));
   SR_TOUCH((k_extend16<16, 16, 1, false, false>));

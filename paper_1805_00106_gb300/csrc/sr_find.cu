@@ -662,13 +662,10 @@ int launch_find_check(const uint64_t* read_off, uint32_t n, uint32_t* status, cu
 
 int launch_find(const FindArgs& a, cudaStream_t st) {
   if (a.nr == 0) return 0;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_find_block<kWideS, kWideT, kWideEntries>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(WideSpace::kBytes)) != cudaSuccess)
-      return -1;
-    attr = true;
-  }
+  // per device, so set for each launch
+  if (cudaFuncSetAttribute(k_find_block<kWideS, kWideT, kWideEntries>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(WideSpace::kBytes)) != cudaSuccess)
+    return -1;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

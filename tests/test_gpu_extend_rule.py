@@ -1,5 +1,5 @@
 """How a batch's item pairs are spread over the chip is chosen by their number
-and classes (every class in one launch on 32 or 16 lanes, or a kernel per class):
+and classes (every class in one launch, or a kernel per class):
 on both sides of each line the scores are those of one forced shape, in both
 readouts, and a small batch's those of the oracle."""
 import numpy as np
@@ -52,9 +52,9 @@ def test_every_row_count_against_the_oracle(sr, mode):
              c_len=np.array(lens) + 60)
     s = sr.Session.open([bytes(ref)])
     o = oracle_run(w, mode=mode)
-    few = gpu_run(s, w, mode=mode)  # 32 lanes
+    few = gpu_run(s, w, mode=mode)  # one launch
     assert not compare(few, o)
-    t = 400  # 9400 pairs in 23 classes: 16 lanes
+    t = 400  # many pairs in 23 classes
     many = dict(w, bases=np.tile(w["bases"], t), read_off=np.concatenate([[0], np.cumsum(np.tile(lens, t))]),
                 cand_off=np.arange(t * len(lens) + 1), **{k: np.tile(w[k], t) for k in ("c_ref", "c_strand", "c_start", "c_len")})
     got = gpu_run(s, many, mode=mode)
@@ -86,3 +86,33 @@ def test_score_sets_on_both_sides_of_the_nonnegative_line(sr, mode, sp, reads):
     g = gpu_run(s, many, sp=sp, mode=mode)
     assert np.array_equal(g["item_score"], np.tile(o["item_score"], t))
     assert np.array_equal(g["item_end"].astype(np.int64), np.tile(o["item_end_j"], t).astype(np.int64))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("reads,lo,hi", [(512, 1, 128), (513, 1, 128), (1088, 250, 250), (1089, 250, 250), (2048, 129, 256),
+                                         (2049, 129, 256)])
+def test_both_sides_of_the_one_launch_line(sr, mode, reads, lo, hi):
+    """2048 pairs of reads up to 128 bases; 4096 and 256 for each class of longer ones."""
+    w = _batch(reads, lo, hi, 8)
+    assert len(w["c_ref"]) // 2 in (2048, 2052, 4352, 4356, 8192, 8196)
+    s = sr.Session.open([bytes(r) for r in w["refs"]])
+    a, b = gpu_run(s, w, mode=mode), gpu_run(s, w, mode=mode, lanes=32, rows=8)
+    for k in ("item_score", "item_end", "best", "cigar"):
+        assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_every_row_count_on_16_lanes(sr, mode):
+    """A score set with mismatch > go + ge: reads at the edges of 16 lanes' rows."""
+    lens = np.array(sorted({m for r in range(1, 17) for m in (16 * r - 1, 16 * r, 16 * r + 1) if m <= 256}))
+    ref = S.ref_iid(60_000, 23)
+    rng = np.random.default_rng(4)
+    pos = rng.integers(100, 59_000, len(lens))
+    parts = [ref[p: p + m].copy() for p, m in zip(pos, lens)]
+    for x in parts:
+        x[rng.random(len(x)) < 0.03] = ord("C")
+    w = dict(refs=[ref], bases=np.concatenate(parts), read_off=np.concatenate([[0], np.cumsum(lens)]),
+             cand_off=np.arange(len(lens) + 1), c_ref=np.zeros(len(lens), np.uint8),
+             c_strand=np.zeros(len(lens), np.uint8), c_start=pos - 30, c_len=lens + 60)
+    s = sr.Session.open([bytes(ref)])
+    assert not compare(gpu_run(s, w, sp=(2, 8, 5, 2), mode=mode), oracle_run(w, sp=(2, 8, 5, 2), mode=mode))
