@@ -34,7 +34,10 @@ RC_FRAC = 0.5  # reads drawn from the reverse strand (aligned through their '-' 
 ENGINE = "batched (length bins, LPT persistent kernels, one CUDA graph)"
 SP = (2, 3, 5, 2)
 METRIC = "SW GCUPS (whole path: pack, bins, extension, select, traceback)"
-OPS_PER_CELL = 3  # packed 16-bit ops per cell of the score-only recurrence (6 per s16x2 pair)
+# packed 16-bit ops per cell of the textbook score-only recurrence (6 per s16x2 pair:
+# a score pick, four DPX, half of two maxima): a fixed yardstick, so that figures
+# compare across builds.  k_extend16 takes 4.5 of the ALU pipe's slots per pair.
+OPS_PER_CELL = 3
 
 
 def parse():
@@ -705,7 +708,7 @@ def main():
                 "kernel": "k_extend16 (all length bins) + k_extend32",
                 "peak_basis": f"{n_sm} SMs x {f_mhz:.0f} MHz (median under load) x "
                               f"{dpx_rate:.1f} packed-16-bit DPX lane-ops/clk/SM (measured) x 2 cells / "
-                              f"{2 * OPS_PER_CELL} ops",
+                              f"{2 * OPS_PER_CELL} ops (a yardstick; the kernel takes 4.5 ALU-pipe slots)",
                 "traceback_ms": round(statistics.mean(tb_ms), 3),
                 "extension_ms": round(1e3 * ext, 3)}
 
