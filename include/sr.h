@@ -237,21 +237,23 @@ void sr_session_close(sr_session* s);
  * each reference's tables are copied as they are (9 bytes per entry and 8 per
  * bucket).  A packed copy of one or two references with at most 2^26 buckets and
  * at most 13 (16-bit keys) or 8 (32-bit keys) entries per bucket on average also
- * gets 64-byte bucket heads (both references' starts and counts and up to 26 or
- * 13 keys, built on the device; left out if they cannot be allocated, or with
- * SR_CAL_HEADS=0 in the environment).
+ * gets bucket heads (both references' starts and counts and the first keys: 32
+ * bytes with 11 or 5 keys where buckets hold at most 4 or 2 entries on average,
+ * else 64 bytes with 27 or 13; built on the device; left out if they cannot be
+ * allocated, or with SR_CAL_HEADS=0 in the environment).
  * sr_candidates_device then returns exactly the list
  * sr_candidates returns for those indexes (same windows, order and hits): one
- * warp per read looks up its seeds, one warp or block per read sorts and
- * merges its CALs, and reads of more than 8192 CALs are emitted, sorted and
- * merged by many blocks each.  The reads may be host memory or, flagged SR_FLAG_DEVICE, device
- * memory (read on the session's stream); params->flags = SR_FLAG_DEVICE leaves
+ * warp per read looks up its seeds, counts equal CALs and merges the distinct
+ * ones; reads in repeats take one block each, and those of more than 12288
+ * distinct CALs are emitted, sorted and merged by many blocks each.  The reads
+ * may be host memory or, flagged SR_FLAG_DEVICE, device memory (read on the session's stream); params->flags = SR_FLAG_DEVICE leaves
  * the list in device memory (its arrays device pointers, the list flagged
  * SR_FLAG_DEVICE), so that reads, windows and the alignment stay on the device
- * (sr_align_batch takes such a list as it is).  The call's scratch (kept seed
- * lookups, 8 bytes per seed and reference, up to 1 GiB; CAL keys and window
- * arrays, 24 bytes per CAL bound, up to 64M bounds; a few words per read; for a
- * host list, the list itself, 8 bytes per read and 18 per window, built on the
+ * (sr_align_batch takes such a list as it is; a freed list's block may serve the
+ * session's next one).  The call's scratch (staged windows, 16 bytes each, and a
+ * few words per read; for reads of the many-block path kept seed lookups, 8 bytes
+ * per seed and reference, up to 1 GiB, and CAL keys and window arrays, 24 bytes
+ * per CAL bound, up to 64M bounds; for a host list, the list itself, 8 bytes per read and 18 per window, built on the
  * device and copied out once through a pinned block of the session's pool)
  * stays allocated in the session for the next call and is released by
  * sr_session_close; calls on one session run one at a time.  Reads
