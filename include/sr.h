@@ -279,8 +279,9 @@ sr_status sr_align_batch(sr_session* s, const sr_reads* reads, const sr_cand_lis
                          const sr_score_params* sp, const sr_align_opts* opts, sr_results** out);
 
 /* The same in three steps, so the device part can be timed and repeated with
- * inputs resident in HBM.  stage copies inputs to device buffers (no kernels);
- * run enqueues every kernel of the path on the stream (pack, work list and
+ * inputs resident in HBM.  stage copies inputs to device buffers, checks them
+ * (many windows by a kernel) and returns when they are complete there: the batch
+ * may run on any stream, and the caller's arrays are free; run enqueues every kernel of the path on the stream (pack, work list and
  * bins, extension, per-read selection, traceback, classification) and waits
  * for it; run_async only enqueues (check with sr_batch_sync); fetch copies the
  * results back. */

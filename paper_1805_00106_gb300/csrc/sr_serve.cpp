@@ -245,7 +245,7 @@ sr_batch* stage_round(Server* sv, Round& rd, cudaStream_t stream) {
   cl.win_start = cstart.data();
   cl.win_len = clen.data();
   sr_batch* b = nullptr;
-  rd.status = batch_stage_internal(sv->s, &reads, &cl, stream, false, &b);
+  rd.status = batch_stage_internal(sv->s, &reads, &cl, stream, false, false, &b);  // the round runs on this stream
   return rd.status == SR_OK ? b : nullptr;
 }
 

@@ -690,20 +690,23 @@ sr_status stage_device(sr_session* s, const sr_reads* reads, const sr_cand_list*
 
 extern "C" sr_status sr_batch_stage(sr_session* s, const sr_reads* reads, const sr_cand_list* cands,
                                     void* cuda_stream, sr_batch** out) {
-  return batch_stage_internal(s, reads, cands, cuda_stream, true, out);
+  return batch_stage_internal(s, reads, cands, cuda_stream, true, true, out);
 }
 
 sr_status sr::batch_stage_internal(sr_session* s, const sr_reads* reads, const sr_cand_list* cands,
-                                   void* cuda_stream, bool check_budget, sr_batch** out) {
-  return batch_stage_range(s, reads, cands, 0, reads ? reads->n_reads : 0, cuda_stream, check_budget, out);
+                                   void* cuda_stream, bool check_budget, bool wait, sr_batch** out) {
+  return batch_stage_range(s, reads, cands, 0, reads ? reads->n_reads : 0, cuda_stream, check_budget, wait, out);
 }
 
 // Stages reads [r0, r1) of the caller's arrays (and their windows) as one
 // batch: the whole list's header is checked, the range's arrays are copied and
 // its offsets made batch-relative on the device.  Reads and windows named in
-// error messages keep their indexes in the caller's arrays.
+// error messages keep their indexes in the caller's arrays.  With wait the
+// batch's arrays are complete when this returns, so that it may run on any
+// stream; without, they may still be on their way on the staging stream, and the
+// batch must run on that one (the caller's arrays are free either way).
 sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_cand_list* cands, uint32_t r0,
-                                uint32_t r1, void* cuda_stream, bool check_budget, sr_batch** out) {
+                                uint32_t r1, void* cuda_stream, bool check_budget, bool wait, sr_batch** out) {
   Trace trace_("sr_batch_stage");
   if (!s || !reads || !cands || !out) return set_error(SR_EINVAL, "sr_batch_stage: null argument");
   *out = nullptr;
@@ -836,7 +839,7 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
     max_m = std::max<uint32_t>(max_m, static_cast<uint32_t>(m));
   }
   // the caller may reuse its arrays once this returns
-  if (!gathered) e = cudaStreamSynchronize(st);
+  if (wait || !gathered) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     sr_batch_free(b);
     return cuda_error("sr_batch_stage copy", e);
@@ -2278,7 +2281,7 @@ static sr_status align_in_parts(sr_session* s, const sr_reads* reads, const sr_c
       }
   };
   for (int k = 0; k < kParts; ++k) {
-    sr_status st = batch_stage_range(s, reads, cands, rr[k], rr[k + 1], s->part_stream[k], true, &b[k]);
+    sr_status st = batch_stage_range(s, reads, cands, rr[k], rr[k + 1], s->part_stream[k], true, false, &b[k]);
     if (st == SR_OK) st = batch_run_async(s, b[k], sp, &oo);
     if (st != SR_OK) {
       drop_parts();
@@ -2435,7 +2438,8 @@ extern "C" sr_status sr_align_batch(sr_session* s, const sr_reads* reads, const 
     }
   }
   sr_batch* b = nullptr;
-  sr_status st = sr_batch_stage(s, reads, cands, opts ? opts->cuda_stream : nullptr, &b);
+  // staged and run on one stream
+  sr_status st = batch_stage_internal(s, reads, cands, opts ? opts->cuda_stream : nullptr, true, false, &b);
   if (st != SR_OK) return st;
   st = batch_run_async(s, b, sp, opts);  // the fetch waits, and checks the run's status
   if (st == SR_OK) st = sr_batch_fetch(s, b, out);
@@ -2628,7 +2632,7 @@ extern "C" sr_status sr_tune(sr_session* s, const sr_score_params* sp, uint32_t 
     cl.win_start = cst.data();
     cl.win_len = cln.data();
     sr_batch* b = nullptr;
-    st = batch_stage_internal(s, &rd, &cl, nullptr, false, &b);
+    st = batch_stage_internal(s, &rd, &cl, nullptr, false, true, &b);
     if (st != SR_OK) break;
     float best_ms = 1e30f, cur_ms = -1.0f;
     TuneBin pick = cur[bi];
