@@ -286,8 +286,8 @@ void find_read(const sr_index* const* idx, uint32_t n_refs, const uint8_t* q, in
   const int a = static_cast<int>(idx[0]->p.address_bases);
   const int kb = 2 * (k - a);
   const uint64_t kmask = mask_bits(kb);
-  const int stride = static_cast<int>(cp.seed_stride ? cp.seed_stride : 1);
-  for (int o = 0; o + k <= m; o += stride) {
+  const int64_t stride = cp.seed_stride ? cp.seed_stride : 1;  // any 32-bit value: o does not wrap
+  for (int64_t o = 0; o + k <= m; o += stride) {
     Kmer km;
     for (int t = 0; t < k; ++t) kmer_push(km, q[o + t], k);
     const uint64_t canon = std::min(km.fwd, km.rc);

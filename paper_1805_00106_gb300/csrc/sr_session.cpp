@@ -1881,6 +1881,9 @@ extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, 
   sr_cand_params cp{};
   if (params) cp = *params;
   if (!cp.seed_stride) cp.seed_stride = 1;
+  // past the longest read any stride takes the seed at 0 only; the kernels step
+  // through a read by 32 strides in 32 bits
+  cp.seed_stride = std::min<uint32_t>(cp.seed_stride, SR_MAX_READ_LEN);
   if ((reads->flags | cp.flags) & ~static_cast<uint32_t>(SR_FLAG_DEVICE))
     return set_error(SR_EINVAL, "sr_candidates_device: unknown flags");
   const bool in_dev = (reads->flags & SR_FLAG_DEVICE) != 0, out_dev = (cp.flags & SR_FLAG_DEVICE) != 0;
