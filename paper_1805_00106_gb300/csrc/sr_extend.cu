@@ -113,8 +113,6 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
   // 6000 53 / 81; of 64 3000 30 / 43.  So up to 4096 pairs and 256 for each class,
   // or 2048 of reads that 32 lanes x 4 rows (128) pad.  (16 lanes per pair were
   // never the fastest by more than 4 us near these lines.)
-  // Score sets whose biased scores may be negative (!ext_nonneg) always take it:
-  // their form of the recurrence is built for it alone.
   uint64_t pairs = 0;
   uint32_t upper[kNumBins], longest = 0;
   int present = 0, width = 0;
@@ -124,7 +122,7 @@ int launch_extend(const BatchDev& b, const DevRefs& refs, const ScoreConst& sc,
     pairs += (class_items[c] + 1) / 2;
     if (class_items[c]) longest = upper[c];
   }
-  const bool one = !ext_nonneg(a) || (!lanes && pairs <= (longest > 128 ? 4096u + 256u * present : 2048u));
+  const bool one = !lanes && pairs <= (longest > 128 ? 4096u + 256u * present : 2048u);
   cudaStream_t s32 = st;  // the int32 class's stream
   if (one) {
     const int k = pairs == 0  ? 0

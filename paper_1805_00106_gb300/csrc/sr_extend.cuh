@@ -30,7 +30,8 @@
 // where add-max for E and for the diagonal and a maximum with the floor took four
 // DPX and one add.  Extension phase: 900k windows of 139-314 columns 6.02 to 5.61
 // ms, 201k of 314 2.66 to 2.47 ms, 240k of 183 in final-row mode 1.11 to 1.00 ms.
-// Score sets with mismatch > go + ge keep the four-DPX form (NN false).
+// Score sets with mismatch > go + ge (linear gaps, for one) keep the four-DPX form
+// (NN false), built for the same shapes.
 //
 // The best cell: per lane, the max over its rows of each column is compared
 // with the running best; a strict improvement records the column, so the
@@ -87,14 +88,18 @@ inline bool ext_nonneg(const ExtArgs& a) { return a.sb <= a.go + a.ge; }
       X(16, 14) X(16, 15) X(16, 16) X(32, 4) X(32, 5) X(32, 6) X(32, 7) X(32, 8)
 #define SR_PLAIN_SHAPES(X) X(16, 16) X(32, 8)
 
-// launch the int16 kernel of one shape and readout mode; -1 if the shape is not built
+// launch the int16 kernel of one shape and readout mode; -1 if the shape is not
+// built (neg: the persistent kernels of score sets that are not ext_nonneg)
 int dispatch_mode0(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st,
                    uint64_t tasks);
 int dispatch_mode1(bool persist, uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st,
                    uint64_t tasks);
 int dispatch_mode2(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st);
-// every length class (at most upper[c] bases in class c) in one launch on 16 or
-// 32 lanes per pair (16 when !ext_nonneg), `pairs` item pairs in all
+int dispatch_neg0(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st, uint64_t tasks);
+int dispatch_neg1(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st, uint64_t tasks);
+int dispatch_neg2(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st);
+// every length class (at most upper[c] bases in class c) in one launch on 32 lanes
+// per pair, `pairs` item pairs in all
 int dispatch_all0(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
 int dispatch_all1(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st);
 
@@ -473,8 +478,9 @@ __device__ __forceinline__ bool ext_tasks(const ExtArgs& a, int cls, uint32_t& p
     // Four (rows <= 16) or three columns per pass: the loop's own instructions are
     // shared, and the code of eight classes' kernels still fits the instruction
     // cache side by side.  33,000 pairs in 23 classes / 450,000: 473 / 5605 us; four
-    // columns for every row count 574 / 5583, two 482 / 5700, one 512 / 6040.
-#pragma unroll (R <= 16 ? 4 : 3)
+    // columns for every row count 574 / 5583, two 482 / 5700, one 512 / 6040.  The
+    // four-DPX form spills less with four (300k windows of 250 bases 3914 us, 3986 with three).
+#pragma unroll (R <= 16 || !NN ? 4 : 3)
     for (int s = 0; s < nsteps; ++s) {
       // lane 0's row above is the top border (H = 0, F = -inf): tin = fin = INIT
       const uint32_t tin = imad(__shfl_up_sync(FULL, Tbot, 1, G) - INIT, nz, INIT);
@@ -576,7 +582,7 @@ __device__ __forceinline__ bool ext_tasks(const ExtArgs& a, int cls, uint32_t& p
 }
 
 // NN: mismatch <= go + ge (ext_nonneg)
-template <int G, int R, int MODE, bool PERSIST, bool NN = true>
+template <int G, int R, int MODE, bool PERSIST, bool NN>
 __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_extend16(ExtArgs a) {
   uint32_t phase = 0;
   ext_tasks<G, R, MODE, PERSIST, true, NN>(a, a.cls, phase);
@@ -584,45 +590,32 @@ __global__ void __launch_bounds__(128, ext_min_blocks<R, MODE, PERSIST>()) k_ext
 
 // Every length class in one launch: a warp takes the longest class's pairs until
 // its queue is empty, then the next class's, each with the fewest rows per lane
-// that hold it (rows[c]: the class's reads have at most G * rows[c] bases).  One
+// that hold it (rows[c]: the class's reads have at most 32 * rows[c] bases).  One
 // kernel per class (k_extend16 on 8 lanes) does less work per cell, but a pair on
 // 8 lanes x 32 rows takes 0.09 ms however few there are (0.04 on 32 lanes x 8), 23
-// classes queue up on eight streams, and each ends in a tail of its own.  32 lanes
-// per pair; 16 for the score sets whose biased scores may be negative, which take
-// it for batches of any size.  Bound by the ALU pipe once
-// its warps fill the chip, before that by the rows' chains of one pair.
+// classes queue up on eight streams, and each ends in a tail of its own.  Bound by
+// the ALU pipe once its warps fill the chip, before that by the rows' chains of one
+// pair.
 struct ExtRows {
   uint8_t r[kNumBins];
 };
-template <int G, int MODE, bool NN>
-__global__ void __launch_bounds__(128, G == 32 ? 6 : MODE == 1 ? 4 : 5) k_extend_all(ExtArgs a, ExtRows rows) {
-  static_assert(G == 16 || G == 32, "16 or 32 lanes per pair");
+template <int MODE, bool NN>
+__global__ void __launch_bounds__(128, 6) k_extend_all(ExtArgs a, ExtRows rows) {
   {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31;
-    ext_init<G>(reinterpret_cast<GroupSmem*>(smem_raw) + ((threadIdx.x >> 5) * (32 / G) + lane / G), lane & (G - 1));
+    ext_init<32>(reinterpret_cast<GroupSmem*>(smem_raw) + (threadIdx.x >> 5), threadIdx.x & 31);
   }
   uint32_t phase = 0;
   for (int c = kNumBins - 1; c >= 0; --c) {
     if (a.class_range[2 * c] == a.class_range[2 * c + 1]) continue;
     bool ok = true;
-#define SR_ROWS(g, n)                                         \
-  case n:                                                     \
-    ok = ext_tasks<g, n, MODE, true, false, NN>(a, c, phase); \
-    break;
-    if constexpr (G == 32) {
-      switch (rows.r[c]) {
-        SR_ROWS(32, 4) SR_ROWS(32, 5) SR_ROWS(32, 6) SR_ROWS(32, 7)
-        default: ok = ext_tasks<32, 8, MODE, true, false, NN>(a, c, phase);
-      }
-    } else {
-      switch (rows.r[c]) {
-        SR_ROWS(16, 5) SR_ROWS(16, 6) SR_ROWS(16, 7) SR_ROWS(16, 8) SR_ROWS(16, 9) SR_ROWS(16, 10)
-        SR_ROWS(16, 11) SR_ROWS(16, 12) SR_ROWS(16, 13) SR_ROWS(16, 14) SR_ROWS(16, 15)
-        default: ok = ext_tasks<16, 16, MODE, true, false, NN>(a, c, phase);
-      }
+    switch (rows.r[c]) {
+      case 4: ok = ext_tasks<32, 4, MODE, true, false, NN>(a, c, phase); break;
+      case 5: ok = ext_tasks<32, 5, MODE, true, false, NN>(a, c, phase); break;
+      case 6: ok = ext_tasks<32, 6, MODE, true, false, NN>(a, c, phase); break;
+      case 7: ok = ext_tasks<32, 7, MODE, true, false, NN>(a, c, phase); break;
+      default: ok = ext_tasks<32, 8, MODE, true, false, NN>(a, c, phase);
     }
-#undef SR_ROWS
     if (!ok) return;
   }
 }
@@ -730,7 +723,7 @@ __global__ void __launch_bounds__(128) k_extend32(ExtArgs a) {
 
 // tasks: the item pairs (0 with PERSIST: not known); a class of few pairs gets
 // only the blocks it needs, which leaves the others to the classes beside it
-template <int G, int R, int MODE, bool PERSIST, bool NN = true>
+template <int G, int R, int MODE, bool PERSIST, bool NN>
 int launch16(const ExtArgs& a, cudaStream_t st, uint64_t tasks) {
   constexpr int kThreads = 128;
   constexpr int groups = (kThreads / 32) * (32 / G);
@@ -764,12 +757,11 @@ int launch16(const ExtArgs& a, cudaStream_t st, uint64_t tasks) {
 }
 
 
-template <int G, int MODE, bool NN>
+template <int MODE, bool NN>
 int launch_all(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStream_t st) {
-  constexpr int kThreads = 128;
-  constexpr int groups = (kThreads / 32) * (32 / G);
+  constexpr int kThreads = 128, groups = kThreads / 32;
   const size_t smem = sizeof(GroupSmem) * groups;
-  auto kern = k_extend_all<G, MODE, NN>;
+  auto kern = k_extend_all<MODE, NN>;
   // per device, so set for each launch
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
     return -1;
@@ -780,11 +772,30 @@ int launch_all(const ExtArgs& a, const uint32_t* upper, uint64_t pairs, cudaStre
   const uint64_t most = static_cast<uint64_t>(nsm) * (per_sm > 0 ? per_sm : 1), need = (pairs + groups - 1) / groups;
   ExtRows rows;
   for (int c = 0; c < kNumBins; ++c) {
-    const uint32_t n = (upper[c] + G - 1) / G, lo = G == 32 ? 4 : 5, hi = 256 / G;
-    rows.r[c] = static_cast<uint8_t>(n < lo ? lo : n > hi ? hi : n);
+    const uint32_t n = (upper[c] + 31) / 32;
+    rows.r[c] = static_cast<uint8_t>(n < 4 ? 4 : n > 8 ? 8 : n);
   }
   kern<<<static_cast<unsigned>(need < most ? need : most), kThreads, smem, st>>>(a, rows);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+}
+
+// the persistent kernel of one shape
+template <int MODE, bool NN>
+int launch_shape(uint32_t lanes, uint32_t rows, const ExtArgs& a, cudaStream_t st, uint64_t tasks) {
+#define SR_CASE(g, r) \
+  if (lanes == g && rows == r) return launch16<g, r, MODE, true, NN>(a, st, tasks);
+  SR_SHAPES(SR_CASE)
+#undef SR_CASE
+  return -1;
+}
+
+template <int MODE, bool NN>
+int touch_shapes() {
+  int n_ = 0;
+#define SR_CASE(g, r) SR_TOUCH((k_extend16<g, r, MODE, true, NN>));
+  SR_SHAPES(SR_CASE)
+#undef SR_CASE
+  return n_;
 }
 
 }  // namespace

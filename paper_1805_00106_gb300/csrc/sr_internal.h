@@ -452,6 +452,9 @@ int extend_shapes(uint32_t* lanes, uint32_t* rows, int cap);
 int preload_mode0();
 int preload_mode1();
 int preload_mode2();
+int preload_neg0();
+int preload_neg1();
+int preload_neg2();
 int preload_extend();
 int preload_kernels();
 int preload_traceback();

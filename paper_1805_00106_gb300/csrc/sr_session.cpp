@@ -217,6 +217,9 @@ static void preload_all(int dev) {
   preload_mode0();
   preload_mode1();
   preload_mode2();
+  preload_neg0();
+  preload_neg1();
+  preload_neg2();
   preload_extend();
   preload_kernels();
   preload_traceback();
