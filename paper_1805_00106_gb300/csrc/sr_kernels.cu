@@ -89,26 +89,85 @@ __global__ void k_pack_reads(const char* bases, const uint64_t* off, uint32_t n_
   if (bad) atomicOr(status, kStBadBase);
 }
 
-// G lanes per read: item -> read map and window validation
-template <int G>
-__global__ void k_items(const uint64_t* cand_off, uint32_t n_reads, const uint8_t* c_ref,
-                        const uint8_t* c_strand, const uint64_t* c_start, const uint32_t* c_len,
-                        DevRefs refs, uint32_t* item_read, uint32_t* status) {
-  const uint64_t r = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) / G;
-  const int lane = threadIdx.x & (G - 1);
-  if (r >= n_reads) return;
-  const uint64_t c0 = cand_off[r], c1 = cand_off[r + 1];
-  bool bad = c1 < c0;
-  for (uint64_t c = c0 + lane; c < c1 && !bad; c += G) {
-    item_read[c] = static_cast<uint32_t>(r);
-    const uint32_t k = c_ref[c];
-    const uint32_t n = c_len[c];
-    bool ok = k < static_cast<uint32_t>(refs.n) && c_strand[c] <= 1u && n >= 1u &&
-              n <= static_cast<uint32_t>(kMaxWinLen);
-    if (ok) ok = c_start[c] + n <= refs.len[k];
-    bad |= !ok;
+// Calls window(c, r, x) once for each window c of the reads r < n, on G lanes per
+// read; read(r, first, c0, cnt, x) gives a read's windows [c0, c0 + cnt) and a word of its
+// own (first: on the first of its lanes, once per read); bad(r) follows where a
+// window of the read was not ok (after a loop without side effects, so that the
+// loads of U rounds are in flight together).  Reads of more windows than
+// 32 rounds of G lanes are walked by their warp and those of more than kBlockWindows
+// by their block once its other reads are done, so that one read of many windows
+// does not hold up a batch of short ones: 300k reads of one window staged in 0.70 ms,
+// with one of 200,000 among them in 1.36 (29 with one lane on it, and 65 instead of 31
+// for the run, where a lane still selects the read's best window).
+constexpr uint32_t kBlockWindows = 4096;
+template <int G, int U, typename Read, typename Window, typename Bad>
+__device__ __forceinline__ void walk_windows(uint32_t n, Read read, Window window, Bad bad) {
+  constexpr uint32_t kMost = 64;  // reads a block keeps for its end; a warp walks those past it
+  __shared__ uint64_t long_c0[kMost];
+  __shared__ uint32_t long_n[kMost], long_r[kMost], long_x[kMost], n_long;
+  if (threadIdx.x == 0) n_long = 0;
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31, g = lane & (G - 1);
+  const uint64_t step = static_cast<uint64_t>(gridDim.x) * blockDim.x / G;
+  auto walk = [&](uint32_t r, uint64_t c0, uint32_t i, uint32_t cnt, uint32_t by, uint32_t x) {
+    bool ok = true;
+#pragma unroll U
+    for (; i < cnt; i += by) ok &= window(c0 + i, r, x);
+    if (!ok) bad(r);
+  };
+  for (uint64_t base = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + (threadIdx.x & ~31u)) / G; base < n; base += step) {
+    const uint64_t r = base + lane / G;
+    uint64_t c0 = 0;
+    uint32_t cnt = 0, x = 0;
+    if (r < n) read(static_cast<uint32_t>(r), g == 0, c0, cnt, x);
+    const bool many = cnt > 32u * G;
+    if (!many) walk(static_cast<uint32_t>(r), c0, g, cnt, G, x);
+    for (uint32_t todo = __ballot_sync(FULL, many && g == 0); todo; todo &= todo - 1) {
+      const int src = __ffs(todo) - 1;
+      const uint32_t wr = static_cast<uint32_t>(base) + src / G, wx = __shfl_sync(FULL, x, src);
+      const uint64_t w0 = __shfl_sync(FULL, c0, src);
+      const uint32_t wn = __shfl_sync(FULL, cnt, src);
+      uint32_t slot = kMost;
+      if (wn > kBlockWindows) {
+        if (lane == 0) slot = atomicAdd(&n_long, 1u);
+        slot = __shfl_sync(FULL, slot, 0);
+      }
+      if (slot >= kMost) {
+        walk(wr, w0, lane, wn, 32, wx);
+      } else if (lane == 0) {
+        long_r[slot] = wr;
+        long_x[slot] = wx;
+        long_c0[slot] = w0;
+        long_n[slot] = wn;
+      }
+    }
   }
-  if (bad) atomicOr(status, kStBadWindow);
+  __syncthreads();
+  for (uint32_t i = 0; i < min(n_long, kMost); ++i)
+    walk(long_r[i], long_c0[i], threadIdx.x, long_n[i], blockDim.x, long_x[i]);
+}
+
+// item -> read map and window validation
+template <int G>
+__global__ void k_items(const uint64_t* __restrict__ cand_off, uint32_t n_reads, const uint8_t* __restrict__ c_ref,
+                        const uint8_t* __restrict__ c_strand, const uint64_t* __restrict__ c_start,
+                        const uint32_t* __restrict__ c_len, DevRefs refs, uint32_t* __restrict__ item_read, uint32_t* status) {
+  walk_windows<G, 1>(
+      n_reads,
+      [&](uint32_t r, bool, uint64_t& c0, uint32_t& cnt, uint32_t&) {
+        c0 = cand_off[r];
+        const uint64_t c1 = cand_off[r + 1];
+        if (c1 < c0) atomicOr(status, kStBadWindow);
+        else cnt = static_cast<uint32_t>(c1 - c0);
+      },
+      [&](uint64_t c, uint32_t r, uint32_t) {
+        const uint32_t k = c_ref[c], s = c_strand[c], n = c_len[c];
+        const uint64_t w0 = c_start[c];
+        item_read[c] = r;
+        return k < static_cast<uint32_t>(refs.n) && s <= 1u && n >= 1u && n <= static_cast<uint32_t>(kMaxWinLen) &&
+               w0 + n <= refs.len[k];
+      },
+      [&](uint32_t) { atomicOr(status, kStBadWindow); });
 }
 
 struct BinArgs {
@@ -449,8 +508,7 @@ int launch_pack_refs(const char* ascii, uint64_t len, uint32_t* words, uint32_t*
 }
 
 // Lanes per read of the kernels that walk a read's windows once: one where reads
-// hold one or two windows on average, eight where they hold more (a read may have
-// hundreds).
+// hold one or two windows on average, eight where they hold more.
 bool few_windows(const BatchDev& b) { return b.n_items <= 2ull * b.n_reads; }
 
 int launch_prepare(const BatchDev& b, const DevRefs& refs, cudaStream_t st) {
@@ -582,16 +640,16 @@ int launch_assemble(const BatchDev& b, int n_refs, bool want_cigar, int32_t item
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-// A batch staged from a read range [r0, r1) of the caller's arrays receives
-// the range's offsets as they are; they are made batch-relative here.
-// ---- checks of a staged batch (few host windows get the same checks on the
-// host): per read, its offsets, length, window
-// count and windows; the first bad read (lowest index) with the reason, and for
-// good batches the DP cells, the longest read and the windows per read length.
+// Checks of a staged batch (few host windows get the same checks on the host): per
+// read, its offsets, length, window count and windows; the first bad read (lowest
+// index) with the reason, and for good batches the DP cells, the longest read and
+// the windows per read length.  The blocks stride over the reads, so that the
+// histogram is cleared and handed on once per block and not once per 256 / G reads.
 template <int G>
-__global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off, uint32_t n, uint64_t nc,
-                              const uint8_t* c_ref, const uint8_t* c_strand, const uint64_t* c_start,
-                              const uint32_t* c_len, DevRefs refs, StageCheck* out) {
+__global__ void __launch_bounds__(256, 6) k_stage_check(const uint64_t* __restrict__ read_off, const uint64_t* __restrict__ cand_off, uint32_t n,
+                              uint64_t nc, const uint8_t* __restrict__ c_ref, const uint8_t* __restrict__ c_strand,
+                              const uint64_t* __restrict__ c_start, const uint32_t* __restrict__ c_len, DevRefs refs,
+                              StageCheck* out) {
   __shared__ uint32_t hist[kMaxReadLen + 1];
   __shared__ unsigned long long cells_sh;
   __shared__ uint32_t longest;
@@ -601,40 +659,36 @@ __global__ void k_stage_check(const uint64_t* read_off, const uint64_t* cand_off
     longest = 0;
   }
   __syncthreads();
-  // G lanes per read; the blocks stride over the reads, so that the histogram is
-  // cleared and handed on once per block and not once per 256 / G reads
-  const uint32_t lane = threadIdx.x & (G - 1);
-  const uint64_t step = static_cast<uint64_t>(gridDim.x) * blockDim.x / G;
   unsigned long long cells = 0;
   uint32_t top = 0;
-  for (uint64_t r = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) / G; r < n; r += step) {
-    uint32_t why = 0;
-    const uint64_t a0 = read_off[r], a1 = read_off[r + 1], c0 = cand_off[r], c1 = cand_off[r + 1];
-    if (a1 < a0 || c1 < c0 || c1 > nc) why = 1;
-    else if (a1 - a0 == 0 || a1 - a0 > static_cast<uint64_t>(kMaxReadLen)) why = 2;
-    else if (c1 - c0 >= (1ull << 19)) why = 3;
-    if (!why) {
-      const uint64_t m = a1 - a0;
-      uint64_t suml = 0;
-      for (uint64_t k = c0 + lane; k < c1; k += G) {
-        const uint32_t ref = c_ref[k], len = c_len[k];
+  auto refuse = [&](uint32_t r, uint32_t why) { atomicMin(&out->bad, (static_cast<unsigned long long>(r) << 3) | why); };
+  walk_windows<G, 4>(
+      n,
+      [&](uint32_t r, bool first, uint64_t& c0, uint32_t& cnt, uint32_t& m) {
+        const uint64_t a0 = read_off[r], a1 = read_off[r + 1], w0 = cand_off[r], w1 = cand_off[r + 1];
+        const uint32_t why = a1 < a0 || w1 < w0 || w1 > nc                                        ? 1
+                             : a1 - a0 == 0 || a1 - a0 > static_cast<uint64_t>(kMaxReadLen) ? 2
+                             : w1 - w0 >= (1ull << 19)                                      ? 3
+                                                                                            : 0;
+        if (why) return refuse(r, why);
+        c0 = w0;
+        cnt = static_cast<uint32_t>(w1 - w0);
+        m = static_cast<uint32_t>(a1 - a0);
+        if (!first) return;
+        if (cnt) atomicAdd(&hist[m], cnt);
+        top = max(top, m);
+      },
+      [&](uint64_t k, uint32_t, uint32_t m) {
+        const uint32_t ref = c_ref[k], strand = c_strand[k], len = c_len[k];
         const uint64_t w0 = c_start[k];
-        const bool ok = ref < static_cast<uint32_t>(refs.n) && c_strand[k] <= 1 && len >= 1 &&
-                        len <= static_cast<uint32_t>(kMaxWinLen) && w0 <= refs.len[ref] && w0 + len <= refs.len[ref];
-        if (!ok) why = 4;
-        suml += len;
-      }
-      cells += m * suml;
-      if (lane == 0) {
-        if (c1 > c0) atomicAdd(&hist[m], static_cast<uint32_t>(c1 - c0));
-        top = max(top, static_cast<uint32_t>(m));
-      }
-    }
-    if (why) atomicMin(&out->bad, (static_cast<unsigned long long>(r) << 3) | why);
-  }
-  top = __reduce_max_sync(0xffffffffu, top);
+        cells += static_cast<uint64_t>(m) * len;
+        return ref < static_cast<uint32_t>(refs.n) && strand <= 1 && len >= 1 && len <= static_cast<uint32_t>(kMaxWinLen) &&
+               w0 <= refs.len[ref] && w0 + len <= refs.len[ref];
+      },
+      [&](uint32_t r) { refuse(r, 4); });
+  top = __reduce_max_sync(FULL, top);
   if ((threadIdx.x & 31) == 0 && top) atomicMax(&longest, top);
-  for (int o = 16; o; o >>= 1) cells += __shfl_xor_sync(0xffffffffu, cells, o);
+  for (int o = 16; o; o >>= 1) cells += __shfl_xor_sync(FULL, cells, o);
   if ((threadIdx.x & 31) == 0 && cells) atomicAdd(&cells_sh, cells);
   __syncthreads();
   for (int k = threadIdx.x; k <= kMaxReadLen; k += blockDim.x)
