@@ -174,7 +174,8 @@ struct sr_session {
   void* cal_buf[kCalBufs] = {};
   uint64_t cal_bytes[kCalBufs] = {};
   void* cal_back = nullptr;  // pinned: what comes back of a call's plan
-  // blocks of freed device lists (guarded by pool_mu, not counted in hbm_used)
+  // blocks of freed device lists (guarded by pool_mu, not counted in hbm_used, given
+  // back where an allocation of the session fails)
   std::vector<std::pair<void*, uint64_t>> list_pool;
 };
 
@@ -512,6 +513,34 @@ uint64_t batch_bytes_estimate(uint32_t n_reads, uint64_t n_items, uint64_t n_bas
 }  // namespace sr
 
 namespace {
+// Gives back the device memory that the session keeps but nothing uses (arenas of
+// freed batches, blocks of freed device lists); false when there is none.
+bool free_idle(sr_session* s) {
+  std::vector<std::pair<void*, uint64_t>> arenas, lists;
+  {
+    std::lock_guard<std::mutex> lk(s->spare_mu);
+    arenas.swap(s->spares);
+  }
+  {
+    std::lock_guard<std::mutex> lk(s->pool_mu);
+    lists.swap(s->list_pool);
+  }
+  for (auto& a : arenas) cudaFree(a.first);
+  for (auto& l : lists) cudaFree(l.first);
+  return !arenas.empty() || !lists.empty();
+}
+
+// cudaMalloc for the session; where memory has run out, again without its idle memory
+cudaError_t dev_malloc(sr_session* s, void** p, uint64_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    if (free_idle(s)) e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+  }
+  return e;
+}
+
 // A batch of n reads, nb bases and nc windows on `stream`, its arena taken from
 // the session's kept arenas or allocated, and its events and side streams from
 // the session's pool.  Counts its bytes in the session's hbm_used.
@@ -548,27 +577,13 @@ sr_status batch_alloc(sr_session* s, uint32_t n, uint64_t nb, uint64_t nc, cudaS
     if (e != cudaSuccess) {
       cudaGetLastError();
       want = b->bytes;
-      e = cudaMalloc(&b->arena, want);
+      e = dev_malloc(s, &b->arena, want);
     }
     if (e != cudaSuccess) {
-      // the kept arenas may be what is in the way
-      cudaGetLastError();
-      std::vector<std::pair<void*, uint64_t>> sp;
-      {
-        std::lock_guard<std::mutex> lk(s->spare_mu);
-        sp.swap(s->spares);
-      }
-      if (!sp.empty()) {
-        for (auto& a : sp) cudaFree(a.first);
-        e = cudaMalloc(&b->arena, want);
-      }
-      if (e != cudaSuccess) {
-        b->arena = nullptr;
-        sr_batch_free(b);
-        cudaGetLastError();
-        return set_error(SR_ENOMEM, "sr_batch_stage: device allocation of %llu bytes failed",
-                         static_cast<unsigned long long>(bytes));
-      }
+      b->arena = nullptr;
+      sr_batch_free(b);
+      return set_error(SR_ENOMEM, "sr_batch_stage: device allocation of %llu bytes failed",
+                       static_cast<unsigned long long>(bytes));
     }
     b->arena_bytes = want;
   }
@@ -1433,7 +1448,7 @@ extern "C" sr_status sr_session_attach_index(sr_session* s, const sr_index* cons
   s->didx = DevIndex{};
   auto up = [&](const void* src, uint64_t bytes, void** dst) -> bool {
     void* d = nullptr;
-    if (cudaMalloc(&d, bytes ? bytes : 1) != cudaSuccess) return false;
+    if (dev_malloc(s, &d, bytes ? bytes : 1) != cudaSuccess) return false;
     s->idx_bufs.push_back(d);
     if (bytes && cudaMemcpy(d, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return false;
     *dst = d;
@@ -1510,15 +1525,13 @@ extern "C" sr_status sr_session_attach_index(sr_session* s, const sr_index* cons
       env_u64("SR_CAL_HEADS", 1, true) != 0) {
     void* ph = nullptr;
     s->didx.head_words = entries <= nbk * per_near ? 8 : 16;
-    if (cudaMalloc(&ph, nbk * s->didx.head_words * 4) == cudaSuccess) {
+    if (dev_malloc(s, &ph, nbk * s->didx.head_words * 4) == cudaSuccess) {
       s->idx_bufs.push_back(ph);
       if (launch_cal_heads(s->didx, nbk, static_cast<uint32_t*>(ph), s->stream) < 0 ||
           cudaStreamSynchronize(s->stream) != cudaSuccess)
         return fail();
       s->didx.heads = static_cast<const uint32_t*>(ph);
-    } else {
-      cudaGetLastError();  // the heads are optional: without them the lookups read jptr / key16
-    }
+    }  // the heads are optional: without them the lookups read jptr / key16
   }
   return SR_OK;
 }
@@ -1549,8 +1562,13 @@ struct CalCall {
       if (e != cudaSuccess) return nullptr;
     }
     void* p = nullptr;
-    const uint64_t want = bytes + bytes / 4;
+    uint64_t want = bytes + bytes / 4;
     e = cudaMalloc(&p, want);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      want = bytes;
+      e = dev_malloc(s, &p, want);
+    }
     if (e == cudaSuccess && was) {
       e = cudaMemcpyAsync(p, was, keep, cudaMemcpyDeviceToDevice, st);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1570,9 +1588,11 @@ struct CalCall {
 };
 
 // ---- device lists.  A list's arrays share one block; the session keeps up to
-// kKeptLists blocks of freed lists for the next ones.  A freed list waits for the
+// kKeptLists blocks of freed lists, of at most kKeptListBytes each, for the next
+// ones, until it needs the memory otherwise (free_idle).  A freed list waits for the
 // device first, as cudaFree did: work on other streams may still read it.
 constexpr size_t kKeptLists = 2;
+constexpr uint64_t kKeptListBytes = 256ull << 20;
 struct DevListBox {
   sr_cand_list pub;  // first: what the caller holds
   sr_session* s;
@@ -1616,15 +1636,7 @@ void* list_block_take(sr_session* s, uint64_t bytes, uint64_t* got) {
   if (cudaMalloc(&p, *got) == cudaSuccess) return p;
   cudaGetLastError();
   *got = bytes;
-  std::vector<std::pair<void*, uint64_t>> kept;  // they may be what is in the way
-  {
-    std::lock_guard<std::mutex> lk(s->pool_mu);
-    kept.swap(s->list_pool);
-  }
-  for (auto& b : kept) cudaFree(b.first);
-  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-  cudaGetLastError();
-  return nullptr;
+  return dev_malloc(s, &p, bytes) == cudaSuccess ? p : nullptr;
 }
 
 void list_block_give(sr_session* s, void* p, uint64_t bytes) {
@@ -1632,8 +1644,9 @@ void list_block_give(sr_session* s, void* p, uint64_t bytes) {
   cudaGetDevice(&dev);
   if (dev != s->device) cudaSetDevice(s->device);
   const bool idle = cudaDeviceSynchronize() == cudaSuccess;
-  void* drop = idle ? nullptr : p;
-  if (idle) {
+  const bool keep = idle && bytes <= kKeptListBytes;
+  void* drop = keep ? nullptr : p;
+  if (keep) {
     std::lock_guard<std::mutex> lk(s->pool_mu);
     s->list_pool.emplace_back(p, bytes);
     if (s->list_pool.size() > kKeptLists) {
@@ -2186,7 +2199,7 @@ extern "C" sr_status sr_batch_report(sr_session* s, sr_batch* b, uint32_t kind, 
   uint32_t* scratch = nullptr;
   sr_report_hit* d_hits = nullptr;
   const uint64_t sw = report_scratch_words(n);
-  cudaError_t e = cudaMalloc(&scratch, sw * 4);
+  cudaError_t e = dev_malloc(s, reinterpret_cast<void**>(&scratch), sw * 4);
   auto fail = [&](const char* where) {
     cudaGetLastError();
     if (scratch) cudaFree(scratch);
@@ -2217,7 +2230,7 @@ extern "C" sr_status sr_batch_report(sr_session* s, sr_batch* b, uint32_t kind, 
     return fail("sr_batch_report host alloc");
   }
   if (total) {
-    e = cudaMalloc(&d_hits, total * sizeof(sr_report_hit));
+    e = dev_malloc(s, reinterpret_cast<void**>(&d_hits), total * sizeof(sr_report_hit));
     if (e != cudaSuccess) return fail("sr_batch_report alloc");
     if (launch_report_write(b->d, nr, kd, n_best, scratch, d_hits, stream) < 0) {
       e = cudaGetLastError();
