@@ -251,7 +251,8 @@ void sr_session_close(sr_session* s);
  * SR_FLAG_DEVICE), so that reads, windows and the alignment stay on the device
  * (sr_align_batch takes such a list as it is; the session keeps up to
  * two freed lists' blocks, of at most 256 MB each, for its next ones, until one of
- * its allocations needs the memory).  The call's scratch (staged windows, 16 bytes each, and a
+ * its allocations needs the memory; a held list outlives the session and keeps
+ * nothing of it but its own arrays).  The call's scratch (staged windows, 16 bytes each, and a
  * few words per read; for reads of the many-block path kept seed lookups, 8 bytes
  * per seed and reference, up to 1 GiB, and CAL keys and window arrays, 24 bytes
  * per CAL bound, up to 64M bounds; for a host list, the list itself, 8 bytes per read and 18 per window, built on the

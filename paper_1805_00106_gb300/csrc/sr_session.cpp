@@ -13,7 +13,6 @@
 #include <mutex>
 #include <string>
 #include <thread>
-#include <unordered_set>
 #include <vector>
 
 #include "sr_host.h"
@@ -345,6 +344,8 @@ extern "C" sr_status sr_session_open_seqs(const char* const* seqs, const uint64_
   return open_common(nullptr, seqs, lens, n_refs, hbm_budget, out);
 }
 
+static void lists_detach(sr_session* s);
+
 static void session_release(sr_session* s) {
   if (s->live.fetch_sub(1) != 1) return;
   for (auto* w : s->d_words) cudaFree(w);
@@ -368,6 +369,7 @@ extern "C" void sr_session_close(sr_session* s) {
     serve_destroy(s->server);
     s->server = nullptr;
   }
+  lists_detach(s);
   session_release(s);
 }
 
@@ -1595,12 +1597,14 @@ constexpr size_t kKeptLists = 2;
 constexpr uint64_t kKeptListBytes = 256ull << 20;
 struct DevListBox {
   sr_cand_list pub;  // first: what the caller holds
-  sr_session* s;
+  sr_session* s;     // nullptr once it has closed: a list keeps its block, not the session
+  int device;
   void* block;
   uint64_t bytes;
+  DevListBox* next;
 };
 std::mutex g_lists_mu;
-std::unordered_set<const void*> g_lists;  // the boxes alive
+DevListBox* g_lists = nullptr;  // the boxes alive
 
 uint64_t list_layout(uint64_t n, uint64_t cap, uint64_t at[7]) {
   const uint64_t bytes[6] = {(n + 1) * 8, cap, cap, cap * 8, cap * 4, cap * 4};
@@ -1876,16 +1880,37 @@ struct FindBufs {
 }  // namespace
 
 bool sr::device_list_free(sr_cand_list* l) {
+  DevListBox* box = nullptr;
   {
     std::lock_guard<std::mutex> lk(g_lists_mu);
-    if (!g_lists.erase(l)) return false;
+    DevListBox** at = &g_lists;
+    while (*at && &(*at)->pub != l) at = &(*at)->next;
+    if (!*at) return false;
+    box = *at;
+    *at = box->next;
   }
-  auto* box = reinterpret_cast<DevListBox*>(l);
-  sr_session* s = box->s;
-  list_block_give(s, box->block, box->bytes);
+  if (box->s) {
+    list_block_give(box->s, box->block, box->bytes);
+    session_release(box->s);
+  } else {
+    int dev = -1;
+    cudaGetDevice(&dev);
+    if (dev != box->device) cudaSetDevice(box->device);
+    cudaFree(box->block);  // waits for the device
+    if (dev >= 0 && dev != box->device) cudaSetDevice(dev);
+  }
   free(box);
-  session_release(s);
   return true;
+}
+
+// the session closes: its lists that are still held no longer refer to it
+static void lists_detach(sr_session* s) {
+  std::lock_guard<std::mutex> lk(g_lists_mu);
+  for (DevListBox* b = g_lists; b; b = b->next)
+    if (b->s == s) {
+      b->s = nullptr;
+      s->live.fetch_sub(1);  // not the last: the closing call holds one
+    }
 }
 
 extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, const sr_cand_params* params,
@@ -2091,6 +2116,7 @@ extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, 
     auto* box = static_cast<DevListBox*>(calloc(1, sizeof(DevListBox)));
     if (!box) return done(set_error(SR_ENOMEM, "sr_candidates_device: out of memory"));
     box->s = s;
+    box->device = s->device;
     box->block = block;
     box->bytes = block_bytes;
     sr_cand_list& l = box->pub;
@@ -2103,10 +2129,11 @@ extern "C" sr_status sr_candidates_device(sr_session* s, const sr_reads* reads, 
     l.win_start = L.start;
     l.win_len = L.len;
     l.hits = L.hits;
-    s->live.fetch_add(1);  // a list keeps its session alive
+    s->live.fetch_add(1);  // until the list is freed or the session closes
     {
       std::lock_guard<std::mutex> lk(g_lists_mu);
-      g_lists.insert(box);
+      box->next = g_lists;
+      g_lists = box;
     }
     *out = &box->pub;
     return SR_OK;

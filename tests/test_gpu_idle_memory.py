@@ -1,6 +1,8 @@
 """Device memory that a session keeps for later calls (blocks of freed device lists,
 arenas of freed batches) does not stand in the way of its own allocations, is bounded,
 and a list that is still held keeps no more than its own arrays."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -15,6 +17,7 @@ MB = 1 << 20
 
 def _free():
     import torch
+    gc.collect()  # sessions of other tests go now or not at all
     torch.cuda.synchronize()
     return torch.cuda.mem_get_info()[0]
 
