@@ -352,10 +352,15 @@ __global__ void __launch_bounds__(32 * kFindWarps, 10) k_find_warp(FindArgs a) {
 // 16384 instead of 8192 slots in the large table, which keeps reads like the one
 // here of 8721 distinct CALs off the large-read path.  The small table leaves room
 // for 10 blocks per SM.
+// Reads of more distinct CALs than the large table takes cost about 0.5 ms each (the
+// many-block path) where the table's cost 0.012 spread over the SMs (2000 reads in a
+// repeat of 12,000 / 12,600 copies 23.0 / 1023 ms, 1035 / 1034 before the tables; one
+// read 1.78 / 1.13 ms).  Cutting to max_cands takes each window's rank here, whatever
+// their number: 2000 reads of 12,000 windows cut to 64 29.9 ms (1068 when more than
+// 4096 windows went to the many-block path).
 constexpr int kElBits = 14;  // bits of an element's number beside its count (at most one per seed)
 constexpr uint32_t kElMask = (1u << kElBits) - 1u;
 static_assert(2 * kMaxReadLen < (1 << (32 - kElBits)), "a CAL's count and an element number in 32 bits");
-constexpr uint32_t kCutWindows = 4096;  // more windows are cut to max_cands by the large-read path
 
 template <int S, int T, uint32_t ENTRIES>
 struct BlockSpace {
@@ -546,14 +551,6 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
     }
     __syncthreads();
     const bool cut = a.max_cands && nwin > a.max_cands;
-    if (cut && nwin > kCutWindows) {
-      if (tid == 0) {
-        a.list_rest[atomicAdd(&a.plan->n_rest, 1u)] = rr;
-        a.nwin[rr] = 0;
-      }
-      __syncthreads();
-      continue;
-    }
     const uint32_t kept = cut ? a.max_cands : nwin;
     if (tid == 0) {
       s_slot = atomicAdd(&a.plan->cursor, static_cast<unsigned long long>(kept));
@@ -572,7 +569,7 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
         if (keep) {
           uint32_t rank = 0;
           const uint32_t h = hits[j];
-          for (uint32_t q2 = 0; q2 < nwin; ++q2) rank += (hits[q2] > h || (hits[q2] == h && q2 < j)) ? 1u : 0u;
+          for (uint32_t q2 = 0; q2 < nwin && rank < a.max_cands; ++q2) rank += (hits[q2] > h || (hits[q2] == h && q2 < j)) ? 1u : 0u;
           keep = rank < a.max_cands;
         }
         at = before + static_cast<uint32_t>(block_exscan(keep ? 1u : 0u, &tot));
