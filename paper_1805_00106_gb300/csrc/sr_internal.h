@@ -255,7 +255,8 @@ struct StageCheck {
   uint32_t pad;
   unsigned long long by_len[kMaxReadLen + 1];  // windows per read length
 };
-int launch_stage_check(const BatchDev& b, const DevRefs& refs, StageCheck* out, cudaStream_t st);
+// rb, cb: what was taken off the caller's offsets (launch_rebase_offsets)
+int launch_stage_check(const BatchDev& b, const DevRefs& refs, uint64_t rb, uint64_t cb, StageCheck* out, cudaStream_t st);
 int launch_first_bad_window(const BatchDev& b, const DevRefs& refs, uint32_t read, StageCheck* out,
                             cudaStream_t st);
 // off[0..n) -= base

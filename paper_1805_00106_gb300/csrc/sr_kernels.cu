@@ -643,13 +643,14 @@ int launch_assemble(const BatchDev& b, int n_refs, bool want_cigar, int32_t item
 // Checks of a staged batch (few host windows get the same checks on the host): per
 // read, its offsets, length, window count and windows; the first bad read (lowest
 // index) with the reason, and for good batches the DP cells, the longest read and
-// the windows per read length.  The blocks stride over the reads, so that the
+// the windows per read length.  The offsets were made batch-relative by taking off rb
+// and cb; they are compared as the caller gave them.  The blocks stride over the reads, so that the
 // histogram is cleared and handed on once per block and not once per 256 / G reads.
 template <int G>
 __global__ void __launch_bounds__(256, 6) k_stage_check(const uint64_t* __restrict__ read_off, const uint64_t* __restrict__ cand_off, uint32_t n,
                               uint64_t nc, const uint8_t* __restrict__ c_ref, const uint8_t* __restrict__ c_strand,
                               const uint64_t* __restrict__ c_start, const uint32_t* __restrict__ c_len, DevRefs refs,
-                              StageCheck* out) {
+                              uint64_t rb, uint64_t cb, StageCheck* out) {
   __shared__ uint32_t hist[kMaxReadLen + 1];
   __shared__ unsigned long long cells_sh;
   __shared__ uint32_t longest;
@@ -666,7 +667,7 @@ __global__ void __launch_bounds__(256, 6) k_stage_check(const uint64_t* __restri
       n,
       [&](uint32_t r, bool first, uint64_t& c0, uint32_t& cnt, uint32_t& m) {
         const uint64_t a0 = read_off[r], a1 = read_off[r + 1], w0 = cand_off[r], w1 = cand_off[r + 1];
-        const uint32_t why = a1 < a0 || w1 < w0 || w1 > nc                                        ? 1
+        const uint32_t why = a1 + rb < a0 + rb || w1 + cb < w0 + cb || w1 + cb > nc + cb ? 1
                              : a1 - a0 == 0 || a1 - a0 > static_cast<uint64_t>(kMaxReadLen) ? 2
                              : w1 - w0 >= (1ull << 19)                                      ? 3
                                                                                             : 0;
@@ -710,7 +711,7 @@ __global__ void k_first_bad_window(uint32_t r, const uint64_t* cand_off, const u
   }
 }
 
-int launch_stage_check(const BatchDev& b, const DevRefs& refs, StageCheck* out, cudaStream_t st) {
+int launch_stage_check(const BatchDev& b, const DevRefs& refs, uint64_t rb, uint64_t cb, StageCheck* out, cudaStream_t st) {
   if (cudaMemsetAsync(out, 0, sizeof(StageCheck), st) != cudaSuccess) return -1;
   if (cudaMemsetAsync(&out->bad, 0xff, 2 * sizeof(unsigned long long), st) != cudaSuccess) return -1;
   if (b.n_reads == 0) return 0;
@@ -719,7 +720,7 @@ int launch_stage_check(const BatchDev& b, const DevRefs& refs, StageCheck* out, 
   const uint64_t blocks = std::min<uint64_t>((b.n_reads * (few ? 1ull : 8ull) + 255) / 256, 152ull * 8);
   auto* kern = few ? k_stage_check<1> : k_stage_check<8>;
   kern<<<static_cast<unsigned>(blocks), 256, 0, st>>>(b.read_off, b.cand_off, b.n_reads, b.n_items, b.c_ref, b.c_strand,
-                                                      b.c_start, b.c_len, refs, out);
+                                                      b.c_start, b.c_len, refs, rb, cb, out);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 

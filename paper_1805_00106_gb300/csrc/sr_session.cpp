@@ -615,10 +615,11 @@ sr_status batch_alloc(sr_session* s, uint32_t n, uint64_t nb, uint64_t nc, cudaS
 
 // Checks a batch's staged arrays by a kernel on their stream and waits for it:
 // what is wrong with the first bad read in hc (its first bad window too), or the
-// batch's cells, longest read and windows per read length
-cudaError_t device_check(sr_batch* b, const DevRefs& refs, cudaStream_t st, StageCheck& hc) {
+// batch's cells, longest read and windows per read length; rb and cb: the batch's
+// first base and window in the caller's arrays
+cudaError_t device_check(sr_batch* b, const DevRefs& refs, uint64_t rb, uint64_t cb, cudaStream_t st, StageCheck& hc) {
   StageCheck* dc = static_cast<StageCheck*>(b->d.check);
-  cudaError_t e = launch_stage_check(b->d, refs, dc, st) < 0 ? cudaGetLastError() : cudaSuccess;
+  cudaError_t e = launch_stage_check(b->d, refs, rb, cb, dc, st) < 0 ? cudaGetLastError() : cudaSuccess;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, dc, sizeof(hc), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e == cudaSuccess && hc.bad != ~0ull && (hc.bad & 7) == 4) {
@@ -682,7 +683,7 @@ sr_status stage_device(sr_session* s, const sr_reads* reads, const sr_cand_list*
   copy(d.c_start, cands->win_start, nc * 8);
   copy(d.c_len, cands->win_len, nc * 4);
   StageCheck hc{};
-  if (e == cudaSuccess) e = device_check(b, s->refs, st, hc);
+  if (e == cudaSuccess) e = device_check(b, s->refs, 0, 0, st, hc);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(st);
     sr_batch_free(b);
@@ -827,7 +828,7 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
   constexpr uint64_t kHostWindows = 4096;
   if (nc > kHostWindows) {
     StageCheck hc{};
-    e = device_check(b, s->refs, st, hc);
+    e = device_check(b, s->refs, rb, cb, st, hc);
     if (e != cudaSuccess) {
       cudaStreamSynchronize(st);
       sr_batch_free(b);
