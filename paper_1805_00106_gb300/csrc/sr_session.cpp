@@ -10,7 +10,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <thread>
 #include <vector>
@@ -198,7 +200,7 @@ struct sr_batch {
   uint64_t i32_items = 0;
   bool ran = false;
   bool assembled = false;  // the last run also assembled the result records (serving rounds)
-  std::vector<char> inputs;  // few input bytes, gathered for one copy
+  std::unique_ptr<char[]> inputs;  // few input bytes, gathered for one copy
   sr_align_opts last_opts{};
   BatchRes res{};  // events, side streams (from the session's pool)
   bool res_ok = false;
@@ -783,12 +785,12 @@ sr_status sr::batch_stage_range(sr_session* s, const sr_reads* reads, const sr_c
              {d.c_len, cands->win_len + cb, nc * 4}};
   const char* in0 = d.bases;
   const uint64_t in_bytes = static_cast<uint64_t>(reinterpret_cast<const char*>(d.c_len) - in0) + nc * 4;
-  const bool gathered = in_bytes <= (48u << 10);
+  if (in_bytes <= (48u << 10)) b->inputs.reset(new (std::nothrow) char[in_bytes]());
+  const bool gathered = b->inputs != nullptr;
   if (gathered) {
-    b->inputs.resize(in_bytes);
     for (const auto& x : in)
-      if (x.bytes) memcpy(b->inputs.data() + (static_cast<const char*>(x.dst) - in0), x.src, x.bytes);
-    if (in_bytes) e = cudaMemcpyAsync(const_cast<char*>(in0), b->inputs.data(), in_bytes, cudaMemcpyHostToDevice, st);
+      if (x.bytes) memcpy(b->inputs.get() + (static_cast<const char*>(x.dst) - in0), x.src, x.bytes);
+    e = cudaMemcpyAsync(const_cast<char*>(in0), b->inputs.get(), in_bytes, cudaMemcpyHostToDevice, st);
   } else {
     for (const auto& x : in)
       if (e == cudaSuccess && x.bytes)
