@@ -2502,7 +2502,7 @@ extern "C" sr_status sr_batch_classify(sr_session* s, sr_batch* b, const sr_clas
   if (!b->ran) return set_error(SR_EINVAL, "sr_batch_classify: batch has not run");
   if (s->n_refs < 2) return set_error(SR_EINVAL, "sr_batch_classify: needs 2 references");
   const int32_t ms = params ? params->min_score : 40, mg = params ? params->margin : 5;
-  cudaStream_t stream = b->stream;
+  cudaStream_t stream = b->last_opts.cuda_stream ? static_cast<cudaStream_t>(b->last_opts.cuda_stream) : b->stream;
   if (launch_classify(b->d, static_cast<int>(s->n_refs), ms, mg, stream) < 0)
     return cuda_error("sr_batch_classify launch", cudaGetLastError());
   cudaError_t e = cudaMemcpyAsync(class_out, b->d.read_class, b->n_reads, cudaMemcpyDeviceToHost, stream);
