@@ -356,7 +356,8 @@ __global__ void __launch_bounds__(32 * kFindWarps, 10) k_find_warp(FindArgs a) {
 // many-block path) where the table's cost 0.012 spread over the SMs (2000 reads in a
 // repeat of 12,000 / 12,600 copies 23.0 / 1023 ms, 1035 / 1034 before the tables; one
 // read 1.78 / 1.13 ms).  Cutting to max_cands takes each window's rank here, whatever
-// their number: 2000 reads of 12,000 windows cut to 64 29.9 ms (1068 when more than
+// their number (a look at max_cands every 256 windows; at each one, 20k reads cut to 64
+// windows took 1302 us, 1289 so): 2000 reads of 12,000 windows 25.5 ms (1068 when more than
 // 4096 windows went to the many-block path).
 constexpr int kElBits = 14;  // bits of an element's number beside its count (at most one per seed)
 constexpr uint32_t kElMask = (1u << kElBits) - 1u;
@@ -569,7 +570,10 @@ __global__ void __launch_bounds__(T) k_find_block(FindArgs a, const uint32_t* li
         if (keep) {
           uint32_t rank = 0;
           const uint32_t h = hits[j];
-          for (uint32_t q2 = 0; q2 < nwin && rank < a.max_cands; ++q2) rank += (hits[q2] > h || (hits[q2] == h && q2 < j)) ? 1u : 0u;
+          for (uint32_t q1 = 0; q1 < nwin && rank < a.max_cands; q1 += 256) {
+            const uint32_t end = min(nwin, q1 + 256);
+            for (uint32_t q2 = q1; q2 < end; ++q2) rank += (hits[q2] > h || (hits[q2] == h && q2 < j)) ? 1u : 0u;
+          }
           keep = rank < a.max_cands;
         }
         at = before + static_cast<uint32_t>(block_exscan(keep ? 1u : 0u, &tot));
