@@ -34,10 +34,12 @@ RC_FRAC = 0.5  # reads drawn from the reverse strand (aligned through their '-' 
 ENGINE = "batched (length bins, LPT persistent kernels, one CUDA graph)"
 SP = (2, 3, 5, 2)
 METRIC = "SW GCUPS (whole path: pack, bins, extension, select, traceback)"
-# packed 16-bit ops per cell of the textbook score-only recurrence (6 per s16x2 pair:
-# a score pick, four DPX, half of two maxima): a fixed yardstick, so that figures
-# compare across builds.  k_extend16 takes 4.5 of the ALU pipe's slots per pair.
-OPS_PER_CELL = 3
+# instructions of k_extend16's recurrence on the ALU pipe per s16x2 cell pair: a
+# score pick, three DPX, half of a column maximum (its adds are on the FMA pipe)
+ALU_SLOTS = 4.5
+# packed 16-bit ops per pair of the textbook score-only recurrence (a score pick,
+# four DPX, half of two maxima): a yardstick that compares across builds
+YARDSTICK_OPS = 6
 
 
 def parse():
@@ -700,7 +702,7 @@ def main():
     dpx_rate, probe_mhz = sr.probe_dpx()
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
     f_mhz = clk["sm_mhz"] if clk else probe_mhz
-    peak_gcups = n_sm * f_mhz * 1e6 * dpx_rate * 2 / (2 * OPS_PER_CELL) / 1e9
+    peak_gcups = n_sm * f_mhz * 1e6 * dpx_rate * 2 / ALU_SLOTS / 1e9
     achieved = cells / ext / 1e9
     traffic = traffic_per_launch(cells)
     roofline = {"bound": "alu", "achieved": round(achieved, 2), "peak": round(peak_gcups, 2),
@@ -708,7 +710,8 @@ def main():
                 "kernel": "k_extend16 (all length bins) + k_extend32",
                 "peak_basis": f"{n_sm} SMs x {f_mhz:.0f} MHz (median under load) x "
                               f"{dpx_rate:.1f} packed-16-bit DPX lane-ops/clk/SM (measured) x 2 cells / "
-                              f"{2 * OPS_PER_CELL} ops (a yardstick; the kernel takes 4.5 ALU-pipe slots)",
+                              f"{ALU_SLOTS} ALU-pipe slots per cell pair (score pick, three DPX, half a column maximum)",
+                "six_op_yardstick": round(peak_gcups * ALU_SLOTS / YARDSTICK_OPS, 2),
                 "traceback_ms": round(statistics.mean(tb_ms), 3),
                 "extension_ms": round(1e3 * ext, 3)}
 

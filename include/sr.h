@@ -258,7 +258,10 @@ void sr_session_close(sr_session* s);
  * per CAL bound, up to 64M bounds; for a host list, the list itself, 8 bytes per read and 18 per window, built on the
  * device and copied out once through a pinned block of the session's pool)
  * stays allocated in the session for the next call and is released by
- * sr_session_close; calls on one session run one at a time.  Reads
+ * sr_session_close; calls on one session run one at a time.  The staging holds two
+ * windows per read to begin with: the first call of a session on reads with more is
+ * searched a second time with the room it turned out to need (10k reads of 29
+ * windows: 2.6 ms, then 1.1).  Reads
  * longer than SR_MAX_READ_LEN or with decreasing offsets are SR_EINVAL,
  * non-ACGT bases SR_EBADBASE, no attached index SR_EINVAL.  params->n_threads
  * is unused. */

@@ -197,8 +197,8 @@ __device__ __forceinline__ uint32_t warp_merge(WarpSpace& w, uint32_t nh, uint64
 }
 
 // What bounds it: random requests to the index, a seed's bucket head and its
-// entry's position (300k reads of 100 bases against 2 x 16 Mbp: 45M of them in 0.77
-// ms, 58 G/s, DRAM 75% busy; the issue slots are 62% busy).  So nothing but the
+// entry's position (300k reads of 100 bases against 2 x 16 Mbp: 45M of them in 0.81
+// ms, 56 G/s, DRAM 72% busy; 2.36 warp instructions per cycle and SM).  So nothing but the
 // lookups touches device memory, and the registers are held to 40 warps per SM to
 // hide their latency.  1M such reads: 2.6 ms, where the count, emit, filter and
 // compaction passes over kept lookups and CALs took 7.2 ms.  128 runs and 64

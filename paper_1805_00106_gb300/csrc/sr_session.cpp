@@ -2287,9 +2287,9 @@ constexpr int kParts = 3;
 constexpr uint64_t kPartEnd[kParts] = {1, 9, 10};
 
 // One large sr_align_batch call as kParts batches of consecutive reads, each on
-// a stream of its own.  A part's copies and host checks run while the parts
-// before it compute, and its results come back while the parts after it
-// compute.  A read's windows all stay in its part, so every result is the one a
+// a stream of its own.  A part's copies run while the parts before it compute (its
+// check, a kernel, waits for room beside theirs), and its results come back while
+// the parts after it compute.  A read's windows all stay in its part, so every result is the one a
 // single batch gives; a later part's window indexes and CIGAR offsets are
 // shifted on the device as its records are assembled.  An input error or a
 // device error (bad base, window, timeout) is returned as it stands: staging
